@@ -100,7 +100,8 @@ typedef struct bldtt_stats {
                                            in its default layout: every 32-target row group
                                            holding a real target meets every real source
                                            (the idle rows of such a group included) */
-    int64_t work_items;                 /* target tiles drained by the interaction kernel */
+    int64_t work_items;                 /* tasks drained by the interaction kernel: target
+                                           tiles, long ones split over their sources */
     int32_t interact_grid;              /* CTAs of the persistent interaction kernel */
     int32_t interact_threads;           /* threads per CTA of that kernel */
     float ms_tree, ms_lists;            /* last bldtt_setup: trees; traversal + work lists */
@@ -142,7 +143,9 @@ typedef struct bldtt_stats {
  * host instead, with identical results.  BLDTT_TREE_CAPACITY and
  * BLDTT_TRAVERSAL_CAPACITY override the initial cluster and traversal buffer
  * capacities (testing: a small start makes the launches regrow and resume;
- * the results do not change).
+ * the results do not change); BLDTT_TASK_CHUNKS overrides the number of
+ * 256-source chunks at which a target tile's work is split into tasks (testing:
+ * the results do not depend on the split, bit for bit).
  * Errors: EINVAL for out-of-range sizes or parameters, a non-finite
  * coordinate or charge, an unknown kernel or precision; ENOMEM; ECUDA;
  * ETIMEOUT if a grid barrier of a cooperative launch waited 5 s in vain.

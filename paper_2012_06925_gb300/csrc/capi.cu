@@ -104,6 +104,8 @@ void release(bldtt_plan* p) {
   dfree(p->pool, s);
   p->pool = nullptr;
   dfree_ptr(p->items, s);
+  dfree_ptr(p->parts, s);
+  dfree_ptr(p->seg_sums, s);
   dfree_ptr(p->item_counter, s);
   dfree_ptr(p->chunk_frame, s);
   dfree_ptr(p->pool_res, s);
@@ -111,6 +113,7 @@ void release(bldtt_plan* p) {
   dfree_ptr(p->eval_part, s);
   dfree_ptr(p->eval_prox, s);
   dfree_ptr(p->sh_items, s);
+  dfree_ptr(p->sh_parts, s);
   dfree_ptr(p->sh_item_box, s);
   dfree_ptr(p->qhat, s);
   dfree_ptr(p->phit, s);
@@ -259,7 +262,11 @@ int setup_impl(bldtt_plan* p, const double* targets, const double* sources, cons
   p->qhat_d[p->deg.n - 1] = p->qhat;
   p->phit_d[p->deg.n - 1] = p->phit;
   BL_TRY(dalloc_n(&p->phi_near, (size_t)p->M, s));
-  BL_TRY(dalloc_n(&p->item_counter, p->segments.size() > 0 ? p->segments.size() : 1, s));
+  p->counter_words = kMaxSegmentsLaunch + (size_t)p->nsplit * kItemGroups;
+  BL_TRY(dalloc_n(&p->item_counter, p->counter_words, s));
+  // autotuning runs a launch by itself: the finished-segment counts start (and end) at zero
+  BL_CUDA(cudaMemsetAsync(p->item_counter, 0, p->counter_words * sizeof(int32_t), s));
+  if (p->nsplit > 0) BL_TRY(dalloc_n(&p->seg_sums, (size_t)p->nsplit * kMaxSegments * kTile, s));
   BL_TRY(build_chunk_frames(p, s));
   // Default layout: warps of empty rows skip their work when that saves at
   // least 2 % of the evaluations (many items smaller than a tile).

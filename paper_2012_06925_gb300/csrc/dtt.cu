@@ -665,7 +665,8 @@ __global__ void k_item_count(int32_t nct, ListView L, const int32_t* __restrict_
                              const int32_t* __restrict__ s_end, int32_t* __restrict__ nitems,
                              int64_t* __restrict__ cost_part, int64_t* __restrict__ cost_prox,
                              unsigned long long* __restrict__ executed,   // [2]: skip, no skip
-                             int64_t* __restrict__ eval_part, int64_t* __restrict__ eval_prox) {
+                             int64_t* __restrict__ eval_part, int64_t* __restrict__ eval_prox,
+                             int64_t part_len, int32_t* __restrict__ nsplit) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= nct) return;
   int64_t cp = 0, sp = 0;
@@ -676,7 +677,9 @@ __global__ void k_item_count(int32_t nct, ListView L, const int32_t* __restrict_
         class_work(L, s_begin, s_end, class_of(BLDTT_PC, i), false, i, a, sp, cp);
     }
   const int32_t tp = cp > 0 ? (end[c] - begin[c] + kTile - 1) / kTile : 0;
-  int32_t items = tp;
+  const PartPlan pp = plan_parts(cp, part_len);
+  int32_t items = tp * pp.parts;
+  int32_t split = pp.parts > 1 ? tp : 0;
   unsigned long long ex = cp > 0 ? (unsigned long long)executed_rows_skip(end[c] - begin[c]) * sp : 0ull;
   unsigned long long ex_ns = cp > 0 ? (unsigned long long)executed_rows_noskip(end[c] - begin[c]) * sp : 0ull;
   eval_part[c] = cp > 0 ? (int64_t)(end[c] - begin[c]) * sp : 0;   // real evaluations (no padding)
@@ -686,7 +689,9 @@ __global__ void k_item_count(int32_t nct, ListView L, const int32_t* __restrict_
     class_work(L, s_begin, s_end, class_of(BLDTT_CP, i), true, i, c, sq, cq);
     class_work(L, s_begin, s_end, class_of(BLDTT_CC, i), false, i, c, sq, cq);
     const int32_t tq = cq > 0 ? (L.deg.np[i] + kTile - 1) / kTile : 0;
-    items += tq;
+    const PartPlan pq = plan_parts(cq, part_len);
+    items += tq * pq.parts;
+    if (pq.parts > 1) split += tq;
     cost_prox[(int64_t)c * kMaxDegrees + i] = cq;
     if (cq > 0) {
       ex += (unsigned long long)executed_rows_skip(L.deg.np[i]) * sq;
@@ -697,6 +702,7 @@ __global__ void k_item_count(int32_t nct, ListView L, const int32_t* __restrict_
   eval_prox[c] = evq;
   nitems[c] = items;
   cost_part[c] = cp;
+  if (split) atomicAdd(nsplit, split);
   // evaluations the kernel performs: every target slot of every tile meets every real source
   if (ex) atomicAdd(executed, ex);
   if (ex_ns) atomicAdd(executed + 1, ex_ns);
@@ -711,16 +717,34 @@ struct SegmentMap {
   int kernel[8];
 };
 
+// The tasks of one tile {c, r, rows, kind} of `chunks` source chunks.
+__device__ __forceinline__ void fill_tasks(int4 tile, int64_t chunks, int64_t part_len, uint32_t key_base,
+                                           int32_t& o, int32_t* next_slot, int4* items, int4* parts,
+                                           uint32_t* keys, int32_t* vals) {
+  const PartPlan q = plan_parts(chunks, part_len);
+  // the slot numbers depend on the order of the atomics, the results do not
+  const int32_t slot = q.parts > 1 ? atomicAdd(next_slot, 1) : -1;
+  const uint32_t kKeyMax = (1u << 24) - 1u;
+  for (int32_t i = 0; i < q.parts; ++i) {
+    const int64_t b = (int64_t)i * q.per * q.len, e = min(chunks, b + (int64_t)q.per * q.len);
+    items[o] = tile;
+    parts[o] = make_int4((int)b, (int)(e - b), slot, q.nseg | (q.len << 8));
+    keys[o] = key_base | (kKeyMax - (uint32_t)min((int64_t)kKeyMax, e - b));
+    vals[o] = o;
+    ++o;
+  }
+}
+
 __global__ void k_item_fill(int32_t nct, const int32_t* __restrict__ off,
                             const int64_t* __restrict__ cost_part, const int64_t* __restrict__ cost_prox,
                             const int32_t* __restrict__ begin, const int32_t* __restrict__ end,
                             const int32_t* __restrict__ problem, const int* __restrict__ prob_kernel,
-                            SegmentMap segmap, DegreeSet deg, int4* __restrict__ items,
-                            uint32_t* __restrict__ keys, int32_t* __restrict__ vals) {
+                            SegmentMap segmap, DegreeSet deg, int64_t part_len, int32_t* __restrict__ next_slot,
+                            int4* __restrict__ items, int4* __restrict__ parts, uint32_t* __restrict__ keys,
+                            int32_t* __restrict__ vals) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= nct) return;
   int32_t o = off[c];
-  const uint32_t kKeyMax = (1u << 24) - 1u;
   uint32_t seg = 0;
   uint32_t sub = 0;          // the shared Coulomb/Yukawa launch: Coulomb items first
   const int kern = prob_kernel[problem[c]];
@@ -730,26 +754,18 @@ __global__ void k_item_fill(int32_t nct, const int32_t* __restrict__ off,
       seg = (uint32_t)i;
       sub = segmap.kernel[i] == kKernCoulombYukawa && kern == BLDTT_YUKAWA ? 1u : 0u;
     }
-  if (cost_part[c] > 0) {
-    uint32_t k = (seg << 25) | (sub << 24) | (kKeyMax - (uint32_t)min((int64_t)kKeyMax, cost_part[c]));
-    for (int32_t r = begin[c]; r < end[c]; r += kTile) {
-      items[o] = make_int4(c, r, min(kTile, end[c] - r), kItemParticles);
-      keys[o] = k;
-      vals[o] = o;
-      ++o;
-    }
-  }
+  const uint32_t key_base = (seg << 25) | (sub << 24);
+  if (cost_part[c] > 0)
+    for (int32_t r = begin[c]; r < end[c]; r += kTile)
+      fill_tasks(make_int4(c, r, min(kTile, end[c] - r), kItemParticles), cost_part[c], part_len, key_base, o,
+                 next_slot, items, parts, keys, vals);
   for (int i = 0; i < deg.n; ++i) {
     const int64_t cq = cost_prox[(int64_t)c * kMaxDegrees + i];
     if (cq <= 0) continue;
     const int32_t np = deg.np[i];
-    uint32_t k = (seg << 25) | (sub << 24) | (kKeyMax - (uint32_t)min((int64_t)kKeyMax, cq));
-    for (int32_t r = 0; r < np; r += kTile) {
-      items[o] = make_int4(c, r, min(kTile, np - r), kItemProxies + i);
-      keys[o] = k;
-      vals[o] = o;
-      ++o;
-    }
+    for (int32_t r = 0; r < np; r += kTile)
+      fill_tasks(make_int4(c, r, min(kTile, np - r), kItemProxies + i), cq, part_len, key_base, o, next_slot,
+                 items, parts, keys, vals);
   }
 }
 
@@ -761,10 +777,14 @@ __global__ void k_segment_starts(const uint32_t* __restrict__ keys, int32_t n, i
   if (i == 0 || (keys[i - 1] >> 25) != sg) first[sg] = i;
 }
 
-__global__ void k_gather_items(const int4* __restrict__ src, const int32_t* __restrict__ idx,
-                               int4* __restrict__ dst, int64_t n) {
+__global__ void k_gather_items(const int4* __restrict__ src, const int4* __restrict__ psrc,
+                               const int32_t* __restrict__ idx, int4* __restrict__ dst,
+                               int4* __restrict__ pdst, int64_t n) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = src[idx[i]];
+  if (i < n) {
+    dst[i] = src[idx[i]];
+    pdst[i] = psrc[idx[i]];
+  }
 }
 
 // Bounding box of every 32-row group of every work item (the targets one warp
@@ -816,6 +836,27 @@ __global__ void k_item_boxes(int32_t nitems, const int4* __restrict__ items, con
   }
 }
 
+// Chunks of a task: a tile's sources are split so that the plan's tile-chunks
+// (counted from its kernel evaluations) make about kTasksPerCta tasks per CTA
+// of six on an SM, but not below a few chunks, where a task's start costs more
+// than the even load gives.  Measured (interaction kernel, GB300): 1E6 points
+// (1.9E6 tile-chunks) 31.9 ms at 4 tasks per CTA, 31.4 at 16-24, 31.3 at 50
+// with 0.2 ms more to list them; 2E4 points on a sphere (4800) 0.25 ms at 1-3
+// chunks, 0.18 at 4-6, 0.21 at 8, 0.45 whole; 2E4 points in FP64 9.6 ms at 1-3,
+// 9.9 at 8, 28 whole.  A plan of many short tiles (512 problems) is not split.
+constexpr int kTasksPerCta = 16;
+static int64_t task_chunks(const bldtt_plan* p) {
+  if (const char* e = std::getenv("BLDTT_TASK_CHUNKS"))   // testing: results do not depend on the split
+    return std::max<int64_t>(1, std::strtoll(e, nullptr, 10));
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess || sms < 1) sms = 1;
+  double evals = 0.0;
+  for (int k = 0; k < 4; ++k) evals += p->interactions[k];
+  const double tiles = evals / ((double)kTile * kChunk);
+  return std::max<int64_t>(p->precision == BLDTT_FP32_BULK ? 4 : 2,
+                           (int64_t)(tiles / ((double)sms * 6 * kTasksPerCta)));
+}
+
 int build_work_items(bldtt_plan* p, cudaStream_t s) {
   bldtt::Counters& cnt = p->setup_counter;
   const Tree& st = p->st;
@@ -853,19 +894,21 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
   dfree_ptr(p->eval_prox, s);
   BL_TRY(dalloc_n(&p->eval_part, nct, s));
   BL_TRY(dalloc_n(&p->eval_prox, nct, s));
+  int32_t* totals = nullptr;   // [0] items, [1] padded pool particles, [2] split tiles, [3] next split slot
+  BL_TRY(dalloc_n(&totals, 4, s));
+  BL_CUDA(cudaMemsetAsync(totals, 0, 4 * sizeof(int32_t), s));
+  const int64_t part_len = task_chunks(p);
   k_item_count<<<nblk(nct, 128), 128, 0, s>>>(nct, L, tt.parent, tt.nchild, tt.begin, tt.end,
                                               st.begin, st.end, nitems, cost_part, cost_prox,
-                                              executed, p->eval_part, p->eval_prox);
+                                              executed, p->eval_part, p->eval_prox, part_len, totals + 2);
   BL_LAUNCHED(cnt.launches);
-  int32_t* totals = nullptr;   // [0] items, [1] padded pool particles
-  BL_TRY(dalloc_n(&totals, 2, s));
   BL_TRY(scan_exclusive_dev(nitems, off, nct, totals, s, cnt));
   BL_CUDA(cudaMemcpyAsync(totals + 1, p->pad_prefix + st.nleaves, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-  int32_t h_tot[2];
+  int32_t h_tot[3];
   BL_TRY(read_device(totals, h_tot, sizeof(h_tot), s));
-  dfree(totals, s);
   const int32_t ni = h_tot[0];
   p->nitems = ni;
+  p->nsplit = h_tot[2];
   p->pool_particles = h_tot[1];
   p->pool_len = h_tot[1];
   for (int i = 0; i < p->deg.n; ++i) {   // proxy blocks of every source cluster, per degree
@@ -873,10 +916,12 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
     p->pool_len += (int64_t)st.nclusters * p->deg.np_pad[i];
   }
   p->np_pad = p->deg.np_pad[p->deg.n - 1];
-  int4* items = nullptr;
+  int4 *items = nullptr, *parts = nullptr;
   uint32_t* keys = nullptr;
   int32_t* vals = nullptr;
   BL_TRY(dalloc_n(&items, ni, s));
+  BL_TRY(dalloc_n(&parts, ni, s));
+  BL_TRY(dalloc_n(&p->parts, ni, s));
   BL_TRY(dalloc_n(&keys, ni, s));
   BL_TRY(dalloc_n(&vals, ni, s));
   BL_TRY(dalloc_n(&p->items, ni, s));
@@ -884,8 +929,8 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
   segmap.n = (int)p->segment_kernels.size();
   for (int i = 0; i < segmap.n; ++i) segmap.kernel[i] = p->segment_kernels[i];
   k_item_fill<<<nblk(nct, 128), 128, 0, s>>>(nct, off, cost_part, cost_prox, tt.begin, tt.end,
-                                             tt.problem, p->prob_kernel, segmap, p->deg, items, keys,
-                                             vals);
+                                             tt.problem, p->prob_kernel, segmap, p->deg, part_len, totals + 3,
+                                             items, parts, keys, vals);
   BL_LAUNCHED(cnt.launches);
   // Grouped by kernel, longest items first within a group (stable), so that
   // each persistent launch's tail is short.
@@ -905,7 +950,7 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
   }
   int32_t h_first[8];
   if (ni > 0) {
-    k_gather_items<<<nblk(ni, 256), 256, 0, s>>>(items, vals, p->items, ni);
+    k_gather_items<<<nblk(ni, 256), 256, 0, s>>>(items, parts, vals, p->items, p->parts, ni);
     BL_LAUNCHED(cnt.launches);
   }
   if (p->precision == BLDTT_FP32_BULK && ni > 0) {
@@ -936,7 +981,7 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
       }
     p->segments.push_back({segmap.kernel[i], h_first[i], end - h_first[i], 0, 0, 0});
   }
-  dfree(items, s); dfree(keys, s); dfree(vals, s);
+  dfree(items, s); dfree(parts, s); dfree(keys, s); dfree(vals, s); dfree(totals, s);
   dfree(nitems, s); dfree(off, s); dfree(cost_part, s); dfree(cost_prox, s);
   return BLDTT_OK;
 }

@@ -11,10 +11,16 @@
 //                   particles)
 //   proxy tiles:    CP and CC entries of one degree on the cluster itself
 //                   (the targets are that degree's proxy points).
-// Each item owns its outputs, so there are no atomics and the summation order
-// is fixed.
+// Each item owns its outputs and its summation order is fixed.
 //
-// Per CTA, one producer warp grabs items from a global counter, walks their
+// An item with many source chunks is split into tasks over its chunks
+// (plan_parts), so that a plan with few items still fills the device and the
+// last tasks are short: 2E4 points make ~200 items for 152 SMs x 6 CTAs, and
+// the launch lasted as long as the longest of them (interaction kernel, GB300:
+// FP64 at 2E4 points, n = 4, 28.3 -> 9.6 ms; FP64 Yukawa at 6E4 321 -> 51 ms;
+// FP32 on a sphere of 2E4 0.45 -> 0.18 ms; 1E6 points 32.4 -> 31.4 ms).
+//
+// Per CTA, one producer warp takes tasks from a global counter, walks their
 // lists and streams the sources, kChunk at a time, from the source pool into
 // a shared-memory ring (3 or 4 stages) with cp.async.bulk (TMA) copies that
 // complete on mbarriers; NCW consumer warps evaluate G for K targets per
@@ -57,6 +63,9 @@ constexpr uint64_t kWaitNs = 20ull * 1000ull * 1000ull * 1000ull;   // 20 s boun
 
 struct InteractView {
   const int4* items;
+  const int4* parts;            // {first chunk, chunks, segment-sum slot or -1, segments | segment length << 8}
+  double* seg_sums;             // [slots][kMaxSegments][kTile]
+  int32_t* arrived;             // [slots][kItemGroups]: segments finished, per consumer warp
   int32_t nitems;
   int32_t* counter;
   // lists and source layout (producer)
@@ -87,12 +96,17 @@ struct InteractView {
   const int* prob_kernel;      // kernel of each problem (read per item by the fused launch)
 };
 
+// Flags of a staged chunk: first of its task, last of its segment, last of its task.
+constexpr unsigned kTaskStart = 1, kSegEnd = 2, kTaskEnd = 4;
+
 struct StageMeta {
-  int item;
+  int item;                     // task index (-1: no more work)
   int count;                    // real sources in the staged chunk
-  int chunk;                    // pool chunk index
+  int slot;                     // split item: its segment-sum slot (-1: the task is a whole item)
+  int seg;                      // the chunk's segment
+  unsigned flags;               // kTaskStart | kSegEnd | kTaskEnd
   unsigned near;                // bit g: target group g may be near the chunk (residuals staged)
-  unsigned long long c2[3];     // frame centre, each component duplicated (f32x2)
+  float c[3];                   // frame centre
   float4 ext;                   // half-extents and near distance tau (-inf: proxies)
 };
 
@@ -127,17 +141,22 @@ __device__ __forceinline__ uint64_t global_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-// Bounded wait: gives up after kWaitNs, raising the plan's error flag.
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int* err) {
-  if (mbar_try_wait(b, parity)) return true;
+// Bounded wait: gives up after kWaitNs, raising the plan's error flag.  The
+// clock is read every 256th attempt only, and the producer sleeps between
+// attempts: a waiting warp shares the issue slots with the warps that compute.
+__device__ __noinline__ bool mbar_wait_slow(uint64_t* b, uint32_t parity, int* err, uint32_t sleep_ns) {
   const uint64_t t0 = global_ns();
-  while (!mbar_try_wait(b, parity)) {
-    if (global_ns() - t0 > kWaitNs) {
+  for (uint32_t n = 1;; ++n) {
+    if (sleep_ns) __nanosleep(sleep_ns);
+    if (mbar_try_wait(b, parity)) return true;
+    if ((n & 255u) == 0 && global_ns() - t0 > kWaitNs) {
       atomicExch(err, kDevErrTimeout);
       return false;
     }
   }
-  return true;
+}
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int* err, uint32_t sleep_ns = 0) {
+  return mbar_try_wait(b, parity) || mbar_wait_slow(b, parity, err, sleep_ns);
 }
 __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, uint32_t bytes,
                                               uint64_t* bar) {
@@ -236,7 +255,11 @@ __device__ __forceinline__ double pair_f64(double dx, double dy, double dz, doub
   return q * ri * exp(-kappa * (r2 * ri));
 }
 
-// ---- producer: walks an item's segments ------------------------------------
+// ---- producer: walks a task's lists -----------------------------------------
+// One warp.  The lanes read the lists 32 entries at a time (source cluster,
+// pool range), so a task that starts in the middle of its item's chunks skips
+// to it in a few memory latencies, and a chunk's near-group test runs on one
+// lane per group; lane 0 issues the copies.
 template <typename Vec, int RES, int STAGES>
 struct Producer {
   const InteractView& v;
@@ -245,139 +268,176 @@ struct Producer {
   StageMeta* meta;
   uint64_t* full;
   uint64_t* empty;
+  const int lane;
   uint32_t it = 0;
   int cur_item = -1;
-  int cur_groups = 0;
-  float* ibox;                  // [6] bounding box of the current item's targets (shared memory)
+  int slot = -1, seg_len = 1;
+  int seg = 0, seg_left = 1;    // the next chunk's segment, chunks left in it
+  int skip = 0, left = 0;       // chunks before the task's first, chunks still to stage
+  unsigned start = 0;           // kTaskStart until the task's first chunk is staged
+  bool has_box = false;
+  float4 glo, ghi;              // lane g: box of the task's target group g
 
   __device__ Producer(const InteractView& v_, Vec (*b)[kChunk], float4 (*r)[RES], StageMeta* m,
-                      uint64_t* f, uint64_t* e, float* box)
-      : v(v_), buf(b), rbuf(r), meta(m), full(f), empty(e), ibox(box) {}
+                      uint64_t* f, uint64_t* e, int lane_)
+      : v(v_), buf(b), rbuf(r), meta(m), full(f), empty(e), lane(lane_) {}
 
-  __device__ __noinline__ void load_item_box() {
-    const float4* gb = v.item_box + (int64_t)cur_item * (2 * kItemGroups);
-    float b[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
-    for (int g = 0; g < cur_groups; ++g) {
-      const float4 lo = gb[2 * g], hi = gb[2 * g + 1];
-      b[0] = fminf(b[0], lo.x);
-      b[1] = fminf(b[1], lo.y);
-      b[2] = fminf(b[2], lo.z);
-      b[3] = fmaxf(b[3], hi.x);
-      b[4] = fmaxf(b[4], hi.y);
-      b[5] = fmaxf(b[5], hi.z);
-    }
-    for (int d = 0; d < 6; ++d) ibox[d] = b[d];
-  }
-
-  // Target groups of the current item whose box comes within tau of the
+  // Target groups of the current task whose box comes within tau of the
   // particle chunk's box (c +- e): a superset of the targets the consumers'
-  // own test finds near.  The item's box is tested first.
+  // own test finds near.
   __device__ __forceinline__ unsigned near_groups(const float4& f, const float4& ext) const {
     if (!(ext.w >= 0.f)) return 0u;       // proxy chunk
-    const float gap = fmaxf(fmaxf(fmaxf(ibox[0] - (f.x + ext.x), (f.x - ext.x) - ibox[3]),
-                                  fmaxf(ibox[1] - (f.y + ext.y), (f.y - ext.y) - ibox[4])),
-                            fmaxf(ibox[2] - (f.z + ext.z), (f.z - ext.z) - ibox[5]));
-    return gap < ext.w ? near_groups_of_item(f, ext) : 0u;
-  }
-  __device__ __noinline__ unsigned near_groups_of_item(const float4 f, const float4 ext) const {
-    const float clo[3] = {f.x - ext.x, f.y - ext.y, f.z - ext.z};
-    const float chi[3] = {f.x + ext.x, f.y + ext.y, f.z + ext.z};
-    const float4* gb = v.item_box + (int64_t)cur_item * (2 * kItemGroups);
-    unsigned mask = 0;
-    for (int g = 0; g < cur_groups; ++g) {
-      const float4 lo = gb[2 * g], hi = gb[2 * g + 1];
-      const float gap = fmaxf(fmaxf(fmaxf(lo.x - chi[0], clo[0] - hi.x), fmaxf(lo.y - chi[1], clo[1] - hi.y)),
-                              fmaxf(lo.z - chi[2], clo[2] - hi.z));
-      if (gap < ext.w) mask |= 1u << g;
-    }
-    return mask;
+    const float gap = fmaxf(fmaxf(fmaxf(glo.x - (f.x + ext.x), (f.x - ext.x) - ghi.x),
+                                  fmaxf(glo.y - (f.y + ext.y), (f.y - ext.y) - ghi.y)),
+                            fmaxf(glo.z - (f.z + ext.z), (f.z - ext.z) - ghi.z));
+    return __ballot_sync(0xffffffffu, has_box && gap < ext.w);
   }
 
-  __device__ bool acquire(int& s) {
+  __device__ __forceinline__ bool acquire(int& s) {
     s = (int)(it % STAGES);
-    return mbar_wait(&empty[s], ((it / STAGES) & 1u) ^ 1u, v.err);
+    return __all_sync(0xffffffffu, mbar_wait(&empty[s], ((it / STAGES) & 1u) ^ 1u, v.err, 500u));
   }
 
-  // Stream pool entries [off, off + len) in kChunk pieces (real entries only).
-  __device__ bool segment(int64_t off, int64_t len) {
-    for (int64_t k = 0; k < len; k += kChunk) {
-      int s;
-      if (!acquire(s)) return false;
-      const int64_t q = (off + k) / kChunk;
-      const float4 f = v.chunk_frame[kChunkInfo * q];
+  // Stage pool chunk q (real entries only).
+  __device__ __forceinline__ bool stage(int q) {
+    const float4 f = v.chunk_frame[(int64_t)kChunkInfo * q];
+    float4 ext = make_float4(0.f, 0.f, 0.f, 0.f);
+    unsigned near = 0;
+    if (std::is_same<Vec, float4>::value) {
+      ext = v.chunk_frame[(int64_t)kChunkInfo * q + 1];
+      near = near_groups(f, ext);
+    }
+    int s;
+    if (!acquire(s)) return false;
+    if (lane == 0) {
       const int count = __float_as_int(f.w);
       StageMeta& m = meta[s];
       m.item = cur_item;
       m.count = count;
-      m.chunk = (int)q;
-      m.near = 0;
+      m.slot = slot;
+      m.seg = seg;
+      m.flags = start | (seg_left == 1 || left == 1 ? kSegEnd : 0u) | (left == 1 ? kTaskEnd : 0u);
+      m.near = near;
       uint32_t bytes;
       if (std::is_same<Vec, float4>::value) {
-        m.c2[0] = f2_pack(f.x, f.x);
-        m.c2[1] = f2_pack(f.y, f.y);
-        m.c2[2] = f2_pack(f.z, f.z);
-        m.ext = v.chunk_frame[kChunkInfo * q + 1];
-        m.near = near_groups(f, m.ext);
+        m.c[0] = f.x;
+        m.c[1] = f.y;
+        m.c[2] = f.z;
+        m.ext = ext;
         bytes = (uint32_t)(((count + 1) / 2) * 32);          // whole pair records
       } else {
         bytes = (uint32_t)(count * sizeof(Vec));
       }
-      const char* src = reinterpret_cast<const char*>(v.pool) + (off + k) * (int64_t)sizeof(Vec);
-      mbar_arrive_tx(&full[s], m.near ? 2 * bytes : bytes);
+      const char* src = reinterpret_cast<const char*>(v.pool) + (int64_t)q * (kChunk * (int64_t)sizeof(Vec));
+      mbar_arrive_tx(&full[s], near ? 2 * bytes : bytes);
       bulk_copy_g2s(buf[s], src, bytes, &full[s]);
-      if (RES == kChunk && m.near)     // the chunk's frame residuals, same record layout
-        bulk_copy_g2s(rbuf[s], v.pool_res + q * (int64_t)(kChunk * 4), bytes, &full[s]);
-      ++it;
+      if (RES == kChunk && near)       // the chunk's frame residuals, same record layout
+        bulk_copy_g2s(rbuf[s], v.pool_res + (int64_t)q * (kChunk * 4), bytes, &full[s]);
+    }
+    __syncwarp();
+    ++it;
+    --left;
+    if (--seg_left == 0) {
+      seg_left = seg_len;
+      ++seg;
+    }
+    start = 0;
+    return true;
+  }
+
+  // Entries [e0, e1) of one list: the particles of the source clusters (i < 0;
+  // all leaves under a cluster are one contiguous pool range, because they are
+  // consecutive in leaf order) or their proxy blocks of degree index i.
+  __device__ bool entries(int32_t e0, int32_t e1, int i) {
+    for (int32_t base = e0; base < e1 && left > 0; base += 32) {
+      int o = 0, n = 0;
+      if (base + lane < e1) {
+        const int32_t src = v.list_src[base + lane];
+        if (i < 0) {
+          const int32_t p0 = v.pad_prefix[v.s_leaf_first[src]], p1 = v.pad_prefix[v.s_leaf_last[src]];
+          o = p0 / kChunk;
+          n = (p1 - p0) / kChunk;
+        } else {
+          n = v.deg.np_pad[i] / kChunk;
+          o = (int)(v.deg.proxy_base[i] / kChunk) + src * n;
+        }
+      }
+      const int cnt = min(32, e1 - base);
+      for (int j = 0; j < cnt && left > 0; ++j) {
+        const int oj = __shfl_sync(0xffffffffu, o, j), nj = __shfl_sync(0xffffffffu, n, j);
+        if (skip >= nj) {
+          skip -= nj;
+          continue;
+        }
+        for (int k = skip; k < nj && left > 0; ++k)
+          if (!stage(oj + k)) return false;
+        skip = 0;
+      }
     }
     return true;
   }
 
-  // Particles of all source leaves under cluster s: one contiguous pool range,
-  // because leaves under a cluster are consecutive in leaf order.
-  __device__ bool leaves_of(int32_t s) {
-    int64_t o = v.pad_prefix[v.s_leaf_first[s]];
-    return segment(o, v.pad_prefix[v.s_leaf_last[s]] - o);
-  }
-
-  // Entries of list class cls of target cluster c: particles of the source
-  // clusters, or their proxy blocks of degree index i (i >= 0).
-  __device__ bool entries(int cls, int i, int32_t c) {
-    const int64_t k = (int64_t)cls * v.nct + c;
-    for (int32_t e = v.list_ptr[k]; e < v.list_ptr[k + 1]; ++e) {
-      const int32_t src = v.list_src[e];
-      const bool ok = i < 0 ? leaves_of(src)
-                            : segment(v.deg.proxy_base[i] + (int64_t)src * v.deg.np_pad[i], v.deg.np_pad[i]);
-      if (!ok) return false;
+  // The lists of target cluster a: class cls0 as particles (degree index -1),
+  // and for lane l in [1, nlists) the class of lane l as proxies of degree
+  // index deg_of(l); one list_ptr pair per lane.
+  __device__ bool run_particles(int32_t leaf) {   // PP and PC of every degree, leaf and ancestors
+    for (int32_t a = leaf; a >= 0 && left > 0;) {
+      const int32_t up = v.t_parent[a];
+      int32_t e0 = 0, e1 = 0;
+      if (lane <= v.deg.n) {
+        const int64_t k = (int64_t)(lane == 0 ? 0 : class_of(BLDTT_PC, lane - 1)) * v.nct + a;
+        e0 = v.list_ptr[k];
+        e1 = v.list_ptr[k + 1];
+      }
+      unsigned todo = __ballot_sync(0xffffffffu, e1 > e0);
+      while (todo) {
+        const int j = __ffs(todo) - 1;
+        todo &= todo - 1;
+        if (!entries(__shfl_sync(0xffffffffu, e0, j), __shfl_sync(0xffffffffu, e1, j), j - 1)) return false;
+      }
+      a = up;
     }
     return true;
   }
 
   __device__ void run() {
     bool ok = true;
-    for (;;) {
-      int idx = atomicAdd(v.counter, 1);
+    while (ok) {
+      int idx = 0;
+      if (lane == 0) idx = atomicAdd(v.counter, 1);
+      idx = __shfl_sync(0xffffffffu, idx, 0);
       if (idx >= v.nitems) break;
-      int4 item = v.items[idx];
+      const int4 item = v.items[idx], part = v.parts[idx];
       cur_item = idx;
-      cur_groups = (item.z + 31) / 32;
-      if (std::is_same<Vec, float4>::value) load_item_box();
-      if (item.w == kItemParticles) {   // PP and PC of every degree, leaf and ancestors
-        for (int32_t a = item.x; a >= 0 && ok; a = v.t_parent[a]) {
-          ok = entries(0, -1, a);
-          for (int i = 0; i < v.deg.n && ok; ++i) ok = entries(class_of(BLDTT_PC, i), i, a);
-        }
+      skip = part.x;
+      left = part.y;
+      slot = part.z;
+      seg_len = seg_left = part.w >> 8;           // a task starts at a segment's start
+      seg = part.x / seg_len;
+      start = kTaskStart;
+      has_box = std::is_same<Vec, float4>::value && lane < (item.z + 31) / 32;
+      if (has_box) {
+        const float4* gb = v.item_box + (int64_t)idx * (2 * kItemGroups);
+        glo = gb[2 * lane];
+        ghi = gb[2 * lane + 1];
+      }
+      if (item.w == kItemParticles) {
+        ok = run_particles(item.x);
       } else {                          // CP and CC of one degree on the cluster itself
         const int i = item.w - kItemProxies;
-        ok = entries(class_of(BLDTT_CP, i), -1, item.x) && entries(class_of(BLDTT_CC, i), i, item.x);
+        const int64_t k0 = (int64_t)class_of(BLDTT_CP, i) * v.nct + item.x;
+        const int64_t k1 = (int64_t)class_of(BLDTT_CC, i) * v.nct + item.x;
+        const int32_t a0 = v.list_ptr[k0], a1 = v.list_ptr[k0 + 1], b0 = v.list_ptr[k1], b1 = v.list_ptr[k1 + 1];
+        ok = entries(a0, a1, -1) && entries(b0, b1, i);
       }
-      if (!ok) break;
     }
     if (ok) {
       int s;
       if (acquire(s)) {
-        meta[s].item = -1;
-        mbar_arrive(&full[s]);
-        ++it;
+        if (lane == 0) {
+          meta[s].item = -1;
+          mbar_arrive(&full[s]);
+        }
         return;
       }
     }
@@ -450,27 +510,26 @@ __device__ __forceinline__ void chunk_f32(const ulonglong2* __restrict__ sb, int
   }
 }
 
-// A consumer thread's targets, split v = hi + lo in FP32 (each duplicated
-// f32x2), kept in shared memory rather than registers: entry (k, d) of the
-// thread is h[(3k + d) * stride].
+// A consumer thread's targets, split v = hi + lo in FP32 and kept in shared
+// memory rather than registers, (hi, lo) in one word: entry (k, d) of the
+// thread is v[(3k + d) * stride].  (Kept duplicated for the packed subtraction
+// they took 12 KB of a CTA's shared memory; with the items' totals beside them
+// only five of the six CTAs then fit an SM: 32.4 -> 32.9 ms at 1E6.)
 struct TargetSplit {
-  const f2_t* h;
-  const f2_t* l;
+  const f2_t* v;
   int stride;
-  __device__ __forceinline__ f2_t hi(int k, int d) const { return h[(3 * k + d) * stride]; }
-  __device__ __forceinline__ f2_t lo(int k, int d) const { return l[(3 * k + d) * stride]; }
+  __device__ __forceinline__ void get(int k, int d, float& hi, float& lo) const {
+    f2_unpack(v[(3 * k + d) * stride], hi, lo);
+  }
 };
 
-// Frame residual (frame_resid) of target slot k in the chunk's frame c2.
-__device__ __forceinline__ void target_residual(const TargetSplit& ts, const f2_t* c2, int k,
-                                                float (&xr)[3]) {
+// Frame residual (frame_resid) of target slot k in the chunk's frame c.
+__device__ __forceinline__ void target_residual(const TargetSplit& ts, const float* c, int k, float (&xr)[3]) {
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    float c, h, l, hi;
-    f2_unpack(c2[d], c, hi);
-    f2_unpack(ts.hi(k, d), h, hi);
-    f2_unpack(ts.lo(k, d), l, hi);
-    xr[d] = frame_resid(h, l, c);
+    float h, l;
+    ts.get(k, d, h, l);
+    xr[d] = frame_resid(h, l, c[d]);
   }
 }
 
@@ -479,7 +538,7 @@ template <int KERN, int K>
 __device__ __forceinline__ void chunk_f32_careful(const ulonglong2* __restrict__ sb,
                                                   const ulonglong2* __restrict__ sr, int npairs,
                                                   const f2_t (&x2)[K][3], const TargetSplit& ts,
-                                                  const f2_t* c2, unsigned near, float (&a)[K],
+                                                  const float* c, unsigned near, float (&a)[K],
                                                   float nk) {
   const f2_t nk2 = f2_pack(nk, nk);
   f2_t acc[K], m2[K], r2x[K][3];
@@ -488,7 +547,7 @@ __device__ __forceinline__ void chunk_f32_careful(const ulonglong2* __restrict__
     const float m = ((near >> k) & 1u) ? 1.f : 0.f;
     m2[k] = f2_pack(m, m);
     float xr[3];
-    target_residual(ts, c2, k, xr);
+    target_residual(ts, c, k, xr);
 #pragma unroll
     for (int d = 0; d < 3; ++d) r2x[k][d] = f2_pack(xr[d], xr[d]);
     acc[k] = 0ull;
@@ -535,14 +594,14 @@ __device__ __forceinline__ float pair_acc_f32(float dx, float dy, float dz, floa
 template <int KERN, int K>
 __device__ __forceinline__ void chunk_f32_slow(const float* __restrict__ sf, const float* __restrict__ res,
                                                int count, const float (&xs)[K][3],
-                                               const TargetSplit& ts, const f2_t* c2, unsigned near,
+                                               const TargetSplit& ts, const float* c, unsigned near,
                                                float prm, float (&a)[K]) {
   // one target slot at a time: few live registers on this rare path
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const bool nr = (near >> k) & 1u;
     float xr[3] = {0.f, 0.f, 0.f};
-    if (nr) target_residual(ts, c2, k, xr);
+    if (nr) target_residual(ts, c, k, xr);
     float acc0 = 0.f, acc1 = 0.f;
     for (int jp = 0; jp < (count + 1) / 2; ++jp) {
 #pragma unroll
@@ -617,6 +676,51 @@ __device__ __forceinline__ void store_output(const InteractView& v, const int4& 
   }
 }
 
+template <int K>
+struct SegSums {
+  double v[K];
+};
+// End of a split item's segment or of an item, per consumer warp (out of line:
+// no register of the packed loop).  A whole item adds the last segment's sums
+// to its totals (tot, in shared memory) and stores them.  A split item's sums go to memory; the
+// warp that finds every segment of the item finished adds them in segment
+// order, the order in which a whole item adds them (so the split does not
+// change the bits), and resets the count for the next compute.
+template <int NCW, int K>
+__device__ __noinline__ void end_segment(const InteractView& v, const int4 item, int task, int slot, int seg,
+                                         unsigned flags, const SegSums<K> a, double* tot) {
+  const int ct = threadIdx.x, lane = ct & 31;
+  if (slot < 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int r = k * NCW * 32 + ct;
+      store_output(v, item, r, tot[r] + a.v[k]);
+    }
+    return;
+  }
+  double* sums = v.seg_sums + (int64_t)slot * (kMaxSegments * kTile);
+#pragma unroll
+  for (int k = 0; k < K; ++k) sums[seg * kTile + k * NCW * 32 + ct] = a.v[k];
+  if (!(flags & kTaskEnd)) return;
+  const int4 part = v.parts[task];
+  const int nseg = part.w & 0xff, len = part.w >> 8;
+  const int mine = (part.x + part.y + len - 1) / len - part.x / len;
+  int32_t* count = v.arrived + (int64_t)slot * kItemGroups + (ct >> 5);
+  __threadfence();
+  __syncwarp();
+  int done = 0;
+  if (lane == 0) done = atomicAdd(count, mine) + mine;
+  if (__shfl_sync(0xffffffffu, done, 0) != nseg) return;
+  __threadfence();
+  for (int k = 0; k < K; ++k) {
+    const int r = k * NCW * 32 + ct;
+    double t = 0.0;
+    for (int g = 0; g < nseg; ++g) t += __ldcg(sums + g * kTile + r);
+    store_output(v, item, r, t);
+  }
+  if (lane == 0) *count = 0;
+}
+
 // Out-of-line entries to the rare paths of the packed kernels, so that their
 // registers do not burden the packed loop: they rebuild the targets' frame
 // coordinates from the shared-memory split (the same rounding as the packed
@@ -626,20 +730,24 @@ struct PartialSums {
   float v[K];
 };
 template <int K>
-__device__ __forceinline__ void frame_targets(const TargetSplit& ts, const f2_t* c2, f2_t (&x2)[K][3]) {
+__device__ __forceinline__ void frame_targets(const TargetSplit& ts, const float* c, f2_t (&x2)[K][3]) {
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const f2_t c = c2[d];
 #pragma unroll
-    for (int k = 0; k < K; ++k) x2[k][d] = f2_add(f2_sub(ts.hi(k, d), c), ts.lo(k, d));
+    for (int k = 0; k < K; ++k) {
+      float h, l;
+      ts.get(k, d, h, l);
+      const float x = frame_main(h, l, c[d]);
+      x2[k][d] = f2_pack(x, x);
+    }
   }
 }
 template <int KERN, int K>
 __device__ __noinline__ PartialSums<K> slow_sums(const float* sf, const float* res, int count,
-                                                 const TargetSplit ts, const f2_t* c2, unsigned near,
+                                                 const TargetSplit ts, const float* c, unsigned near,
                                                  float prm) {
   f2_t x2[K][3];
-  frame_targets<K>(ts, c2, x2);
+  frame_targets<K>(ts, c, x2);
   float xs[K][3];
 #pragma unroll
   for (int k = 0; k < K; ++k)
@@ -649,12 +757,11 @@ __device__ __noinline__ PartialSums<K> slow_sums(const float* sf, const float* r
       f2_unpack(x2[k][d], xs[k][d], hi);
     }
   PartialSums<K> out;
-  chunk_f32_slow<KERN, K>(sf, res, count, xs, ts, c2, near, prm, out.v);
+  chunk_f32_slow<KERN, K>(sf, res, count, xs, ts, c, near, prm, out.v);
   return out;
 }
 // One staged chunk in FP32 for K targets (partial sums in a[]).  ts holds
-// the targets' FP32 splits and c2 the chunk's frame centre (duplicated
-// f32x2), x2 the targets' frame coordinates, ext the chunk's half-extents and
+// the targets' FP32 splits and c the chunk's frame centre, x2 the targets' frame coordinates, ext the chunk's half-extents and
 // near distance tau, res its staged frame residuals, and bit k of `slot` says
 // that the producer found target slot k's group near the chunk.  A target
 // with max_d (|x''_d| - e_d) < tau is near: the warp then takes the careful
@@ -664,7 +771,7 @@ __device__ __noinline__ PartialSums<K> slow_sums(const float* sf, const float* r
 template <int KERN, int K>
 __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rbuf, int count,
                                                const f2_t (&x2)[K][3], const TargetSplit& ts,
-                                               const f2_t* c2, const float4* ext_p, unsigned slot, bool warp_full,
+                                               const float* c, const float4* ext_p, unsigned slot, bool warp_full,
                                                float prm, float (&a)[K]) {
   const float* sf = reinterpret_cast<const float*>(buf);
   const float* res = reinterpret_cast<const float*>(rbuf);
@@ -689,13 +796,13 @@ __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rb
     any_near = __any_sync(0xffffffffu, near != 0);
   }
   if (AlwaysGuarded<KERN>::value) {
-    chunk_f32_slow<KERN, K>(sf, res, count, xs, ts, c2, near, prm, a);
+    chunk_f32_slow<KERN, K>(sf, res, count, xs, ts, c, near, prm, a);
     return;
   }
   const ulonglong2* sb = reinterpret_cast<const ulonglong2*>(buf);
   if (any_near) {
     chunk_f32_careful<KERN, K>(sb, reinterpret_cast<const ulonglong2*>(rbuf), (count + 1) / 2, x2, ts,
-                               c2, near, a, prm);
+                               c, near, a, prm);
   } else if (K > 1 && !warp_full) {
     // the warp's last target row lies beyond a partial tile: evaluate the others only
     constexpr int K1 = K > 1 ? K - 1 : 1;
@@ -711,7 +818,7 @@ __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rb
 #pragma unroll
   for (int k = 0; k < K; ++k) bad = bad || not_finite(a[k]);
   if (__any_sync(0xffffffffu, bad)) {
-    const PartialSums<K> r = slow_sums<KERN, K>(sf, res, count, ts, c2, near, prm);
+    const PartialSums<K> r = slow_sums<KERN, K>(sf, res, count, ts, c, near, prm);
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = r.v[k];
   }
@@ -761,23 +868,20 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
   __syncthreads();
 
   if (warp == NCW) {
-    if (lane == 0) {
-      __shared__ float s_ibox[6];
-      Producer<Vec, kRes, STAGES> prod(v, sbuf, sres, smeta, full, empty, s_ibox);
-      prod.run();
-    }
+    Producer<Vec, kRes, STAGES> prod(v, sbuf, sres, smeta, full, empty, lane);
+    prod.run();
     return;
   }
 
   const int ct = threadIdx.x;   // consumer thread 0..kConsumers-1
-  int cur = -1;
   int4 item = make_int4(0, 0, 0, 0);
   double X[K][3];               // FP64 targets (FP64 path)
   // FP32 split of this thread's targets (FP32 path), in shared memory
   constexpr int kSplit = F32 ? K * 3 * kConsumers : 1;
-  __shared__ __align__(16) f2_t s_th[kSplit], s_tl[kSplit];
-  const TargetSplit ts{s_th + ct, s_tl + ct, kConsumers};
-  double acc[K];
+  __shared__ __align__(16) f2_t s_hl[kSplit];
+  const TargetSplit ts{s_hl + ct, kConsumers};
+  double acc[K];                // the current segment's sums
+  __shared__ double s_tot[K * kConsumers];   // the item's finished segments (in shared memory: no register)
   bool warp_full = true;
   bool warp_active = true;
   float prm = 0.f;              // its FP32 parameter
@@ -786,15 +890,9 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
   for (uint32_t it = 0;; ++it) {
     const int s = (int)(it % STAGES);
     if (!mbar_wait(&full[s], (it / STAGES) & 1u, v.err)) return;
-    const int mi = smeta[s].item;
-    if (mi != cur) {
-      if (cur >= 0) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) store_output(v, item, k * kConsumers + ct, acc[k]);
-      }
-      if (mi < 0) return;
-      cur = mi;
-      item = v.items[mi];
+    if (smeta[s].item < 0) return;
+    if (smeta[s].flags & kTaskStart) {
+      item = v.items[smeta[s].item];
       const int pid = v.t_problem[item.x];
       prm = v.prob_prm[pid];
       kappa = v.prob_kappa[pid];
@@ -807,14 +905,14 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         acc[k] = 0.0;
+        s_tot[k * kConsumers + ct] = 0.0;
         target_coords(v, item, k * kConsumers + ct, X[k][0], X[k][1], X[k][2]);
         if (F32) {
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
             const float h = (float)X[k][d];
             const float l = (float)(X[k][d] - (double)h);
-            s_th[(3 * k + d) * kConsumers + ct] = f2_pack(h, h);
-            s_tl[(3 * k + d) * kConsumers + ct] = f2_pack(l, l);
+            s_hl[(3 * k + d) * kConsumers + ct] = f2_pack(h, l);
           }
         }
       }
@@ -824,13 +922,8 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
       // no real target in this warp's rows: nothing to evaluate
     } else if constexpr (F32) {
       f2_t x2[K][3];
-      const f2_t* c2 = smeta[s].c2;
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const f2_t c = c2[d];
-#pragma unroll
-        for (int k = 0; k < K; ++k) x2[k][d] = f2_add(f2_sub(ts.hi(k, d), c), ts.lo(k, d));
-      }
+      const float* c = smeta[s].c;
+      frame_targets<K>(ts, c, x2);
       const float4* ext = &smeta[s].ext;
       const unsigned gm = smeta[s].near;
       unsigned slot = 0;
@@ -840,11 +933,11 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
       }
       float a[K];
       if (KERN != kKernCoulombYukawa)
-        eval_chunk_f32<KERN, K>(sbuf[s], sres[s], count, x2, ts, c2, ext, slot, warp_full, prm, a);
+        eval_chunk_f32<KERN, K>(sbuf[s], sres[s], count, x2, ts, c, ext, slot, warp_full, prm, a);
       else if (yukawa)
-        eval_chunk_f32<BLDTT_YUKAWA, K>(sbuf[s], sres[s], count, x2, ts, c2, ext, slot, warp_full, prm, a);
+        eval_chunk_f32<BLDTT_YUKAWA, K>(sbuf[s], sres[s], count, x2, ts, c, ext, slot, warp_full, prm, a);
       else
-        eval_chunk_f32<BLDTT_COULOMB, K>(sbuf[s], sres[s], count, x2, ts, c2, ext, slot, warp_full, prm, a);
+        eval_chunk_f32<BLDTT_COULOMB, K>(sbuf[s], sres[s], count, x2, ts, c, ext, slot, warp_full, prm, a);
 #pragma unroll
       for (int k = 0; k < K; ++k) acc[k] += (double)a[k];
     } else {
@@ -857,6 +950,26 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
         eval_chunk_f64<BLDTT_COULOMB, K>(sbuf[s], count, X, kappa, a);
 #pragma unroll
       for (int k = 0; k < K; ++k) acc[k] += a[k];
+    }
+    // read again (volatile): kept from the top, the flags would hold a register through the packed loop
+    const unsigned flags = *static_cast<volatile unsigned*>(&smeta[s].flags);
+    if (flags & kSegEnd) {
+      const int slot = smeta[s].slot;
+      if (slot < 0 && !(flags & kTaskEnd)) {       // a whole item's segment: into its totals
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          s_tot[k * kConsumers + ct] += acc[k];
+          acc[k] = 0.0;
+        }
+      } else {
+        SegSums<K> a;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          a.v[k] = acc[k];
+          acc[k] = 0.0;
+        }
+        end_segment<NCW, K>(v, item, smeta[s].item, slot, smeta[s].seg, flags, a, s_tot);
+      }
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s]);
@@ -927,6 +1040,10 @@ int interaction_grids(bldtt_plan* p) {
   for (auto& seg : p->segments) {
     int per_sm = 0;
     seg.threads = layout_threads(seg.layout);
+    // all of the SM's 228 KB as shared memory: at the default carveout five of the six CTAs fit
+    BL_CUDA(cudaFuncSetAttribute(select_kernel(seg.kernel, f32, seg.layout),
+                                 cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxShared));
     BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
         &per_sm, select_kernel(seg.kernel, f32, seg.layout), seg.threads, 0));
     if (per_sm < 1) per_sm = 1;
@@ -942,6 +1059,9 @@ static InteractView make_view(const bldtt_plan* p) {
   const Tree& st = p->st;
   InteractView v;
   v.items = p->items;
+  v.parts = p->parts;
+  v.seg_sums = p->seg_sums;
+  v.arrived = p->item_counter + kMaxSegmentsLaunch;
   v.nitems = p->nitems;
   v.counter = p->item_counter;
   v.list_ptr = p->list_ptr;
@@ -977,6 +1097,7 @@ static int launch_segment(const bldtt_plan* p, const InteractView& base, int g, 
   const auto& seg = p->segments[g];
   InteractView v = base;
   v.items = p->items + seg.first;
+  v.parts = p->parts + seg.first;
   v.nitems = seg.count;
   v.counter = p->item_counter + g;
   if (v.item_box) v.item_box = p->item_box + (int64_t)seg.first * (2 * kItemGroups);
@@ -996,7 +1117,7 @@ int run_segment(bldtt_plan* p, int g, cudaStream_t s) {
 int run_interactions(bldtt_plan* p, cudaStream_t s) {
   if (p->nitems == 0 || p->segments.empty()) return BLDTT_OK;
   const InteractView v = make_view(p);
-  BL_CUDA(cudaMemsetAsync(p->item_counter, 0, p->segments.size() * sizeof(int32_t), s));
+  BL_CUDA(cudaMemsetAsync(p->item_counter, 0, p->counter_words * sizeof(int32_t), s));
   for (int g = 0; g < (int)p->segments.size(); ++g) {
     BL_TRY(launch_segment(p, v, g, s));
     BL_LAUNCHED(p->compute_counter.launches);

@@ -34,6 +34,8 @@ constexpr int kChunk = 256;                    // sources per staged chunk (one 
 constexpr int kTile = 256;                     // targets per work item of the interaction kernel
 constexpr int kChunkInfo = 2;                  // float4 per pool chunk description
 constexpr int kItemGroups = kTile / 32;        // 32-row target groups per work item
+constexpr int kMaxSegments = 16;               // segments of a work item's chunks (see plan_parts)
+constexpr int kMaxSegmentsLaunch = 8;          // persistent launches (kernel groups) of a plan
 constexpr int kMaxDegrees = 8;                 // interpolation degrees of one plan
 // Segment kernel id of a persistent launch that drains the Coulomb and the
 // Yukawa problems of a batch together (the kernel is chosen per work item).
@@ -111,6 +113,27 @@ __device__ __forceinline__ void split_f64(double v, float& hi, float& lo) {
 // Work-item kinds: particle targets, or the proxy points of degree index
 // (kind - kItemProxies) of a target cluster.
 enum ItemKind { kItemParticles = 0, kItemProxies = 1 };
+
+// Division of a work item's `chunks` source chunks.  The item's sums are added
+// per segment of `len` consecutive chunks (at most kMaxSegments segments; the
+// segmentation depends on the item alone), and the segments' sums in order, so
+// that an item's result does not depend on how its segments are shared out as
+// tasks: `parts` tasks of `per` segments each (the last may be shorter), at
+// most about part_len chunks a task.
+struct PartPlan {
+  int32_t len, nseg, per, parts;
+};
+__host__ __device__ inline PartPlan plan_parts(int64_t chunks, int64_t part_len) {
+  PartPlan q;
+  const int64_t len = (chunks + kMaxSegments - 1) / kMaxSegments;
+  q.len = (int32_t)(len > 0 ? len : 1);
+  q.nseg = (int32_t)((chunks + q.len - 1) / q.len);
+  const int64_t want = part_len / q.len > 1 ? part_len / q.len : 1;      // segments per task at most
+  const int32_t parts = (int32_t)((q.nseg + want - 1) / want);
+  q.per = parts > 0 ? (q.nseg + parts - 1) / parts : 1;
+  q.parts = q.per > 0 ? (q.nseg + q.per - 1) / q.per : 0;
+  return q;
+}
 
 // Error flag codes written by kernels into plan->dev_err.
 enum DevErr { kDevErrNone = 0, kDevErrTimeout = 1, kDevErrBounds = 2 };
@@ -332,8 +355,13 @@ struct bldtt_plan {
 
   // Work items of the interaction kernel, sorted by decreasing cost.
   int4* items = nullptr;              // {cluster, row_begin, row_count, kind}
-  int32_t nitems = 0;
-  int32_t* item_counter = nullptr;    // one per segment
+  int4* parts = nullptr;              // task i: {first chunk, chunks, split slot or -1, nseg | len << 8}
+  int32_t nitems = 0;                 // tasks: the tiles, long ones split over their sources (plan_parts)
+  int32_t nsplit = 0;                 // split tiles
+  double* seg_sums = nullptr;         // [nsplit][kMaxSegments][kTile] segment sums of the split tiles
+  // [kMaxSegmentsLaunch] next task of each segment, then [nsplit][kItemGroups] finished segments
+  int32_t* item_counter = nullptr;
+  size_t counter_words = 0;
   double executed_evaluations = 0.0;
   // Evaluations the interaction kernel performs with and without idle warps
   // skipping their work (rows of 32-target groups holding no real target).
@@ -367,6 +395,7 @@ struct bldtt_plan {
   double sh_evals = 0.0;              // evaluations of the cached shard's items
   double computed_evals = 0.0;        // evaluations of the last compute's items
   int4* sh_items = nullptr;
+  int4* sh_parts = nullptr;
   float4* sh_item_box = nullptr;
   int32_t sh_nitems = 0;
   std::vector<Segment> sh_segments;

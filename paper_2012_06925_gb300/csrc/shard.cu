@@ -54,17 +54,19 @@ __global__ void k_shard_flags(int32_t nitems, const int4* __restrict__ items,
   flag[i] = keep ? 1 : 0;
 }
 
-__global__ void k_shard_gather(int32_t nitems, const int4* __restrict__ items,
+__global__ void k_shard_gather(int32_t nitems, const int4* __restrict__ items, const int4* __restrict__ parts,
                                const float4* __restrict__ box, const int32_t* __restrict__ flag,
                                const int32_t* __restrict__ pos, int4* __restrict__ out_items,
+                               int4* __restrict__ out_parts,
                                float4* __restrict__ out_box) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t i = t / (2 * kItemGroups + 1);
   const int r = (int)(t % (2 * kItemGroups + 1));
   if (i >= nitems || !flag[i]) return;
-  if (r == 2 * kItemGroups)
+  if (r == 2 * kItemGroups) {
     out_items[pos[i]] = items[i];
-  else if (box)
+    out_parts[pos[i]] = parts[i];
+  } else if (box)
     out_box[(int64_t)pos[i] * 2 * kItemGroups + r] = box[i * 2 * kItemGroups + r];
 }
 
@@ -106,6 +108,7 @@ static int shard_items(bldtt_plan* p, int shard, cudaStream_t s) {
   if (p->shard_cached == shard) return BLDTT_OK;
   const int32_t lo = p->shard_begin[shard], hi = p->shard_begin[shard + 1];
   dfree_ptr(p->sh_items, s);
+  dfree_ptr(p->sh_parts, s);
   dfree_ptr(p->sh_item_box, s);
   p->sh_nitems = 0;
   p->sh_segments.clear();
@@ -124,10 +127,11 @@ static int shard_items(bldtt_plan* p, int shard, cudaStream_t s) {
     const int32_t kept = h_pos[ni];
     if (kept > 0) {
       BL_TRY(dalloc_n(&p->sh_items, kept, s));
+      BL_TRY(dalloc_n(&p->sh_parts, kept, s));
       if (p->item_box) BL_TRY(dalloc_n(&p->sh_item_box, (size_t)kept * 2 * kItemGroups, s));
       const int64_t threads = (int64_t)ni * (2 * kItemGroups + 1);
-      k_shard_gather<<<nblk(threads, 256), 256, 0, s>>>(ni, p->items, p->item_box, flag, pos, p->sh_items,
-                                                        p->sh_item_box);
+      k_shard_gather<<<nblk(threads, 256), 256, 0, s>>>(ni, p->items, p->parts, p->item_box, flag, pos,
+                                                        p->sh_items, p->sh_parts, p->sh_item_box);
       BL_LAUNCHED(p->compute_counter.launches);
     }
     for (const auto& seg : p->segments) {
@@ -159,19 +163,21 @@ static int shard_items(bldtt_plan* p, int shard, cudaStream_t s) {
 // The plan's full work set, swapped for one shard's during a compute.
 struct WorkSwap {
   bldtt_plan* p;
-  int4* items;
+  int4 *items, *parts;
   float4* box;
   int32_t nitems;
   std::vector<bldtt_plan::Segment> segments;
-  explicit WorkSwap(bldtt_plan* plan) : p(plan), items(plan->items), box(plan->item_box),
+  explicit WorkSwap(bldtt_plan* plan) : p(plan), items(plan->items), parts(plan->parts), box(plan->item_box),
                                         nitems(plan->nitems), segments(plan->segments) {
     p->items = p->sh_items;
+    p->parts = p->sh_parts;
     p->item_box = p->sh_item_box;
     p->nitems = p->sh_nitems;
     p->segments = p->sh_segments;
   }
   ~WorkSwap() {
     p->items = items;
+    p->parts = parts;
     p->item_box = box;
     p->nitems = nitems;
     p->segments = segments;
