@@ -91,7 +91,7 @@ struct InteractView {
   int* err;
   // per-problem kernel parameters (read once per work item)
   const int32_t* t_problem;    // target cluster -> problem
-  const float* prob_prm;       // FP32 kernel parameter (see pair_f32)
+  const float* prob_prm;       // FP32 kernel parameter (fp32_parameter)
   const double* prob_kappa;
   const int* prob_kernel;      // kernel of each problem (read per item by the fused launch)
 };
@@ -222,27 +222,13 @@ __device__ __forceinline__ T poly_kernel(T dx, T dy, T dz) {
 }
 
 // Kernels that need an explicit r = 0 guard on every pair (finite at r = 0, or
-// the test kernel); they take the scalar path in FP32.
+// the test kernel, which takes the scalar path in FP32).
 template <int KERN>
 struct AlwaysGuarded {
   static constexpr bool value = KERN == BLDTT_OSCILLATORY || KERN == BLDTT_REG_COULOMB ||
                                 KERN == BLDTT_TEST_POLY;
 };
 
-// q * G in FP32; GUARD makes a pair at r^2 == 0 contribute 0.  prm is the
-// kernel parameter in the form the kernel uses (Yukawa: -kappa*log2(e);
-// oscillatory: kappa; regularized Coulomb: kappa^2).
-template <int KERN, bool GUARD>
-__device__ __forceinline__ float pair_f32(float dx, float dy, float dz, float q, float prm) {
-  float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-  if (KERN == BLDTT_TEST_POLY) return r2 > 0.f ? q * poly_kernel<float>(dx, dy, dz) : 0.f;
-  if ((GUARD || AlwaysGuarded<KERN>::value) && !(r2 > 0.f)) return 0.f;
-  if (KERN == BLDTT_REG_COULOMB) return q * rsqrt_approx(r2 + prm);
-  float ri = rsqrt_approx(r2);
-  if (KERN == BLDTT_COULOMB) return q * ri;
-  if (KERN == BLDTT_OSCILLATORY) return (q * ri) * sinf(prm * (r2 * ri));
-  return (q * ri) * exp2_approx(r2 * ri * prm);
-}
 template <int KERN, bool GUARD>
 __device__ __forceinline__ double pair_f64(double dx, double dy, double dz, double q, double kappa) {
   double r2 = dx * dx + dy * dy + dz * dz;
@@ -448,18 +434,63 @@ struct Producer {
 };
 
 // ---- consumers --------------------------------------------------------------
-// Packed evaluation of target k against the source pair (s0, s1):
-// acc += (q0 G(x - s0), q1 G(x - s1)).
+// sin(pi k r) of two values: k r = n + f with n the nearest integer, sin =
+// (-1)^n f P(f^2) with P the degree-4 minimax polynomial of sin(pi f)/f on
+// |f| <= 1/2 (absolute error 7.6e-9 with these float coefficients, found one
+// after the other so that each absorbs the rounding of those before it).  n comes from
+// adding 1.5 * 2^23 (its parity is the sum's last bit; rint and the conversion
+// to int run on the MUFU's pipe, which the rsqrts fill), and the fraction from
+// one fused multiply-add, so it carries the rounding of r and of k only, as an
+// argument k r rounded to float would.  For arguments beyond 2^22 the phase is
+// noise in float; the clamp keeps |sin| <= 1.
+__device__ __forceinline__ f2_t sinpi2(f2_t r, f2_t k) {
+  const f2_t big = f2_pack(12582912.f, 12582912.f);
+  const f2_t t = f2_fma(r, k, big);
+  float f0, f1, t0, t1, p0, p1;
+  f2_unpack(f2_fma(r, k, f2_sub(big, t)), f0, f1);
+  f2_unpack(t, t0, t1);
+  const f2_t f = f2_pack(fminf(fmaxf(f0, -0.5f), 0.5f), fminf(fmaxf(f1, -0.5f), 0.5f));
+  const f2_t s = f2_mul(f, f);
+  f2_t p = f2_fma(s, f2_pack(0.07643287628889084f, 0.07643287628889084f),
+                  f2_pack(-0.597625195980072f, -0.597625195980072f));
+  p = f2_fma(p, s, f2_pack(2.549957752227783f, 2.549957752227783f));
+  p = f2_fma(p, s, f2_pack(-5.1677021980285645f, -5.1677021980285645f));
+  p = f2_fma(p, s, f2_pack(3.141592502593994f, 3.141592502593994f));
+  f2_unpack(f2_mul(p, f), p0, p1);
+  return f2_pack(__uint_as_float(__float_as_uint(p0) ^ (__float_as_uint(t0) << 31)),
+                 __uint_as_float(__float_as_uint(p1) ^ (__float_as_uint(t1) << 31)));
+}
+
+// Packed evaluation of target k against the source pair (s0, s1) at
+// differences d: acc += (q0 G(x - s0), q1 G(x - s1)).  prm2 is the kernel
+// parameter as fp32_parameter gives it, duplicated.  The oscillatory and
+// regularized kernels stay finite at r = 0 and select the pair away here (r^2
+// replaced by 1, the charge by 0); Coulomb and Yukawa leave a non-finite sum,
+// which the chunk's caller redoes.  The scalar guarded loop that the former two
+// used to take for every pair (four shared-memory loads and a branch per
+// evaluation, sinf) ran at 0.67 and 2.6 evaluations per clock and SM against
+// 12.4 of the packed Coulomb loop.
 template <int KERN>
-__device__ __forceinline__ f2_t pair2_eval(f2_t dx, f2_t dy, f2_t dz, f2_t q2, f2_t acc, f2_t nk2) {
-  const f2_t r2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
+__device__ __forceinline__ f2_t pair2_eval(f2_t dx, f2_t dy, f2_t dz, f2_t q2, f2_t acc, f2_t prm2) {
+  f2_t r2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
   float r0, r1;
   f2_unpack(r2, r0, r1);
+  if (AlwaysGuarded<KERN>::value) {
+    float q0, q1;
+    f2_unpack(q2, q0, q1);
+    q2 = f2_pack(r0 > 0.f ? q0 : 0.f, r1 > 0.f ? q1 : 0.f);
+    r0 = r0 > 0.f ? r0 : 1.f;
+    r1 = r1 > 0.f ? r1 : 1.f;
+    r2 = f2_pack(r0, r1);
+    if (KERN == BLDTT_REG_COULOMB) f2_unpack(f2_add(r2, prm2), r0, r1);
+  }
   const f2_t ri = f2_pack(rsqrt_approx(r0), rsqrt_approx(r1));
-  if (KERN == BLDTT_COULOMB) return f2_fma(q2, ri, acc);
-  // Yukawa: q ri exp2(-kappa log2(e) r), r = r2 ri
+  if (KERN == BLDTT_COULOMB || KERN == BLDTT_REG_COULOMB) return f2_fma(q2, ri, acc);
+  const f2_t r = f2_mul(r2, ri);
+  if (KERN == BLDTT_OSCILLATORY) return f2_fma(f2_mul(q2, ri), sinpi2(r, prm2), acc);
+  // Yukawa: q ri exp2(-kappa log2(e) r)
   float e0, e1;
-  f2_unpack(f2_mul(f2_mul(r2, ri), nk2), e0, e1);
+  f2_unpack(f2_mul(r, prm2), e0, e1);
   return f2_fma(f2_mul(q2, ri), f2_pack(exp2_approx(e0), exp2_approx(e1)), acc);
 }
 template <int KERN>
@@ -568,19 +599,17 @@ __device__ __forceinline__ void chunk_f32_careful(const ulonglong2* __restrict__
   }
 }
 
-// One pair in the fast path's scalar arithmetic (the packed path computes
-// exactly this per lane), with the r = 0 guard: acc + q G(d).
+// One pair in the packed path's arithmetic (bit for bit per lane), with the
+// r = 0 guard: acc + q G(d).  Coulomb, Yukawa and the test kernel.
 template <int KERN>
 __device__ __forceinline__ float pair_acc_f32(float dx, float dy, float dz, float q, float prm,
                                               float acc) {
   const float r2 = fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx)));
   if (!(r2 > 0.f)) return acc;
+  if (KERN == BLDTT_TEST_POLY) return __fadd_rn(acc, q * poly_kernel<float>(dx, dy, dz));
   if (KERN == BLDTT_COULOMB) return fmaf(q, rsqrt_approx(r2), acc);
-  if (KERN == BLDTT_YUKAWA) {
-    const float ri = rsqrt_approx(r2);
-    return fmaf(__fmul_rn(q, ri), exp2_approx(__fmul_rn(__fmul_rn(r2, ri), prm)), acc);
-  }
-  return __fadd_rn(acc, pair_f32<KERN, true>(dx, dy, dz, q, prm));
+  const float ri = rsqrt_approx(r2);
+  return fmaf(__fmul_rn(q, ri), exp2_approx(__fmul_rn(__fmul_rn(r2, ri), prm)), acc);
 }
 
 // Scalar evaluation of a staged chunk: the same two partial sums (even and
@@ -795,8 +824,8 @@ __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rb
     }
     any_near = __any_sync(0xffffffffu, near != 0);
   }
-  if (AlwaysGuarded<KERN>::value) {
-    chunk_f32_slow<KERN, K>(sf, res, count, xs, ts, c, near, prm, a);
+  if (KERN == BLDTT_TEST_POLY) {
+    chunk_f32_slow<BLDTT_TEST_POLY, K>(sf, res, count, xs, ts, c, near, prm, a);
     return;
   }
   const ulonglong2* sb = reinterpret_cast<const ulonglong2*>(buf);
@@ -814,6 +843,7 @@ __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rb
   } else {
     chunk_f32<KERN, K>(sb, (count + 1) / 2, x2, a, prm);
   }
+  if (AlwaysGuarded<KERN>::value) return;
   bool bad = false;
 #pragma unroll
   for (int k = 0; k < K; ++k) bad = bad || not_finite(a[k]);
