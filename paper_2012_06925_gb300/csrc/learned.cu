@@ -151,13 +151,6 @@ __device__ void load_net(const __nv_bfloat16* gw, const float* gb, int nout, __n
   __syncthreads();
 }
 
-__host__ __device__ inline size_t net_smem_bytes(int nout) {
-  size_t w = (size_t)sel_weight_count(nout) * sizeof(__nv_bfloat16);
-  w = (w + 15) / 16 * 16;
-  return w + (size_t)sel_bias_count(nout) * sizeof(float) +
-         (size_t)kSelWarps * (2 * kHidden + 8 + 32) * sizeof(float);
-}
-
 // ---- selection inside the traversal -----------------------------------------
 struct SelParams {
   int nout, ndeg;
@@ -280,112 +273,244 @@ int select_pairs(bldtt_plan* p, const int2* pairs, int32_t F, int16_t* choice, c
 }
 
 // ---- training ------------------------------------------------------------------
-__global__ void k_to_bf16(const float* __restrict__ params, ParamLayout L, int nout,
-                          __nv_bfloat16* __restrict__ w, float* __restrict__ b) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t in[4] = {kFeatures, kHidden, kHidden, kHidden};
-  const int64_t out[4] = {kHidden, kHidden, kHidden, nout};
-  int64_t wo = 0, bo = 0;
+// The master parameters of one layer into shared memory as bf16: Wt[k][j] (the
+// forward pass: a warp's lanes read neighbouring neurons) and, if Wr is given,
+// Wr[j][k] (the backward pass: neighbouring inputs).
+__device__ void load_params(const float* __restrict__ params, const ParamLayout& L, int nout, __nv_bfloat16* wt,
+                            __nv_bfloat16* wr, float* sb) {
+  const int K[4] = {kFeatures, kHidden, kHidden, kHidden};
+  const int J[4] = {kHidden, kHidden, kHidden, nout};
+  int o = 0, ob = 0;
   for (int l = 0; l < 4; ++l) {
-    const int64_t nw = in[l] * out[l];
-    if (i < nw) w[wo + i] = __float2bfloat16_rn(params[L.w[l] + i]);
-    if (i < out[l]) b[bo + i] = params[L.b[l] + i];
-    wo += nw;
-    bo += out[l];
+    const int n = K[l] * J[l];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const __nv_bfloat16 v = __float2bfloat16_rn(params[L.w[l] + i]);
+      wt[o + (i % K[l]) * J[l] + i / K[l]] = v;
+      if (wr) wr[o + i] = v;
+    }
+    for (int i = threadIdx.x; i < J[l]; i += blockDim.x) sb[ob + i] = params[L.b[l] + i];
+    o += n;
+    ob += J[l];
   }
 }
 
-// Forward of a batch, keeping what the backward pass needs:
-// keep[b] = [x(8) | z1 a1 z2 a2 z3 a3 (6 x 64)], y[b][nout].
+__host__ __device__ inline size_t train_weight_bytes(int nout) {
+  return ((size_t)sel_weight_count(nout) * sizeof(__nv_bfloat16) + 15) / 16 * 16;
+}
+// Per-warp scratch of the training kernels: two activation or gradient rows and the inputs.
+constexpr int kTrainWarpFloats = 2 * kHidden + 8;
+__host__ __device__ inline size_t train_smem_bytes(int nout, bool backward) {
+  return train_weight_bytes(nout) * (backward ? 2 : 1) + (size_t)sel_bias_count(nout) * sizeof(float) +
+         (size_t)kSelWarps * kTrainWarpFloats * sizeof(float);
+}
+
+// What a sample's backward pass and the weight gradients read: [x(8) | z1 a1 z2
+// a2 z3 a3 (6 x 64)] and [dL/dy (24) | dL/dz3, dL/dz2, dL/dz1 (3 x 64)].
 constexpr int kKeep = 8 + 6 * kHidden;
-__global__ void k_mlp_forward(const float* __restrict__ xin, int64_t B, const __nv_bfloat16* __restrict__ gw,
-                              const float* __restrict__ gb, int nout, float* __restrict__ y,
-                              float* __restrict__ keep) {
+constexpr int kGradOut = 24;
+constexpr int kGradRow = kGradOut + 3 * kHidden;
+
+__global__ void k_mlp_forward(const float* __restrict__ xin, int64_t B, const float* __restrict__ params,
+                              ParamLayout L, int nout, float* __restrict__ y) {
   extern __shared__ __align__(16) unsigned char sraw[];
   __nv_bfloat16* sw = reinterpret_cast<__nv_bfloat16*>(sraw);
-  size_t wbytes = ((size_t)sel_weight_count(nout) * sizeof(__nv_bfloat16) + 15) / 16 * 16;
-  float* sb = reinterpret_cast<float*>(sraw + wbytes);
+  float* sb = reinterpret_cast<float*>(sraw + train_weight_bytes(nout));
   float* swarp = sb + sel_bias_count(nout);
-  load_net(gw, gb, nout, sw, sb);
+  load_params(params, L, nout, sw, nullptr, sb);
+  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* act = swarp + warp * (2 * kHidden + 8 + 32);
+  float* act = swarp + warp * kTrainWarpFloats;
   float* x = act + 2 * kHidden;
   const NetSmem net{sw, sb, nout};
   for (int64_t i = (int64_t)blockIdx.x * kSelWarps + warp; i < B; i += (int64_t)gridDim.x * kSelWarps) {
     if (lane < kFeatures) x[lane] = bf16r(xin[i * kFeatures + lane]);
     __syncwarp();
-    float* kp = keep ? keep + i * kKeep : nullptr;
-    if (kp && lane < kFeatures) kp[lane] = x[lane];
-    const float v = mlp_forward_warp(net, x, act, kp ? kp + 8 : nullptr);
+    const float v = mlp_forward_warp(net, x, act, nullptr);
     if (lane < nout) y[i * nout + lane] = v;
     __syncwarp();
   }
 }
 
-// Deterministic block sums: out[0] = sum mask, out[1] = sum (mask (y - T))^2.
-__global__ void k_loss_sums(const float* __restrict__ y, const float* __restrict__ T,
-                            const float* __restrict__ mask, int64_t n, float* __restrict__ out) {
-  __shared__ double s0[256], s1[256];
-  double a = 0.0, b = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-    const double d = (double)mask[i] * ((double)y[i] - (double)T[i]);
-    a += mask[i];
-    b += d * d;
-  }
-  s0[threadIdx.x] = a;
-  s1[threadIdx.x] = b;
+// Forward and backward pass of every sample, one warp each, in one launch (the
+// layers used to be a launch each: conversion, forward, loss, output gradient
+// and three backward steps).  The output gradient is left undivided by the mask
+// count, dL/dy cnt = 2 mask (y - T), because the count is known only after all
+// samples; the weight gradients divide their sums.  Backward through a layer:
+// gz[k] = (sum_j g[j] W[j][k]) [z[k] > 0], j in increasing order.  part[block] =
+// (sum mask, sum (mask (y - T))^2) of the block's samples.
+__global__ void __launch_bounds__(32 * kSelWarps) k_train_samples(
+    const float* __restrict__ xin, const float* __restrict__ T, const float* __restrict__ mask, int64_t B,
+    const float* __restrict__ params, ParamLayout L, int nout, float* __restrict__ keep,
+    float* __restrict__ grad, double2* __restrict__ part) {
+  extern __shared__ __align__(16) unsigned char sraw[];
+  __shared__ double2 sred[kSelWarps];
+  const size_t wbytes = train_weight_bytes(nout);
+  __nv_bfloat16* wt = reinterpret_cast<__nv_bfloat16*>(sraw);
+  __nv_bfloat16* wr = reinterpret_cast<__nv_bfloat16*>(sraw + wbytes);
+  float* sb = reinterpret_cast<float*>(sraw + 2 * wbytes);
+  float* swarp = sb + sel_bias_count(nout);
+  load_params(params, L, nout, wt, wr, sb);
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      s0[threadIdx.x] += s0[threadIdx.x + w];
-      s1[threadIdx.x] += s1[threadIdx.x + w];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* act = swarp + warp * kTrainWarpFloats;
+  float* x = act + 2 * kHidden;
+  const NetSmem net{wt, sb, nout};
+  double sm = 0.0, sl = 0.0;
+  for (int64_t i = (int64_t)blockIdx.x * kSelWarps + warp; i < B; i += (int64_t)gridDim.x * kSelWarps) {
+    float* kp = keep + i * kKeep;
+    float* gr = grad + i * kGradRow;
+    if (lane < kFeatures) {
+      x[lane] = bf16r(xin[i * kFeatures + lane]);
+      kp[lane] = x[lane];
+    }
+    __syncwarp();
+    const float y = mlp_forward_warp(net, x, act, kp + 8);
+    float* g = act;                            // dL/dy, then the hidden layers' dL/dz, alternating
+    float* gn = act + kHidden;
+    __syncwarp();
+    if (lane < nout) {
+      const float mk = mask[i * nout + lane], t = T[i * nout + lane];
+      const float v = 2.f * mk * (y - t);
+      g[lane] = v;
+      gr[lane] = v;
+      const double d = (double)mk * ((double)y - (double)t);
+      sm += mk;
+      sl += d * d;
+    }
+    __syncwarp();
+    const __nv_bfloat16* W = wr + kHidden * kFeatures + 2 * kHidden * kHidden;   // the output layer's
+    for (int l = 3; l >= 1; --l) {
+      const int J = l == 3 ? nout : kHidden;
+      float v[2];
+      for (int h = 0; h < 2; ++h) {
+        const int k = lane + 32 * h;
+        float a = 0.f;
+        for (int j = 0; j < J; ++j) a = fmaf(g[j], __bfloat162float(W[j * kHidden + k]), a);
+        // this thread wrote its own pre-activations z[k] of layer l
+        v[h] = kp[8 + 2 * (l - 1) * kHidden + k] > 0.f ? a : 0.f;
+      }
+      for (int h = 0; h < 2; ++h) {
+        gn[lane + 32 * h] = v[h];
+        gr[kGradOut + (3 - l) * kHidden + lane + 32 * h] = v[h];
+      }
+      __syncwarp();
+      float* tmp = g;
+      g = gn;
+      gn = tmp;
+      W -= kHidden * kHidden;
+    }
+  }
+  for (int o = 16; o; o >>= 1) {
+    sm += __shfl_xor_sync(0xffffffffu, sm, o);
+    sl += __shfl_xor_sync(0xffffffffu, sl, o);
+  }
+  if (lane == 0) sred[warp] = make_double2(sm, sl);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double2 v = sred[0];
+    for (int w = 1; w < kSelWarps; ++w) {
+      v.x += sred[w].x;
+      v.y += sred[w].y;
+    }
+    part[blockIdx.x] = v;
+  }
+}
+
+// Weight and bias gradients of all layers in one launch: dW[j][k] = sum_b
+// g[b][j] a[b][k] / cnt, db[j] = sum_b g[b][j] / cnt, each sum sequential over
+// the batch in float.  A block takes kGradJ neurons of one layer, a thread one
+// input k of them (thread 64: the biases), so a sample's activation is read
+// once for kGradJ products; kGradB samples at a time come through shared memory
+// (one thread per weight reading both factors from memory took 4 x ~100 us at
+// 1024 samples, the latency of 1024 dependent steps).
+constexpr int kGradJ = 4;
+constexpr int kGradB = 64;
+constexpr int kGradThreads = 96;
+__global__ void __launch_bounds__(kGradThreads) k_weight_grads(const float* __restrict__ keep,
+                                                              const float* __restrict__ grad, int64_t B,
+                                                              ParamLayout L, int nout,
+                                                              const double2* __restrict__ part, int nparts,
+                                                              float* __restrict__ out, float* __restrict__ loss) {
+  __shared__ __align__(16) float sa[2][kGradB][kHidden];
+  __shared__ __align__(16) float sg[2][kGradB][kGradJ];
+  __shared__ float scnt;
+  const int per = kHidden / kGradJ;             // blocks per hidden layer
+  const int l = blockIdx.x / per < 3 ? blockIdx.x / per : 3;
+  const int j0 = (blockIdx.x - l * per) * kGradJ;
+  const int J = l == 3 ? nout : kHidden, K = l == 0 ? kFeatures : kHidden;
+  const int aoff = l == 0 ? 0 : 8 + (2 * l - 1) * kHidden;               // x, a1, a2, a3
+  const int goff = l == 3 ? 0 : kGradOut + (2 - l) * kHidden;            // dL/dy, dL/dz3, dL/dz2, dL/dz1
+  const int tid = threadIdx.x;
+  if (tid < 32) {                               // the mask count and the loss, in block order
+    double m = 0.0, q = 0.0;
+    for (int i = tid; i < nparts; i += 32) {
+      m += part[i].x;
+      q += part[i].y;
+    }
+    for (int o = 16; o; o >>= 1) {
+      m += __shfl_xor_sync(0xffffffffu, m, o);
+      q += __shfl_xor_sync(0xffffffffu, q, o);
+    }
+    if (tid == 0) {
+      const double cnt = m > 1.0 ? m : 1.0;
+      scnt = (float)cnt;
+      if (blockIdx.x == 0 && loss) *loss = (float)(q / cnt);
+    }
+  }
+  auto stage = [&](int buf, int64_t base) {     // asynchronous copies of one set of samples
+    const int n = (int)min((int64_t)kGradB, B - base);
+    for (int i = tid; i < n * (kHidden / 4); i += kGradThreads) {
+      const int b = i / (kHidden / 4), k = (i % (kHidden / 4)) * 4;
+      if (k < (K + 3) / 4 * 4) {
+        const float* src = keep + (base + b) * kKeep + aoff + k;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(&sa[buf][b][k])),
+                     "l"(src));
+      }
+    }
+    for (int b = tid; b < n; b += kGradThreads) {
+      const float* src = grad + (base + b) * kGradRow + goff + j0;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(
+                       (uint32_t)__cvta_generic_to_shared(&sg[buf][b][0])),
+                   "l"(src));
+    }
+    asm volatile("cp.async.commit_group;");
+  };
+  float acc[kGradJ] = {0.f, 0.f, 0.f, 0.f};
+  const bool mine = tid < K || tid == kHidden;
+  stage(0, 0);
+  for (int64_t base = 0, it = 0; base < B; base += kGradB, ++it) {
+    const int buf = (int)(it & 1);
+    if (base + kGradB < B) {
+      stage(buf ^ 1, base + kGradB);
+      asm volatile("cp.async.wait_group 1;");
+    } else {
+      asm volatile("cp.async.wait_group 0;");
+    }
+    __syncthreads();
+    const int n = (int)min((int64_t)kGradB, B - base);
+    if (mine) {
+#pragma unroll 8
+      for (int b = 0; b < n; ++b) {
+        const float a = tid < kHidden ? sa[buf][b][tid] : 1.f;
+        const float4 g = *reinterpret_cast<const float4*>(sg[buf][b]);
+        acc[0] = fmaf(g.x, a, acc[0]);
+        acc[1] = fmaf(g.y, a, acc[1]);
+        acc[2] = fmaf(g.z, a, acc[2]);
+        acc[3] = fmaf(g.w, a, acc[3]);
+      }
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    const double cnt = s0[0] > 1.0 ? s0[0] : 1.0;
-    out[0] = (float)cnt;
-    out[1] = (float)(s1[0] / cnt);
+  if (!mine) return;
+  for (int r = 0; r < kGradJ; ++r) {
+    const int j = j0 + r;
+    if (j >= J) break;
+    if (tid < kHidden)
+      out[L.w[l] + (int64_t)j * K + tid] = acc[r] / scnt;
+    else
+      out[L.b[l] + j] = acc[r] / scnt;
   }
-}
-
-// dL/dy = 2 mask (y - T) / cnt.
-__global__ void k_out_grad(const float* __restrict__ y, const float* __restrict__ T,
-                           const float* __restrict__ mask, int64_t n, const float* __restrict__ sums,
-                           float* __restrict__ gy) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) gy[i] = 2.f * mask[i] * (y[i] - T[i]) / sums[0];
-}
-
-// dW[j][k] = sum_b g[b][j] a[b][k], db[j] = sum_b g[b][j] (sequential over b).
-// a rows: a_of(b) = base + b * stride + off.
-__global__ void k_weight_grad(const float* __restrict__ g, int gstride, int J, const float* __restrict__ a,
-                              int64_t astride, int aoff, int K, int64_t B, float* __restrict__ dW,
-                              float* __restrict__ db) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < (int64_t)J * K) {
-    const int j = (int)(t / K), k = (int)(t % K);
-    float acc = 0.f;
-    for (int64_t b = 0; b < B; ++b) acc = fmaf(g[b * gstride + j], a[b * astride + aoff + k], acc);
-    dW[t] = acc;
-  } else if (t < (int64_t)J * K + J) {
-    const int j = (int)(t - (int64_t)J * K);
-    float acc = 0.f;
-    for (int64_t b = 0; b < B; ++b) acc += g[b * gstride + j];
-    db[j] = acc;
-  }
-}
-
-// gz_prev[b][k] = (sum_j g[b][j] W[j][k]) [z_prev[b][k] > 0].
-__global__ void k_back(const float* __restrict__ g, int J, const __nv_bfloat16* __restrict__ W, int K,
-                       const float* __restrict__ keep, int zoff, int64_t B, float* __restrict__ gprev) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= B * K) return;
-  const int64_t b = t / K;
-  const int k = (int)(t % K);
-  float acc = 0.f;
-  for (int j = 0; j < J; ++j) acc = fmaf(g[b * J + j], __bfloat162float(W[(int64_t)j * K + k]), acc);
-  gprev[t] = keep[b * kKeep + zoff + k] > 0.f ? acc : 0.f;
 }
 
 __global__ void k_adam(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
@@ -615,21 +740,11 @@ int bldtt_mlp_forward(const float* params, int num_out, const float* x, int64_t 
     return BLDTT_EINVAL;
   }
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  const ParamLayout L(num_out);
-  __nv_bfloat16* w = nullptr;
-  float* b = nullptr;
-  BL_TRY(dalloc_n(&w, (size_t)sel_weight_count(num_out), s));
-  BL_TRY(dalloc_n(&b, (size_t)sel_bias_count(num_out), s));
-  k_to_bf16<<<nblk(kHidden * kHidden, 256), 256, 0, s>>>(params, L, num_out, w, b);
+  const size_t sm = train_smem_bytes(num_out, false);
+  k_mlp_forward<<<nblk(batch, kSelWarps) > 4096 ? 4096 : nblk(batch, kSelWarps), 32 * kSelWarps, sm, s>>>(
+      x, batch, params, ParamLayout(num_out), num_out, y);
   int64_t dummy = 0;
   BL_LAUNCHED(dummy);
-  const size_t sm = net_smem_bytes(num_out);
-  BL_CUDA(cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k_mlp_forward<<<nblk(batch, kSelWarps) > 4096 ? 4096 : nblk(batch, kSelWarps), 32 * kSelWarps, sm, s>>>(
-      x, batch, w, b, num_out, y, nullptr);
-  BL_LAUNCHED(dummy);
-  dfree(w, s);
-  dfree(b, s);
   return BLDTT_OK;
 }
 
@@ -642,59 +757,21 @@ int bldtt_mlp_gradients(const float* params, int num_out, const float* x, const 
   }
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const ParamLayout L(num_out);
-  __nv_bfloat16* w = nullptr;
-  float *b = nullptr, *y = nullptr, *keep = nullptr, *g1 = nullptr, *g2 = nullptr, *sums = nullptr;
-  BL_TRY(dalloc_n(&w, (size_t)sel_weight_count(num_out), s));
-  BL_TRY(dalloc_n(&b, (size_t)sel_bias_count(num_out), s));
-  BL_TRY(dalloc_n(&y, (size_t)batch * num_out, s));
-  BL_TRY(dalloc_n(&keep, (size_t)batch * kKeep, s));
-  BL_TRY(dalloc_n(&g1, (size_t)batch * kHidden, s));
-  BL_TRY(dalloc_n(&g2, (size_t)batch * kHidden, s));
-  BL_TRY(dalloc_n(&sums, 2, s));
+  const unsigned blocks = nblk(batch, kSelWarps) > 4096 ? 4096 : nblk(batch, kSelWarps);
+  float *keep = nullptr, *grad = nullptr;
+  double2* part = nullptr;
+  Arena scratch;                       // freed, in stream order, when it goes out of scope
+  scratch.add(&keep, (size_t)batch * kKeep);
+  scratch.add(&grad, (size_t)batch * kGradRow);
+  scratch.add(&part, blocks);
+  BL_TRY(scratch.alloc(s));
   int64_t dummy = 0;
-  k_to_bf16<<<nblk(kHidden * kHidden, 256), 256, 0, s>>>(params, L, num_out, w, b);
+  const size_t sm = train_smem_bytes(num_out, true);
+  k_train_samples<<<blocks, 32 * kSelWarps, sm, s>>>(x, target, mask, batch, params, L, num_out, keep, grad, part);
   BL_LAUNCHED(dummy);
-  const size_t sm = net_smem_bytes(num_out);
-  BL_CUDA(cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k_mlp_forward<<<nblk(batch, kSelWarps) > 4096 ? 4096 : nblk(batch, kSelWarps), 32 * kSelWarps, sm, s>>>(
-      x, batch, w, b, num_out, y, keep);
+  const unsigned jb = 3 * (kHidden / kGradJ) + nblk(num_out, kGradJ);
+  k_weight_grads<<<jb, kGradThreads, 0, s>>>(keep, grad, batch, L, num_out, part, (int)blocks, grads, loss);
   BL_LAUNCHED(dummy);
-  const int64_t ny = batch * num_out;
-  k_loss_sums<<<1, 256, 0, s>>>(y, target, mask, ny, sums);
-  BL_LAUNCHED(dummy);
-  // g1 <- dL/dy (batch x num_out, fits: num_out <= 24 < 64)
-  k_out_grad<<<nblk(ny, 256), 256, 0, s>>>(y, target, mask, ny, sums, g1);
-  BL_LAUNCHED(dummy);
-  // layer 4 (output): a3 at keep offset 8 + 5*64
-  const int aoff[4] = {0, 8 + 1 * kHidden, 8 + 3 * kHidden, 8 + 5 * kHidden};   // a0 = x, a1, a2, a3
-  const int zoff[3] = {8 + 0 * kHidden, 8 + 2 * kHidden, 8 + 4 * kHidden};      // z1, z2, z3
-  const int K[4] = {kFeatures, kHidden, kHidden, kHidden};
-  const int J[4] = {kHidden, kHidden, kHidden, num_out};
-  const __nv_bfloat16* Wl[4];
-  {
-    int64_t o = 0;
-    for (int l = 0; l < 4; ++l) {
-      Wl[l] = w + o;
-      o += (int64_t)K[l] * J[l];
-    }
-  }
-  float* g = g1;
-  float* gn = g2;
-  for (int l = 3; l >= 0; --l) {
-    const int64_t nt = (int64_t)J[l] * K[l] + J[l];
-    k_weight_grad<<<nblk(nt, 128), 128, 0, s>>>(g, J[l], J[l], keep, kKeep, aoff[l], K[l], batch,
-                                                 grads + L.w[l], grads + L.b[l]);
-    BL_LAUNCHED(dummy);
-    if (l > 0) {
-      k_back<<<nblk(batch * K[l], 256), 256, 0, s>>>(g, J[l], Wl[l], K[l], keep, zoff[l - 1], batch, gn);
-      BL_LAUNCHED(dummy);
-      float* tmp = g;
-      g = gn;
-      gn = tmp;
-    }
-  }
-  if (loss) BL_CUDA(cudaMemcpyAsync(loss, sums + 1, sizeof(float), cudaMemcpyDeviceToDevice, s));
-  dfree(w, s); dfree(b, s); dfree(y, s); dfree(keep, s); dfree(g1, s); dfree(g2, s); dfree(sums, s);
   return BLDTT_OK;
 }
 
