@@ -63,7 +63,9 @@ enum bldtt_kernel {
 
 /* Arithmetic of the kernel evaluations. */
 enum bldtt_precision {
-    BLDTT_FP64 = 0,       /* plain FP64 everywhere */
+    BLDTT_FP64 = 0,       /* FP64 results everywhere; the Coulomb, Yukawa and
+                             regularized kernels are evaluated in 64-bit fixed point,
+                             to within FP64's last rounding */
     BLDTT_FP32_BULK = 1   /* kernel evaluations and Lagrange contractions in FP32, in
                              coordinate frames local to each source cluster, summed in
                              FP64 every 256 sources; barycentric weights, the
