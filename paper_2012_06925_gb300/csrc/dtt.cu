@@ -842,8 +842,8 @@ __global__ void k_item_boxes(int32_t nitems, const int4* __restrict__ items, con
 // than the even load gives.  Measured (interaction kernel, GB300): 1E6 points
 // (1.9E6 tile-chunks) 31.9 ms at 4 tasks per CTA, 31.4 at 16-24, 31.3 at 50
 // with 0.2 ms more to list them; 2E4 points on a sphere (4800) 0.25 ms at 1-3
-// chunks, 0.18 at 4-6, 0.21 at 8, 0.45 whole; 2E4 points in FP64 9.6 ms at 1-3,
-// 9.9 at 8, 28 whole.  A plan of many short tiles (512 problems) is not split.
+// chunks, 0.18 at 4-6, 0.21 at 8, 0.45 whole; 2E4 points in FP64 2.2 ms at 1-2,
+// 2.3 at 3, 2.4 at 4.  A plan of many short tiles (512 problems) is not split.
 constexpr int kTasksPerCta = 16;
 static int64_t task_chunks(const bldtt_plan* p) {
   if (const char* e = std::getenv("BLDTT_TASK_CHUNKS"))   // testing: results do not depend on the split

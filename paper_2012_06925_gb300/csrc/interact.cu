@@ -235,8 +235,8 @@ struct Param64 {
 };
 // Coulomb, Yukawa and regularized run in fixed point: the FP64 pipe (1.7 lanes
 // per clock and SM) took 12 to 45 instructions per evaluation, now 4.  2E4
-// Coulomb particles: 9.6 -> 3.2 ms in this kernel (n 8, theta 0.7); 6E4 Yukawa:
-// 51 -> 9.5 ms.
+// Coulomb particles: 9.6 -> 3.2 ms in this kernel (n 4, theta 0.7, leaves of
+// 500); 6E4 Yukawa (n 7, theta 0.8, leaves of 1000): 51 -> 9.7 ms.
 template <int KERN>
 __device__ __forceinline__ double kernel_f64(double dx, double dy, double dz, const Param64& prm) {
   if (KERN == BLDTT_COULOMB) return fixed64::inv_r(dx, dy, dz);
@@ -680,6 +680,24 @@ __device__ __forceinline__ void chunk_f64(const double4* __restrict__ sb, int co
   }
 }
 
+// The same for the warp's real rows: its last target slot is left out where
+// none of its rows holds a target.  The FP64 pipe bounds this path, so an idle
+// row costs what a real one does: 2E4 Coulomb particles in leaves of 312 (a
+// full tile and one of 56 rows) 3.2 -> 2.2 ms.
+template <int KERN, int K>
+__device__ __forceinline__ void rows_f64(const double4* __restrict__ sb, int count, const double (&x)[K][3],
+                                         bool warp_full, double (&a)[K], const Param64& prm) {
+  if (K == 1 || warp_full) {
+    chunk_f64<KERN, K>(sb, count, x, a, prm);
+    return;
+  }
+  constexpr int K1 = K > 1 ? K - 1 : 1;
+  double a1[K1];
+  chunk_f64<KERN, K1>(sb, count, *reinterpret_cast<const double(*)[K1][3]>(&x), a1, prm);
+#pragma unroll
+  for (int k = 0; k < K; ++k) a[k] = k < K1 ? a1[k < K1 ? k : 0] : 0.0;
+}
+
 // Absolute coordinates of target row r of an item (a particle or a proxy point).
 __device__ __forceinline__ void target_coords(const InteractView& v, const int4& item, int r,
                                               double& X, double& Y, double& Z) {
@@ -928,8 +946,9 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
       // does any row of this warp's last target slot hold a real target?
       warp_full = (K - 1) * kConsumers + (warp * 32) < item.z;
       // does any row of its first slot?  (if not, the warp only keeps the ring
-      // going; layouts for plans with many small items skip such warps' work)
-      if (SKIP) warp_active = warp * 32 < item.z;
+      // going; FP64, and layouts for plans with many small items, skip such
+      // warps' work)
+      if (SKIP || !F32) warp_active = warp * 32 < item.z;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         acc[k] = 0.0;
@@ -946,7 +965,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
       }
     }
     const int count = smeta[s].count;
-    if (SKIP && !warp_active) {
+    if ((SKIP || !F32) && !warp_active) {
       // no real target in this warp's rows: nothing to evaluate
     } else if constexpr (F32) {
       f2_t x2[K][3];
@@ -971,11 +990,11 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
     } else {
       double a[K];
       if (KERN != kKernCoulombYukawa)
-        chunk_f64<KERN, K>(reinterpret_cast<const double4*>(sbuf[s]), count, X, a, prm64);
+        rows_f64<KERN, K>(reinterpret_cast<const double4*>(sbuf[s]), count, X, warp_full, a, prm64);
       else if (yukawa)
-        chunk_f64<BLDTT_YUKAWA, K>(reinterpret_cast<const double4*>(sbuf[s]), count, X, a, prm64);
+        rows_f64<BLDTT_YUKAWA, K>(reinterpret_cast<const double4*>(sbuf[s]), count, X, warp_full, a, prm64);
       else
-        chunk_f64<BLDTT_COULOMB, K>(reinterpret_cast<const double4*>(sbuf[s]), count, X, a, prm64);
+        rows_f64<BLDTT_COULOMB, K>(reinterpret_cast<const double4*>(sbuf[s]), count, X, warp_full, a, prm64);
 #pragma unroll
       for (int k = 0; k < K; ++k) acc[k] += a[k];
     }
@@ -1030,8 +1049,8 @@ static const void* kernel_for(int layout) {
   if constexpr (F32) {
     if (layout >= kLayoutSkip) return kernel_for_skip<F32, KERN, true>(layout - kLayoutSkip);
   }
-  // FP64: the skipping instances are not built (the FP64 path's cost is its
-  // arithmetic, not idle rows); a skipping layout runs its base layout.
+  // FP64 leaves idle rows out in every layout (rows_f64); a skipping layout is
+  // its base layout.
   return kernel_for_skip<F32, KERN, false>(layout % kLayoutSkip);
 }
 

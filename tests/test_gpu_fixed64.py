@@ -75,3 +75,19 @@ def test_plan_and_direct_sum_agree_to_rounding():
             phi = p.compute()
         ref = B.direct_sum(pts, pts, q, kernel, kappa)
         assert torch.max(torch.abs(phi / ref - 1)).item() <= 700 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("kernel,kappa", [(B.COULOMB, 0.0), (B.YUKAWA, 0.7), (B.OSCILLATORY, 2.0)])
+@pytest.mark.parametrize("m", [1, 31, 32, 33, 127, 128, 129, 160, 255, 256, 257, 300])
+def test_partial_target_tiles(m, kernel, kappa):
+    """Warps and target slots without a real row are left out; the rows that are there are not."""
+    rng = np.random.default_rng(m)
+    tgt = torch.from_numpy(rng.uniform(-1, 1, (3, m))).cuda()
+    src = torch.from_numpy(rng.uniform(-1, 1, (3, 300))).cuda()
+    q = torch.from_numpy(rng.uniform(0.5, 1.5, 300)).cuda()
+    with B.Plan(tgt, src, q, kernel=kernel, kappa=kappa, n=2, theta=0.0, N0=512, M0=512,
+                precision=B.FP64) as p:
+        phi = p.compute()
+    ref = B.direct_sum(tgt, src, q, kernel, kappa)
+    scale = B.direct_sum(tgt, src, q, B.COULOMB, 0.0)       # bounds the sum of |terms|
+    assert torch.max(torch.abs(phi - ref) / scale).item() <= 310 * 2.0 ** -53
