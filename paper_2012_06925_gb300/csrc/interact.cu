@@ -48,11 +48,12 @@
 // residuals; a flagged warp adds the residuals of both points to the
 // coordinate differences of its near targets (see eval_chunk_f32).
 //
-// A pair at distance 0 contributes nothing.  The fast path evaluates
-// 1/sqrt(r^2) unguarded; a chunk whose partial sum is not finite (only
-// possible when some r^2 == 0) is recomputed by the warp with the guard, in
-// the same arithmetic and order, so that a target's result never depends on
-// which warp or consumer layout evaluated it.
+// A pair at distance 0 contributes nothing.  Only a target near a chunk (or in
+// it) can meet one, so the guard stands in the careful path alone, for warps
+// with a target inside the chunk's box; the plain path evaluates unguarded, and
+// a sum that is not finite all the same (r^2 underflows) is redone with the
+// guard.  The arithmetic and the order are the same throughout, so a target's
+// result never depends on which warp or consumer layout evaluated it.
 #include <type_traits>
 
 #include "fixed64.cuh"
@@ -219,8 +220,9 @@ __device__ __forceinline__ T poly_kernel(T dx, T dy, T dz) {
          (T)0.5 * dy * dy;
 }
 
-// Kernels that need an explicit r = 0 guard on every pair (finite at r = 0, or
-// the test kernel, which takes the scalar path in FP32).
+// Kernels whose near chunks all take the guarded call: finite at r = 0, so that
+// a coincident pair would not show in the sum (and their loop is long: a second
+// copy of it beside the plain one spills registers).
 template <int KERN>
 struct AlwaysGuarded {
   static constexpr bool value = KERN == BLDTT_OSCILLATORY || KERN == BLDTT_REG_COULOMB ||
@@ -471,28 +473,22 @@ __device__ __forceinline__ f2_t sinpi2(f2_t r, f2_t k) {
 
 // Packed evaluation of target k against the source pair (s0, s1) at
 // differences d: acc += (q0 G(x - s0), q1 G(x - s1)).  prm2 is the kernel
-// parameter as fp32_parameter gives it, duplicated.  The oscillatory and
-// regularized kernels stay finite at r = 0 and select the pair away here (r^2
-// replaced by 1, the charge by 0); Coulomb and Yukawa leave a non-finite sum,
-// which the chunk's caller redoes.  The scalar guarded loop that the former two
-// used to take for every pair (four shared-memory loads and a branch per
-// evaluation, sinf) ran at 0.67 and 2.6 evaluations per clock and SM against
-// 12.4 of the packed Coulomb loop.
-template <int KERN>
+// parameter as fp32_parameter gives it, duplicated.  GUARD: a pair at r = 0 is
+// left out (two compares and two selects a pair of evaluations).  The scalar
+// guarded loop that the oscillatory and regularized kernels used to take for
+// every pair (four shared-memory loads and a branch per evaluation, sinf) ran
+// at 0.67 and 2.6 evaluations per clock and SM against 12.4 of the packed
+// Coulomb loop; packed with the guard on every pair 3.8 and 9.4, with the guard
+// in near chunks only 4.5 and 11.1.
+template <int KERN, bool GUARD = false>
 __device__ __forceinline__ f2_t pair2_eval(f2_t dx, f2_t dy, f2_t dz, f2_t q2, f2_t acc, f2_t prm2) {
   f2_t r2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
   float r0, r1;
   f2_unpack(r2, r0, r1);
-  if (AlwaysGuarded<KERN>::value) {
-    float q0, q1;
-    f2_unpack(q2, q0, q1);
-    q2 = f2_pack(r0 > 0.f ? q0 : 0.f, r1 > 0.f ? q1 : 0.f);
-    r0 = r0 > 0.f ? r0 : 1.f;
-    r1 = r1 > 0.f ? r1 : 1.f;
-    r2 = f2_pack(r0, r1);
-    if (KERN == BLDTT_REG_COULOMB) f2_unpack(f2_add(r2, prm2), r0, r1);
-  }
-  const f2_t ri = f2_pack(rsqrt_approx(r0), rsqrt_approx(r1));
+  const bool k0 = !GUARD || r0 > 0.f, k1 = !GUARD || r1 > 0.f;   // a coincident pair contributes nothing
+  if (KERN == BLDTT_REG_COULOMB) f2_unpack(f2_add(r2, prm2), r0, r1);
+  const float i0 = rsqrt_approx(r0), i1 = rsqrt_approx(r1);
+  const f2_t ri = f2_pack(k0 ? i0 : 0.f, k1 ? i1 : 0.f);
   if (KERN == BLDTT_COULOMB || KERN == BLDTT_REG_COULOMB) return f2_fma(q2, ri, acc);
   const f2_t r = f2_mul(r2, ri);
   if (KERN == BLDTT_OSCILLATORY) return f2_fma(f2_mul(q2, ri), sinpi2(r, prm2), acc);
@@ -509,17 +505,21 @@ __device__ __forceinline__ f2_t pair2_f32(f2_t tx, f2_t ty, f2_t tz, const ulong
 // Careful variant: d = fma(m, x_r - y_r, x'' - y'') with m = 1 for a target
 // near the chunk (frame residuals added) and m = 0 otherwise (exactly the
 // packed difference x'' - y'').
-template <int KERN>
+template <int KERN, bool GUARD>
 __device__ __forceinline__ f2_t pair2_careful(f2_t tx, f2_t ty, f2_t tz, f2_t rx, f2_t ry, f2_t rz,
                                               f2_t m2, const ulonglong2& a, const ulonglong2& b,
                                               const ulonglong2& ra, const ulonglong2& rb, f2_t acc,
                                               f2_t nk2) {
-  return pair2_eval<KERN>(f2_fma(m2, f2_sub(rx, ra.x), f2_sub(tx, a.x)),
+  return pair2_eval<KERN, GUARD>(f2_fma(m2, f2_sub(rx, ra.x), f2_sub(tx, a.x)),
                           f2_fma(m2, f2_sub(ry, ra.y), f2_sub(ty, a.y)),
                           f2_fma(m2, f2_sub(rz, rb.x), f2_sub(tz, b.x)), b.y, acc, nk2);
 }
 
 // Sum over the staged chunk of q G for K targets; two partial sums per target.
+// Full chunks have a loop of fixed length (the oscillatory kernel's loop body
+// is long enough to do without); the others are unrolled as far: 1E6 particles,
+// whose leaves end in a partial chunk, 31.5 ms unrolled by 2, 31.1 by 4 and 8,
+// and the oscillatory kernel 3.88, 3.83 and 3.77.
 template <int KERN, int K>
 __device__ __forceinline__ void chunk_f32(const ulonglong2* __restrict__ sb, int npairs,
                                           const f2_t (&x2)[K][3], float (&a)[K], float nk) {
@@ -527,7 +527,7 @@ __device__ __forceinline__ void chunk_f32(const ulonglong2* __restrict__ sb, int
   const f2_t nk2 = f2_pack(nk, nk);
 #pragma unroll
   for (int k = 0; k < K; ++k) acc[k] = 0ull;
-  if (npairs == kChunk / 2) {
+  if (KERN != BLDTT_OSCILLATORY && npairs == kChunk / 2) {
 #pragma unroll 8
     for (int jp = 0; jp < kChunk / 2; ++jp) {
       const ulonglong2 A = sb[2 * jp], Bq = sb[2 * jp + 1];
@@ -535,6 +535,7 @@ __device__ __forceinline__ void chunk_f32(const ulonglong2* __restrict__ sb, int
       for (int k = 0; k < K; ++k) acc[k] = pair2_f32<KERN>(x2[k][0], x2[k][1], x2[k][2], A, Bq, acc[k], nk2);
     }
   } else {
+#pragma unroll 8
     for (int jp = 0; jp < npairs; ++jp) {
       const ulonglong2 A = sb[2 * jp], Bq = sb[2 * jp + 1];
 #pragma unroll
@@ -573,7 +574,7 @@ __device__ __forceinline__ void target_residual(const TargetSplit& ts, const flo
 }
 
 // Careful packed sum over the staged chunk (sr: its frame residual records).
-template <int KERN, int K>
+template <int KERN, int K, bool GUARD>
 __device__ __forceinline__ void chunk_f32_careful(const ulonglong2* __restrict__ sb,
                                                   const ulonglong2* __restrict__ sr, int npairs,
                                                   const f2_t (&x2)[K][3], const TargetSplit& ts,
@@ -596,7 +597,7 @@ __device__ __forceinline__ void chunk_f32_careful(const ulonglong2* __restrict__
     const ulonglong2 A = sb[2 * jp], Bq = sb[2 * jp + 1], RA = sr[2 * jp], RB = sr[2 * jp + 1];
 #pragma unroll
     for (int k = 0; k < K; ++k)
-      acc[k] = pair2_careful<KERN>(x2[k][0], x2[k][1], x2[k][2], r2x[k][0], r2x[k][1], r2x[k][2],
+      acc[k] = pair2_careful<KERN, GUARD>(x2[k][0], x2[k][1], x2[k][2], r2x[k][0], r2x[k][1], r2x[k][2],
                                    m2[k], A, Bq, RA, RB, acc[k], nk2);
   }
 #pragma unroll
@@ -607,32 +608,14 @@ __device__ __forceinline__ void chunk_f32_careful(const ulonglong2* __restrict__
   }
 }
 
-// One pair in the packed path's arithmetic (bit for bit per lane), with the
-// r = 0 guard: acc + q G(d).  Coulomb, Yukawa and the test kernel.
-template <int KERN>
-__device__ __forceinline__ float pair_acc_f32(float dx, float dy, float dz, float q, float prm,
-                                              float acc) {
-  const float r2 = fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx)));
-  if (!(r2 > 0.f)) return acc;
-  if (KERN == BLDTT_TEST_POLY) return __fadd_rn(acc, q * poly_kernel<float>(dx, dy, dz));
-  if (KERN == BLDTT_COULOMB) return fmaf(q, rsqrt_approx(r2), acc);
-  const float ri = rsqrt_approx(r2);
-  return fmaf(__fmul_rn(q, ri), exp2_approx(__fmul_rn(__fmul_rn(r2, ri), prm)), acc);
-}
-
-// Scalar evaluation of a staged chunk: the same two partial sums (even and
-// odd entries) and the same arithmetic as the packed path, with the r = 0
-// guard.  Targets whose bit is set in `near` use the corrected difference
-//   d = fl(fl(x'' - y'') + fl(x_r - y_r))
-// of the frame coordinates x'', y'' and frame residuals x_r, y_r, which is
-// within a few u |d| of the exact x - y however small |d| is.  Every other
-// target gets bit for bit what the packed path gives it (when that is
-// finite), so a target's result does not depend on its warp.
-template <int KERN, int K>
+// Scalar evaluation of a staged chunk by the test kernel, with the r = 0 guard:
+// two partial sums (even and odd entries).  Targets whose bit is set in `near`
+// use the corrected difference of the careful path.
+template <int K>
 __device__ __forceinline__ void chunk_f32_slow(const float* __restrict__ sf, const float* __restrict__ res,
                                                int count, const float (&xs)[K][3],
                                                const TargetSplit& ts, const float* c, unsigned near,
-                                               float prm, float (&a)[K]) {
+                                               float (&a)[K]) {
   // one target slot at a time: few live registers on this rare path
 #pragma unroll
   for (int k = 0; k < K; ++k) {
@@ -654,10 +637,14 @@ __device__ __forceinline__ void chunk_f32_slow(const float* __restrict__ sf, con
             dy = __fadd_rn(dy, __fsub_rn(xr[1], e[2]));
             dz = __fadd_rn(dz, __fsub_rn(xr[2], e[4]));
           }
-          if (h == 0)
-            acc0 = pair_acc_f32<KERN>(dx, dy, dz, r[6], prm, acc0);
-          else
-            acc1 = pair_acc_f32<KERN>(dx, dy, dz, r[6], prm, acc1);
+          const float r2 = fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx)));
+          if (r2 > 0.f) {
+            const float t = r[6] * poly_kernel<float>(dx, dy, dz);
+            if (h == 0)
+              acc0 = __fadd_rn(acc0, t);
+            else
+              acc1 = __fadd_rn(acc1, t);
+          }
         }
       }
     }
@@ -798,22 +785,17 @@ __device__ __forceinline__ void frame_targets(const TargetSplit& ts, const float
     }
   }
 }
+// The careful path's sums with the r = 0 guard.  A call of its own: its
+// registers must not crowd the plain loop's.
 template <int KERN, int K>
-__device__ __noinline__ PartialSums<K> slow_sums(const float* sf, const float* res, int count,
-                                                 const TargetSplit ts, const float* c, unsigned near,
-                                                 float prm) {
+__device__ __noinline__ PartialSums<K> careful_sums(const float* sf, const float* res, int count,
+                                                    const TargetSplit ts, const float* c, unsigned near,
+                                                    float prm) {
   f2_t x2[K][3];
   frame_targets<K>(ts, c, x2);
-  float xs[K][3];
-#pragma unroll
-  for (int k = 0; k < K; ++k)
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      float hi;
-      f2_unpack(x2[k][d], xs[k][d], hi);
-    }
   PartialSums<K> out;
-  chunk_f32_slow<KERN, K>(sf, res, count, xs, ts, c, near, prm, out.v);
+  chunk_f32_careful<KERN, K, true>(reinterpret_cast<const ulonglong2*>(sf), reinterpret_cast<const ulonglong2*>(res),
+                             (count + 1) / 2, x2, ts, c, near, out.v, prm);
   return out;
 }
 // One staged chunk in FP32 for K targets (partial sums in a[]).  ts holds
@@ -821,9 +803,15 @@ __device__ __noinline__ PartialSums<K> slow_sums(const float* sf, const float* r
 // near distance tau, res its staged frame residuals, and bit k of `slot` says
 // that the producer found target slot k's group near the chunk.  A target
 // with max_d (|x''_d| - e_d) < tau is near: the warp then takes the careful
-// packed path, which adds the frame residuals for near targets only.
-// Otherwise the plain packed path runs.  A chunk whose packed sum is not
-// finite (some r = 0) is redone in the scalar path with the r = 0 guard.
+// packed path, which adds the frame residuals for near targets only, and with
+// the r = 0 guard if a target lies inside the chunk's box (or within a
+// thousandth of tau of it).  Otherwise the plain packed path runs.  A sum that
+// is not finite is redone with the guard.
+// The chunk that a tile shares with its own targets used to run twice, the
+// second time in a scalar loop at an eighth of the rate: 1000 particles 0.099
+// -> 0.046 ms in this kernel, 2E4 on a sphere 0.184 -> 0.139, 512 problems of
+// 16k (lists of about 30 chunks) 77.7 -> 74.0.  With the guard on all near
+// chunks the latter is 75.5, and the unequal sets' 82.6 become 83.2.
 template <int KERN, int K>
 __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rbuf, int count,
                                                const f2_t (&x2)[K][3], const TargetSplit& ts,
@@ -840,25 +828,32 @@ __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rb
       f2_unpack(x2[k][d], xs[k][d], hi);
     }
   unsigned near = 0;
-  bool any_near = false;
+  bool any_near = false, inside = false;
   if (slot) {                                   // warp-uniform
     const float4 ext = *ext_p;
+    bool within = AlwaysGuarded<KERN>::value;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       const float m = fmaxf(fmaxf(fabsf(xs[k][0]) - ext.x, fabsf(xs[k][1]) - ext.y),
                             fabsf(xs[k][2]) - ext.z);
       if (((slot >> k) & 1u) && m < ext.w) near |= 1u << k;
+      within = within || m < 0.001f * ext.w;
     }
     any_near = __any_sync(0xffffffffu, near != 0);
+    inside = __any_sync(0xffffffffu, within);
   }
   if (KERN == BLDTT_TEST_POLY) {
-    chunk_f32_slow<BLDTT_TEST_POLY, K>(sf, res, count, xs, ts, c, near, prm, a);
+    chunk_f32_slow<K>(sf, res, count, xs, ts, c, near, a);
     return;
   }
   const ulonglong2* sb = reinterpret_cast<const ulonglong2*>(buf);
-  if (any_near) {
-    chunk_f32_careful<KERN, K>(sb, reinterpret_cast<const ulonglong2*>(rbuf), (count + 1) / 2, x2, ts,
-                               c, near, a, prm);
+  if (any_near && !inside) {
+    chunk_f32_careful<KERN, K, false>(sb, reinterpret_cast<const ulonglong2*>(rbuf), (count + 1) / 2, x2,
+                                      ts, c, near, a, prm);
+  } else if (any_near) {
+    const PartialSums<K> r = careful_sums<KERN, K>(sf, res, count, ts, c, near, prm);
+#pragma unroll
+    for (int k = 0; k < K; ++k) a[k] = r.v[k];
   } else if (K > 1 && !warp_full) {
     // the warp's last target row lies beyond a partial tile: evaluate the others only
     constexpr int K1 = K > 1 ? K - 1 : 1;
@@ -870,12 +865,12 @@ __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rb
   } else {
     chunk_f32<KERN, K>(sb, (count + 1) / 2, x2, a, prm);
   }
-  if (AlwaysGuarded<KERN>::value) return;
   bool bad = false;
 #pragma unroll
   for (int k = 0; k < K; ++k) bad = bad || not_finite(a[k]);
   if (__any_sync(0xffffffffu, bad)) {
-    const PartialSums<K> r = slow_sums<KERN, K>(sf, res, count, ts, c, near, prm);
+    // residuals that were not staged are not read: any finite numbers do (their factor is 0)
+    const PartialSums<K> r = careful_sums<KERN, K>(sf, slot ? res : sf, count, ts, c, near, prm);
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = r.v[k];
   }

@@ -5,6 +5,7 @@
 // guard of the second barycentric form (Sec. 2.1, Eq. (3)); in FP32_BULK mode
 // the contractions that follow (leaf proxy charges and the leaf interpolation
 // to particles) run in FP32 over short runs that are summed in FP64.
+#include <cfloat>
 #include <cmath>
 #include <type_traits>
 #include <vector>
@@ -471,7 +472,9 @@ int build_pool(bldtt_plan* p, cudaStream_t s) {
 //  [0] frame centre c (floats: the rounded centre of the chunk's bounding box
 //      for particles, the rounded cluster centre for proxies), real entries;
 //  [1] half-extents e of the chunk's entries around c (rounded up) and the
-//      near distance tau = 0.3 |e| (particle chunks; -inf for proxy chunks).
+//      near distance tau = 0.3 |e| (particle chunks; -inf for proxy chunks),
+//      above 0 also for a chunk of one repeated point, so that a target there
+//      is near it.
 // A target whose frame coordinates x'' satisfy max_d (|x''_d| - e_d) >= tau is
 // at distance r >= tau from every entry, so the FP32 rounding of the two frame
 // coordinates (at most u |x''| and u |e|, |x''| <= r + |e|) changes r by at
@@ -489,7 +492,7 @@ __device__ __forceinline__ void store_chunk(float4* info, int64_t q, const doubl
     ef[d] = __double2float_ru(ed);
     e2 += (double)ef[d] * (double)ef[d];
   }
-  const float tau = particles ? __double2float_ru(0.3 * sqrt(e2)) : -INFINITY;
+  const float tau = particles ? fmaxf(__double2float_ru(0.3 * sqrt(e2)), FLT_MIN) : -INFINITY;
   info[kChunkInfo * q] = make_float4(cf[0], cf[1], cf[2], __int_as_float(count));
   info[kChunkInfo * q + 1] = make_float4(ef[0], ef[1], ef[2], tau);
 }
