@@ -303,68 +303,64 @@ __global__ void __launch_bounds__(kDttThreads) k_dtt_all(
   }
 }
 
-// Root pair (r, r) of every problem r.
-__global__ void k_root_pairs(int2* __restrict__ front, int32_t P) {
+// Root pair (r, r) of every problem r; g (of a cooperative traversal) is reset.
+__global__ void k_root_pairs(int2* __restrict__ front, int32_t P, DttGrid* __restrict__ g) {
   const int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r < P) front[r] = make_int2(r, r);
+  if (g && r == 0) {
+    *g = DttGrid{};
+    g->F0 = P;
+  }
 }
 
-__global__ void k_iota(int32_t* v, int64_t n) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) v[i] = (int32_t)i;
-}
+static inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
-__global__ void k_gather_i32(const int32_t* __restrict__ src, const int32_t* __restrict__ idx,
-                             int32_t* __restrict__ dst, int64_t n) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = src[idx[i]];
-}
-
-__global__ void k_key_hist(const uint32_t* __restrict__ keys, int64_t n, int32_t* __restrict__ cnt) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) atomicAdd(&cnt[keys[i]], 1);
-}
-
-// Kernel evaluations per list class (Eqs. (6), (8), (12), (15)); integer sums,
-// exact.  Each CTA sums its entries per class in shared memory first, so the
-// global counters see one atomic per class and CTA.
-__global__ void k_count_evals(const int32_t* __restrict__ et, const int32_t* __restrict__ es,
-                              const uint32_t* __restrict__ key, int64_t n, int32_t nct,
-                              TreeView tt, TreeView st, DegreeSet deg,
-                              unsigned long long* __restrict__ out) {
+// The lists from the sorted entries, in one launch: thread i gathers entry i
+// and counts its kernel evaluations (Eqs. (6), (8), (12), (15); integer sums,
+// exact, one atomic per class and CTA), and finds offset i of the CSR by
+// bisection (its first entry with a key >= i; a histogram and its scan took
+// five launches).  out: kMaxClasses evaluation counters, then the class
+// offsets list_ptr[k * nct], k = 0..nclass, as int32.
+__global__ void k_lists(const uint32_t* __restrict__ key, const int32_t* __restrict__ order,
+                        const int32_t* __restrict__ ent_t, const int32_t* __restrict__ ent_s, int64_t n,
+                        int32_t nct, int nclass, TreeView tt, TreeView st, DegreeSet deg,
+                        int32_t* __restrict__ list_tgt, int32_t* __restrict__ list_src,
+                        int32_t* __restrict__ list_ptr, unsigned long long* __restrict__ out) {
   __shared__ unsigned long long part[kMaxClasses];
   if (threadIdx.x < kMaxClasses) part[threadIdx.x] = 0ull;
   __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
+    const int32_t o = order[i], t = ent_t[o], s = ent_s[o];
+    list_tgt[i] = t;
+    list_src[i] = s;
     const int c = (int)(key[i] / (uint32_t)nct);
     const int type = class_type(c);
     const int64_t np = deg.np[class_degree(c)];
-    int64_t ct = tt.end[et[i]] - tt.begin[et[i]], cs = st.end[es[i]] - st.begin[es[i]];
-    int64_t v = type == BLDTT_PP ? ct * cs : type == BLDTT_PC ? ct * np : type == BLDTT_CP ? np * cs : np * np;
+    const int64_t ct = tt.end[t] - tt.begin[t], cs = st.end[s] - st.begin[s];
+    const int64_t v = type == BLDTT_PP ? ct * cs : type == BLDTT_PC ? ct * np : type == BLDTT_CP ? np * cs : np * np;
     atomicAdd(&part[c], (unsigned long long)v);
+  }
+  if (i <= (int64_t)nclass * nct) {
+    int64_t lo = 0, hi = n;
+    while (lo < hi) {
+      const int64_t m = (lo + hi) >> 1;
+      if ((int64_t)key[m] < i) lo = m + 1; else hi = m;
+    }
+    list_ptr[i] = (int32_t)lo;
+    if (i % nct == 0) reinterpret_cast<int32_t*>(out + kMaxClasses)[i / nct] = (int32_t)lo;
   }
   __syncthreads();
   if (threadIdx.x < kMaxClasses && part[threadIdx.x]) atomicAdd(&out[threadIdx.x], part[threadIdx.x]);
 }
 
-static inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
-
-// Offsets list_ptr[k * nct], k = 0..nclass, written as int32 after the
-// kMaxClasses evaluation counters of `out`.
-__global__ void k_class_bounds(const int32_t* __restrict__ list_ptr, int32_t nct, int nclass,
-                               unsigned long long* __restrict__ out) {
-  int32_t* o = reinterpret_cast<int32_t*>(out + kMaxClasses);
-  for (int k = threadIdx.x; k <= nclass; k += blockDim.x) o[k] = list_ptr[(int64_t)k * nct];
-}
-
-// The fixed-rule traversal from the P root pairs in `roots` by one cooperative
+// The fixed-rule traversal from the P root pairs by one cooperative
 // launch (k_dtt_all).  On success *E receives the entry count, the three entry
 // arrays are allocated here and *done is set; when a buffer would overflow the
 // capacity is doubled and the launch repeated (twice at most), after which
 // *done stays false and the caller runs the level-by-level loop.
-static int traverse_cooperative(bldtt_plan* p, const TreeView& tt, const TreeView& st, const int2* roots,
-                                int32_t P, int32_t** ent_t, int32_t** ent_s, uint32_t** ent_key,
+static int traverse_cooperative(bldtt_plan* p, const TreeView& tt, const TreeView& st, int32_t P,
+                                int32_t** ent_t, int32_t** ent_s, uint32_t** ent_key,
                                 int64_t* E, bool* done, cudaStream_t s) {
   *done = false;
   if (cooperative_set_up_disabled()) return BLDTT_OK;
@@ -400,9 +396,8 @@ static int traverse_cooperative(bldtt_plan* p, const TreeView& tt, const TreeVie
     BL_TRY(dalloc_n(&et, cap, s));
     BL_TRY(dalloc_n(&es, cap, s));
     BL_TRY(dalloc_n(&ek, cap, s));
-    BL_CUDA(cudaMemsetAsync(g, 0, sizeof(DttGrid), s));
-    BL_CUDA(cudaMemcpyAsync(b0, roots, (size_t)P * sizeof(int2), cudaMemcpyDeviceToDevice, s));
-    BL_CUDA(cudaMemcpyAsync(&g->F0, &P, sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    k_root_pairs<<<nblk(P, 256), 256, 0, s>>>(b0, P, g);
+    BL_LAUNCHED(p->setup_counter.launches);
     int64_t np = p->deg.np[imax];
     double theta = p->theta;
     int variant = p->variant;
@@ -452,9 +447,6 @@ int build_lists(bldtt_plan* p, cudaStream_t s) {
   // One root pair per problem (Alg. 2 starts from the two roots of each problem).
   const int32_t P = p->tt.nroots;
   fcap = std::max(fcap, (size_t)P);
-  BL_TRY(dalloc_n(&front, fcap, s));
-  k_root_pairs<<<nblk(P, 256), 256, 0, s>>>(front, P);
-  BL_LAUNCHED(cnt.launches);
   int32_t F = P;
   int64_t E = 0;
   const int imax = p->deg.n - 1;
@@ -465,7 +457,7 @@ int build_lists(bldtt_plan* p, cudaStream_t s) {
     bool done = false;
     int32_t *ct = nullptr, *cs = nullptr;
     uint32_t* ck = nullptr;
-    BL_TRY(traverse_cooperative(p, tt, st, front, P, &ct, &cs, &ck, &E, &done, s));
+    BL_TRY(traverse_cooperative(p, tt, st, P, &ct, &cs, &ck, &E, &done, s));
     if (done) {
       ent_t = ct;
       ent_s = cs;
@@ -474,6 +466,9 @@ int build_lists(bldtt_plan* p, cudaStream_t s) {
     }
   }
   if (F > 0) {   // the level-by-level loop's buffers
+    BL_TRY(dalloc_n(&front, fcap, s));
+    k_root_pairs<<<nblk(P, 256), 256, 0, s>>>(front, P, nullptr);
+    BL_LAUNCHED(cnt.launches);
     BL_TRY(dalloc_n(&next, ncap, s));
     BL_TRY(dalloc_n(&ent_t, ecap, s));
     BL_TRY(dalloc_n(&ent_s, ecap, s));
@@ -538,45 +533,24 @@ int build_lists(bldtt_plan* p, cudaStream_t s) {
   int key_bits = 1;
   while ((1ull << key_bits) < (unsigned long long)nclass * (unsigned long long)nct) ++key_bits;
   int32_t* order = nullptr;
-  BL_TRY(dalloc_n(&order, E, s));
-  if (E > 0) {
-    k_iota<<<nblk(E, 256), 256, 0, s>>>(order, E);
-    BL_LAUNCHED(cnt.launches);
-  }
-  BL_TRY(radix_sort_pairs(ent_key, order, E, key_bits, s, cnt));
-  BL_TRY(dalloc_n(&p->list_src, E, s));
-  BL_TRY(dalloc_n(&p->list_tgt, E, s));
-  if (E > 0) {
-    k_gather_i32<<<nblk(E, 256), 256, 0, s>>>(ent_s, order, p->list_src, E);
-    BL_LAUNCHED(cnt.launches);
-    k_gather_i32<<<nblk(E, 256), 256, 0, s>>>(ent_t, order, p->list_tgt, E);
-    BL_LAUNCHED(cnt.launches);
-  }
-  int64_t nkeys = (int64_t)nclass * nct;
-  int32_t* hist = nullptr;
-  BL_TRY(dalloc_n(&hist, nkeys, s));
-  BL_TRY(dalloc_n(&p->list_ptr, nkeys + 1, s));
-  BL_CUDA(cudaMemsetAsync(hist, 0, nkeys * sizeof(int32_t), s));
-  if (E > 0) {
-    k_key_hist<<<nblk(E, 256), 256, 0, s>>>(ent_key, E, hist);
-    BL_LAUNCHED(cnt.launches);
-  }
-  BL_TRY(scan_exclusive_dev(hist, p->list_ptr, nkeys, p->list_ptr + nkeys, s, cnt));   // total last
-
+  const int64_t nkeys = (int64_t)nclass * nct;
   // evals: kMaxClasses counters, then room for the nclass + 1 class offsets
   constexpr int kRead = kMaxClasses + (kMaxClasses + 2) / 2;
   unsigned long long* evals = nullptr;
-  BL_TRY(dalloc_n(&evals, kRead, s));
+  Arena scratch;
+  scratch.add(&order, E);
+  scratch.add(&evals, kRead);
+  BL_TRY(scratch.alloc(s));
   BL_CUDA(cudaMemsetAsync(evals, 0, kRead * sizeof(unsigned long long), s));
-  if (E > 0) {
-    k_count_evals<<<nblk(E, 256), 256, 0, s>>>(p->list_tgt, p->list_src, ent_key, E, nct, tt, st,
-                                               p->deg, evals);
-    BL_LAUNCHED(cnt.launches);
-  }
-  // class boundaries of the CSR and the evaluation counts, in one read
-  unsigned long long h_read[kMaxClasses + (kMaxClasses + 2) / 2];
-  k_class_bounds<<<1, 32, 0, s>>>(p->list_ptr, nct, nclass, evals);
+  BL_TRY(sort_order(ent_key, order, E, key_bits, s, cnt));
+  BL_TRY(dalloc_n(&p->list_src, E, s));
+  BL_TRY(dalloc_n(&p->list_tgt, E, s));
+  BL_TRY(dalloc_n(&p->list_ptr, nkeys + 1, s));
+  k_lists<<<nblk(std::max<int64_t>(E, nkeys + 1), 256), 256, 0, s>>>(
+      ent_key, order, ent_t, ent_s, E, nct, nclass, tt, st, p->deg, p->list_tgt, p->list_src, p->list_ptr, evals);
   BL_LAUNCHED(cnt.launches);
+  // class boundaries of the CSR and the evaluation counts, in one read
+  unsigned long long h_read[kRead];
   BL_TRY(read_device(evals, h_read, sizeof(h_read), s));
   const unsigned long long* h_evals = h_read;
   const int32_t* h_ptr = reinterpret_cast<const int32_t*>(h_read + kMaxClasses);
@@ -598,7 +572,7 @@ int build_lists(bldtt_plan* p, cudaStream_t s) {
     set_error("interaction list CSR holds %d entries, traversal produced %lld", h_ptr[nclass], (long long)E);
     return BLDTT_EINTERNAL;
   }
-  dfree(evals, s); dfree(hist, s); dfree(order, s);
+  scratch.release(s);
   dfree(ent_t, s); dfree(ent_s, s); dfree(ent_key, s);
   return BLDTT_OK;
 }
@@ -626,19 +600,19 @@ struct ListView {
 
 // Real sources (no padding) and pool chunks that the entries of list class
 // `cls` of target cluster c contribute: particles of source clusters
-// (particles = true) or proxies of degree index i.
+// (particles = true) or proxies of degree index i; this lane's share.
 __device__ __forceinline__ void class_work(const ListView& L, const int32_t* s_begin, const int32_t* s_end,
-                                           int cls, bool particles, int i, int32_t c, int64_t& sources,
-                                           int64_t& chunks) {
+                                           int cls, bool particles, int i, int32_t c, int lane,
+                                           int64_t& sources, int64_t& chunks) {
   const int64_t k = (int64_t)cls * L.nct + c;
   const int32_t e0 = L.ptr[k], e1 = L.ptr[k + 1];
   if (particles) {
-    for (int32_t e = e0; e < e1; ++e) {
+    for (int32_t e = e0 + lane; e < e1; e += 32) {
       const int32_t s = L.src[e];
       sources += s_end[s] - s_begin[s];
       chunks += (L.pad_prefix[L.s_leaf_last[s]] - L.pad_prefix[L.s_leaf_first[s]]) / kChunk;
     }
-  } else {
+  } else if (lane == 0) {
     sources += (int64_t)(e1 - e0) * L.deg.np[i];
     chunks += (int64_t)(e1 - e0) * (L.deg.np_pad[i] / kChunk);
   }
@@ -655,10 +629,16 @@ __device__ __forceinline__ int64_t executed_rows_noskip(int64_t m) {
   return m - r + (r == 0 ? 0 : (r <= kTile / 2 ? kTile / 2 : (r + 31) / 32 * 32));
 }
 
+__device__ __forceinline__ int64_t warp_sum(int64_t v) {
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // Items of target cluster c: tiles of its particles (a leaf: PP and PC of every
 // degree, on the leaf and on each ancestor), and tiles of its proxy points of
 // degree i (CP and CC of degree i on the cluster itself).  cost_prox is
-// [nct][kMaxDegrees].
+// [nct][kMaxDegrees].  One warp per cluster: its lists are walked 32 entries at
+// a time.
 __global__ void k_item_count(int32_t nct, ListView L, const int32_t* __restrict__ parent,
                              const int32_t* __restrict__ nchild, const int32_t* __restrict__ begin,
                              const int32_t* __restrict__ end, const int32_t* __restrict__ s_begin,
@@ -666,43 +646,51 @@ __global__ void k_item_count(int32_t nct, ListView L, const int32_t* __restrict_
                              int64_t* __restrict__ cost_part, int64_t* __restrict__ cost_prox,
                              unsigned long long* __restrict__ executed,   // [2]: skip, no skip
                              int64_t* __restrict__ eval_part, int64_t* __restrict__ eval_prox,
-                             int64_t part_len, int32_t* __restrict__ nsplit) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nct) return;
+                             int64_t part_len, int32_t* __restrict__ nsplit, int32_t* __restrict__ longest) {
+  const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (c >= nct) return;                 // whole warps
   int64_t cp = 0, sp = 0;
   if (nchild[c] == 0)   // PP + PC of the leaf and of all its ancestors (Sec. 2.7 chain)
     for (int32_t a = c; a >= 0; a = parent[a]) {
-      class_work(L, s_begin, s_end, 0, true, 0, a, sp, cp);
+      class_work(L, s_begin, s_end, 0, true, 0, a, lane, sp, cp);
       for (int i = 0; i < L.deg.n; ++i)
-        class_work(L, s_begin, s_end, class_of(BLDTT_PC, i), false, i, a, sp, cp);
+        class_work(L, s_begin, s_end, class_of(BLDTT_PC, i), false, i, a, lane, sp, cp);
     }
+  cp = warp_sum(cp);
+  sp = warp_sum(sp);
   const int32_t tp = cp > 0 ? (end[c] - begin[c] + kTile - 1) / kTile : 0;
   const PartPlan pp = plan_parts(cp, part_len);
+  int64_t len = (int64_t)pp.per * pp.len;     // chunks of its longest task, or more
   int32_t items = tp * pp.parts;
   int32_t split = pp.parts > 1 ? tp : 0;
   unsigned long long ex = cp > 0 ? (unsigned long long)executed_rows_skip(end[c] - begin[c]) * sp : 0ull;
   unsigned long long ex_ns = cp > 0 ? (unsigned long long)executed_rows_noskip(end[c] - begin[c]) * sp : 0ull;
-  eval_part[c] = cp > 0 ? (int64_t)(end[c] - begin[c]) * sp : 0;   // real evaluations (no padding)
   int64_t evq = 0;
   for (int i = 0; i < L.deg.n; ++i) {   // CP + CC of degree i on the cluster itself
     int64_t cq = 0, sq = 0;
-    class_work(L, s_begin, s_end, class_of(BLDTT_CP, i), true, i, c, sq, cq);
-    class_work(L, s_begin, s_end, class_of(BLDTT_CC, i), false, i, c, sq, cq);
+    class_work(L, s_begin, s_end, class_of(BLDTT_CP, i), true, i, c, lane, sq, cq);
+    class_work(L, s_begin, s_end, class_of(BLDTT_CC, i), false, i, c, lane, sq, cq);
+    cq = warp_sum(cq);
+    sq = warp_sum(sq);
     const int32_t tq = cq > 0 ? (L.deg.np[i] + kTile - 1) / kTile : 0;
     const PartPlan pq = plan_parts(cq, part_len);
+    len = max(len, (int64_t)pq.per * pq.len);
     items += tq * pq.parts;
     if (pq.parts > 1) split += tq;
-    cost_prox[(int64_t)c * kMaxDegrees + i] = cq;
+    if (lane == 0) cost_prox[(int64_t)c * kMaxDegrees + i] = cq;
     if (cq > 0) {
       ex += (unsigned long long)executed_rows_skip(L.deg.np[i]) * sq;
       ex_ns += (unsigned long long)executed_rows_noskip(L.deg.np[i]) * sq;
     }
     if (cq > 0) evq += (int64_t)L.deg.np[i] * sq;
   }
+  if (lane) return;
+  eval_part[c] = cp > 0 ? (int64_t)(end[c] - begin[c]) * sp : 0;   // real evaluations (no padding)
   eval_prox[c] = evq;
   nitems[c] = items;
   cost_part[c] = cp;
   if (split) atomicAdd(nsplit, split);
+  atomicMax(longest, (int32_t)min(len, (int64_t)INT32_MAX));
   // evaluations the kernel performs: every target slot of every tile meets every real source
   if (ex) atomicAdd(executed, ex);
   if (ex_ns) atomicAdd(executed + 1, ex_ns);
@@ -719,18 +707,16 @@ struct SegmentMap {
 
 // The tasks of one tile {c, r, rows, kind} of `chunks` source chunks.
 __device__ __forceinline__ void fill_tasks(int4 tile, int64_t chunks, int64_t part_len, uint32_t key_base,
-                                           int32_t& o, int32_t* next_slot, int4* items, int4* parts,
-                                           uint32_t* keys, int32_t* vals) {
+                                           uint32_t key_max, int32_t& o, int32_t* next_slot, int4* items,
+                                           int4* parts, uint32_t* keys) {
   const PartPlan q = plan_parts(chunks, part_len);
   // the slot numbers depend on the order of the atomics, the results do not
   const int32_t slot = q.parts > 1 ? atomicAdd(next_slot, 1) : -1;
-  const uint32_t kKeyMax = (1u << 24) - 1u;
   for (int32_t i = 0; i < q.parts; ++i) {
     const int64_t b = (int64_t)i * q.per * q.len, e = min(chunks, b + (int64_t)q.per * q.len);
     items[o] = tile;
     parts[o] = make_int4((int)b, (int)(e - b), slot, q.nseg | (q.len << 8));
-    keys[o] = key_base | (kKeyMax - (uint32_t)min((int64_t)kKeyMax, e - b));
-    vals[o] = o;
+    keys[o] = key_base | (key_max - (uint32_t)min((int64_t)key_max, e - b));
     ++o;
   }
 }
@@ -739,9 +725,9 @@ __global__ void k_item_fill(int32_t nct, const int32_t* __restrict__ off,
                             const int64_t* __restrict__ cost_part, const int64_t* __restrict__ cost_prox,
                             const int32_t* __restrict__ begin, const int32_t* __restrict__ end,
                             const int32_t* __restrict__ problem, const int* __restrict__ prob_kernel,
-                            SegmentMap segmap, DegreeSet deg, int64_t part_len, int32_t* __restrict__ next_slot,
-                            int4* __restrict__ items, int4* __restrict__ parts, uint32_t* __restrict__ keys,
-                            int32_t* __restrict__ vals) {
+                            SegmentMap segmap, DegreeSet deg, int64_t part_len, int len_bits,
+                            int32_t* __restrict__ next_slot,
+                            int4* __restrict__ items, int4* __restrict__ parts, uint32_t* __restrict__ keys) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= nct) return;
   int32_t o = off[c];
@@ -754,37 +740,33 @@ __global__ void k_item_fill(int32_t nct, const int32_t* __restrict__ off,
       seg = (uint32_t)i;
       sub = segmap.kernel[i] == kKernCoulombYukawa && kern == BLDTT_YUKAWA ? 1u : 0u;
     }
-  const uint32_t key_base = (seg << 25) | (sub << 24);
+  const uint32_t key_base = (seg << (len_bits + 1)) | (sub << len_bits), key_max = (1u << len_bits) - 1u;
   if (cost_part[c] > 0)
     for (int32_t r = begin[c]; r < end[c]; r += kTile)
-      fill_tasks(make_int4(c, r, min(kTile, end[c] - r), kItemParticles), cost_part[c], part_len, key_base, o,
-                 next_slot, items, parts, keys, vals);
+      fill_tasks(make_int4(c, r, min(kTile, end[c] - r), kItemParticles), cost_part[c], part_len, key_base,
+                 key_max, o, next_slot, items, parts, keys);
   for (int i = 0; i < deg.n; ++i) {
     const int64_t cq = cost_prox[(int64_t)c * kMaxDegrees + i];
     if (cq <= 0) continue;
     const int32_t np = deg.np[i];
     for (int32_t r = 0; r < np; r += kTile)
-      fill_tasks(make_int4(c, r, min(kTile, np - r), kItemProxies + i), cq, part_len, key_base, o, next_slot,
-                 items, parts, keys, vals);
+      fill_tasks(make_int4(c, r, min(kTile, np - r), kItemProxies + i), cq, part_len, key_base, key_max, o,
+                 next_slot, items, parts, keys);
   }
 }
 
-// First item of every segment (keys sorted): first[seg] = i where the segment starts.
-__global__ void k_segment_starts(const uint32_t* __restrict__ keys, int32_t n, int32_t* __restrict__ first) {
-  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+// Items in their sorted order, and one past the first item of every segment
+// (0: none): first[seg] = i + 1 where the segment starts.
+__global__ void k_gather_items(const uint32_t* __restrict__ keys, int seg_shift, const int4* __restrict__ src,
+                               const int4* __restrict__ psrc, const int32_t* __restrict__ idx,
+                               int4* __restrict__ dst, int4* __restrict__ pdst, int64_t n,
+                               int32_t* __restrict__ first) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const uint32_t sg = keys[i] >> 25;
-  if (i == 0 || (keys[i - 1] >> 25) != sg) first[sg] = i;
-}
-
-__global__ void k_gather_items(const int4* __restrict__ src, const int4* __restrict__ psrc,
-                               const int32_t* __restrict__ idx, int4* __restrict__ dst,
-                               int4* __restrict__ pdst, int64_t n) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) {
-    dst[i] = src[idx[i]];
-    pdst[i] = psrc[idx[i]];
-  }
+  dst[i] = src[idx[i]];
+  pdst[i] = psrc[idx[i]];
+  const uint32_t sg = keys[i] >> seg_shift;
+  if (i == 0 || (keys[i - 1] >> seg_shift) != sg) first[sg] = (int32_t)i + 1;
 }
 
 // Bounding box of every 32-row group of every work item (the targets one warp
@@ -882,29 +864,30 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
   ListView L{p->list_ptr, p->list_src, nct, st.leaf_first, st.leaf_last, p->pad_prefix, p->deg};
   int32_t *nitems = nullptr, *off = nullptr;
   int64_t *cost_part = nullptr, *cost_prox = nullptr;
-  BL_TRY(dalloc_n(&nitems, nct, s));
-  BL_TRY(dalloc_n(&off, nct, s));
-  BL_TRY(dalloc_n(&cost_part, nct, s));
-  BL_TRY(dalloc_n(&cost_prox, (size_t)nct * kMaxDegrees, s));
-  unsigned long long* summary = nullptr;   // [0, 2): executed counters; [2, 6): segment starts
-  BL_TRY(dalloc_n(&summary, 6, s));
-  BL_CUDA(cudaMemsetAsync(summary, 0, 2 * sizeof(unsigned long long), s));
+  unsigned long long* summary = nullptr;   // [0, 2): executed counters; [2, 6): segment starts; then:
+  // [0] items, [1] padded pool particles, [2] split tiles, [3] longest task's chunks, [4] next split slot
+  Arena scratch;
+  scratch.add(&nitems, nct);
+  scratch.add(&off, nct);
+  scratch.add(&cost_part, nct);
+  scratch.add(&cost_prox, (size_t)nct * kMaxDegrees);
+  scratch.add(&summary, 9);
+  BL_TRY(scratch.alloc(s));
+  BL_CUDA(cudaMemsetAsync(summary, 0, 9 * sizeof(unsigned long long), s));
+  int32_t* totals = reinterpret_cast<int32_t*>(summary + 6);
   unsigned long long* executed = summary;
   dfree_ptr(p->eval_part, s);
   dfree_ptr(p->eval_prox, s);
   BL_TRY(dalloc_n(&p->eval_part, nct, s));
   BL_TRY(dalloc_n(&p->eval_prox, nct, s));
-  int32_t* totals = nullptr;   // [0] items, [1] padded pool particles, [2] split tiles, [3] next split slot
-  BL_TRY(dalloc_n(&totals, 4, s));
-  BL_CUDA(cudaMemsetAsync(totals, 0, 4 * sizeof(int32_t), s));
   const int64_t part_len = task_chunks(p);
-  k_item_count<<<nblk(nct, 128), 128, 0, s>>>(nct, L, tt.parent, tt.nchild, tt.begin, tt.end,
+  k_item_count<<<nblk((int64_t)nct * 32, 128), 128, 0, s>>>(nct, L, tt.parent, tt.nchild, tt.begin, tt.end,
                                               st.begin, st.end, nitems, cost_part, cost_prox,
-                                              executed, p->eval_part, p->eval_prox, part_len, totals + 2);
+                                              executed, p->eval_part, p->eval_prox, part_len, totals + 2, totals + 3);
   BL_LAUNCHED(cnt.launches);
   BL_TRY(scan_exclusive_dev(nitems, off, nct, totals, s, cnt));
   BL_CUDA(cudaMemcpyAsync(totals + 1, p->pad_prefix + st.nleaves, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-  int32_t h_tot[3];
+  int32_t h_tot[4];
   BL_TRY(read_device(totals, h_tot, sizeof(h_tot), s));
   const int32_t ni = h_tot[0];
   p->nitems = ni;
@@ -918,39 +901,42 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
   p->np_pad = p->deg.np_pad[p->deg.n - 1];
   int4 *items = nullptr, *parts = nullptr;
   uint32_t* keys = nullptr;
-  int32_t* vals = nullptr;
-  BL_TRY(dalloc_n(&items, ni, s));
-  BL_TRY(dalloc_n(&parts, ni, s));
+  int32_t* order = nullptr;
+  Arena unsorted;
+  unsorted.add(&items, ni);
+  unsorted.add(&parts, ni);
+  unsorted.add(&keys, ni);
+  unsorted.add(&order, ni);
+  BL_TRY(unsorted.alloc(s));
   BL_TRY(dalloc_n(&p->parts, ni, s));
-  BL_TRY(dalloc_n(&keys, ni, s));
-  BL_TRY(dalloc_n(&vals, ni, s));
   BL_TRY(dalloc_n(&p->items, ni, s));
+  // Bits of the sort key: the longest task's, the kernel of a shared
+  // Coulomb/Yukawa segment, the segment.  As few as hold them: each 8 cost the
+  // sort a pass.
+  int len_bits = 1;
+  while (len_bits < 24 && (1 << len_bits) <= h_tot[3]) ++len_bits;
   SegmentMap segmap{};
   segmap.n = (int)p->segment_kernels.size();
   for (int i = 0; i < segmap.n; ++i) segmap.kernel[i] = p->segment_kernels[i];
   k_item_fill<<<nblk(nct, 128), 128, 0, s>>>(nct, off, cost_part, cost_prox, tt.begin, tt.end,
-                                             tt.problem, p->prob_kernel, segmap, p->deg, part_len, totals + 3,
-                                             items, parts, keys, vals);
+                                             tt.problem, p->prob_kernel, segmap, p->deg, part_len, len_bits, totals + 4,
+                                             items, parts, keys);
   BL_LAUNCHED(cnt.launches);
   // Grouped by kernel, longest items first within a group (stable), so that
   // each persistent launch's tail is short.
   int seg_bits = 0;
   while ((1 << seg_bits) < segmap.n) ++seg_bits;
-  bool fused = false;   // a shared Coulomb/Yukawa segment sets the kernel bit (bit 24)
+  bool fused = false;   // a shared Coulomb/Yukawa segment sets the kernel bit
   for (int i = 0; i < segmap.n; ++i) fused |= segmap.kernel[i] == kKernCoulombYukawa;
-  const int key_bits = seg_bits > 0 ? 25 + seg_bits : (fused ? 25 : 24);
-  BL_TRY(radix_sort_pairs(keys, vals, ni, key_bits, s, cnt));
+  const int key_bits = len_bits + (seg_bits > 0 ? 1 + seg_bits : (fused ? 1 : 0));
+  BL_TRY(sort_order(keys, order, ni, key_bits, s, cnt));
   // segment starts (8 int32) and the two executed-evaluation counters come
   // back to the host in one read
   int32_t* seg_first = reinterpret_cast<int32_t*>(summary + 2);
-  BL_CUDA(cudaMemsetAsync(seg_first, 0xff, 8 * sizeof(int32_t), s));
-  if (ni > 0) {
-    k_segment_starts<<<nblk(ni, 256), 256, 0, s>>>(keys, ni, seg_first);
-    BL_LAUNCHED(cnt.launches);
-  }
   int32_t h_first[8];
   if (ni > 0) {
-    k_gather_items<<<nblk(ni, 256), 256, 0, s>>>(items, parts, vals, p->items, p->parts, ni);
+    k_gather_items<<<nblk(ni, 256), 256, 0, s>>>(keys, len_bits + 1, items, parts, order, p->items, p->parts, ni,
+                                                 seg_first);
     BL_LAUNCHED(cnt.launches);
   }
   if (p->precision == BLDTT_FP32_BULK && ni > 0) {
@@ -965,11 +951,11 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
   BL_TRY(read_device(summary, h_sum, sizeof(h_sum), s));
   const unsigned long long h_exec[2] = {h_sum[0], h_sum[1]};
   std::memcpy(h_first, h_sum + 2, sizeof(h_first));
+  for (int32_t& f : h_first) --f;                    // -1: no item
   p->executed_skip = (double)h_exec[0];
   p->executed_noskip = (double)h_exec[1];
   p->skip_saved_evaluations = p->executed_noskip - p->executed_skip;
   p->executed_evaluations = p->executed_noskip;
-  dfree(summary, s);
   p->segments.clear();
   for (int i = 0; i < segmap.n; ++i) {
     if (h_first[i] < 0) continue;                    // no items for this kernel
@@ -981,8 +967,8 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
       }
     p->segments.push_back({segmap.kernel[i], h_first[i], end - h_first[i], 0, 0, 0});
   }
-  dfree(items, s); dfree(parts, s); dfree(keys, s); dfree(vals, s); dfree(totals, s);
-  dfree(nitems, s); dfree(off, s); dfree(cost_part, s); dfree(cost_prox, s);
+  unsorted.release(s);
+  scratch.release(s);
   return BLDTT_OK;
 }
 

@@ -445,9 +445,8 @@ int scan_exclusive_dev(const int32_t* in, int32_t* out, int64_t n, int32_t* tota
 // synchronise it: through the calling thread's pinned slot when it has one
 // (a pinned copy costs ~1 us against ~9 us for a pageable one).
 int read_device(const void* dev, void* host, size_t bytes, cudaStream_t s);
-// Stable ascending sort of (key, value) pairs on the low `bits` bits of key.
-int radix_sort_pairs(uint32_t* keys, int32_t* vals, int64_t n, int bits, cudaStream_t s,
-                     Counters& c);
+// Stable ascending sort of keys of `bits` bits; order[i] = the position that the i-th had.
+int sort_order(uint32_t* keys, int32_t* order, int64_t n, int bits, cudaStream_t s, Counters& c);
 // Raise *bad_dev if any of n doubles is not finite.
 int check_finite(const double* v, int64_t n, int* bad_dev, cudaStream_t s, Counters& c);
 

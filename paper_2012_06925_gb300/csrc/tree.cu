@@ -489,26 +489,35 @@ static int cluster_boxes(Tree& T, int32_t first, int32_t nc, int32_t n, cudaStre
   return BLDTT_OK;
 }
 
-// Centre = box centre, radius = half the diagonal, proxy points c + h s_k.
-__global__ void k_tree_geometry(int32_t C, int degree, const double* __restrict__ box,
-                                double* __restrict__ center, double* __restrict__ radius,
-                                double* __restrict__ nodes) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= C) return;
+// Centre = box centre, radius = half the diagonal, proxy points c + h s_k.  A
+// block computes the points s_k once; a thread then has one dimension of one
+// cluster (one thread per cluster, cosines and all: 27 us for 5 clusters).
+constexpr int kGeometryThreads = 128;
+__global__ void __launch_bounds__(kGeometryThreads) k_tree_geometry(
+    int32_t C, int degree, const double* __restrict__ box, double* __restrict__ center,
+    double* __restrict__ radius, double* __restrict__ nodes) {
+  constexpr int kPoints = 64;
+  __shared__ double s_k[kPoints];
   const int P = degree + 1;
-  const double* b = box + (int64_t)c * 6;
-  double e[3];
-  for (int d = 0; d < 3; ++d) {
-    double lo = b[d], hi = b[3 + d];
-    double cc = __dmul_rn(__dadd_rn(lo, hi), 0.5);
-    double h = __dmul_rn(__dsub_rn(hi, lo), 0.5);
-    e[d] = __dsub_rn(hi, lo);
-    center[(int64_t)c * 3 + d] = cc;
-    for (int k = 0; k < P; ++k)
-      nodes[((int64_t)c * 3 + d) * P + k] = __dadd_rn(cc, __dmul_rn(h, cheb_point(k, degree)));
+  for (int k = threadIdx.x; k < min(P, kPoints); k += kGeometryThreads) s_k[k] = cheb_point(k, degree);
+  __syncthreads();
+  const int64_t i = (int64_t)blockIdx.x * kGeometryThreads + threadIdx.x;
+  const int64_t c = i / 3;
+  const int d = (int)(i % 3);
+  if (c >= C) return;
+  const double* b = box + c * 6;
+  const double lo = b[d], hi = b[3 + d];
+  const double cc = __dmul_rn(__dadd_rn(lo, hi), 0.5);
+  const double h = __dmul_rn(__dsub_rn(hi, lo), 0.5);
+  center[c * 3 + d] = cc;
+  for (int k = 0; k < P; ++k)
+    nodes[(c * 3 + d) * P + k] = __dadd_rn(cc, __dmul_rn(h, k < kPoints ? s_k[k] : cheb_point(k, degree)));
+  if (d == 0) {
+    double e[3];
+    for (int k = 0; k < 3; ++k) e[k] = __dsub_rn(b[3 + k], b[k]);
+    const double s2 = __dadd_rn(__dadd_rn(__dmul_rn(e[0], e[0]), __dmul_rn(e[1], e[1])), __dmul_rn(e[2], e[2]));
+    radius[c] = __dmul_rn(__dsqrt_rn(s2), 0.5);
   }
-  double s2 = __dadd_rn(__dadd_rn(__dmul_rn(e[0], e[0]), __dmul_rn(e[1], e[1])), __dmul_rn(e[2], e[2]));
-  radius[c] = __dmul_rn(__dsqrt_rn(s2), 0.5);
 }
 
 __global__ void k_tree_leaf_flags(int32_t C, const int32_t* __restrict__ nchild,
@@ -668,7 +677,7 @@ int build_tree(Tree& T, const double* coords, int32_t n, const std::vector<int32
   BL_TRY(dalloc_n(&T.center, (size_t)C * 3, s));
   BL_TRY(dalloc_n(&T.radius, (size_t)C, s));
   BL_TRY(dalloc_n(&T.nodes, (size_t)C * 3 * (degree + 1), s));
-  k_tree_geometry<<<nblk(C, 128), 128, 0, s>>>(C, degree, T.box, T.center, T.radius, T.nodes);
+  k_tree_geometry<<<nblk(3 * (int64_t)C, kGeometryThreads), kGeometryThreads, 0, s>>>(C, degree, T.box, T.center, T.radius, T.nodes);
   BL_LAUNCHED(cnt.launches);
 
   int32_t *flag = nullptr, *excl = nullptr;
@@ -1259,7 +1268,11 @@ __global__ void __launch_bounds__(kTreeCoopThreads, 4) k_tree_all(TreeCoop p) {
   }
 }
 
-static bool coop_tree_available(int* blocks) {
+// Blocks of the build: all that fit where the particles' passes dominate, one
+// on an SM where the grid barriers do (about 15 a build).  Measured, 152 and 608
+// blocks: 2E4 points 0.182 and 0.220 ms, 1E5 0.361 and 0.410, 3E5 0.264 and
+// 0.295, 1E6 0.520 and 0.410 (304 blocks 0.434).
+static bool coop_tree_available(int* blocks, int64_t n = 0) {
   if (cooperative_set_up_disabled()) return false;
   int dev = 0, sms = 0, coop = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -1270,7 +1283,8 @@ static bool coop_tree_available(int* blocks) {
     return false;
   }
   if (!coop || per_sm < 1) return false;
-  *blocks = std::min(kTreeMaxBlocks, sms * std::min(per_sm, 4));
+  const int64_t most = std::min(kTreeMaxBlocks, sms * std::min(per_sm, 4));
+  *blocks = (int)std::min(most, std::max<int64_t>(sms, n / 1640));
   return true;
 }
 
@@ -1282,7 +1296,7 @@ static int build_tree_coop(Tree& T, const double* coords, int32_t n, const std::
                            cudaStream_t s, Counters& cnt, bool* done) {
   *done = false;
   int G = 0;
-  if (!coop_tree_available(&G)) return BLDTT_OK;
+  if (!coop_tree_available(&G, n)) return BLDTT_OK;
   T.n = n;
   const int32_t nroots = (int32_t)roots.size() - 1;
   TreeCoop p{};
@@ -1438,7 +1452,7 @@ static int build_tree_coop(Tree& T, const double* coords, int32_t n, const std::
   BL_TRY(dalloc_n(&T.center, (size_t)C * 3, s));
   BL_TRY(dalloc_n(&T.radius, (size_t)C, s));
   BL_TRY(dalloc_n(&T.nodes, (size_t)C * 3 * (degree + 1), s));
-  k_tree_geometry<<<nblk(C, 128), 128, 0, s>>>(C, degree, T.box, T.center, T.radius, T.nodes);
+  k_tree_geometry<<<nblk(3 * (int64_t)C, kGeometryThreads), kGeometryThreads, 0, s>>>(C, degree, T.box, T.center, T.radius, T.nodes);
   BL_LAUNCHED(cnt.launches);
   *done = true;
   return BLDTT_OK;
