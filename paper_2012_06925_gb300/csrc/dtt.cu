@@ -330,16 +330,24 @@ __global__ void k_lists(const uint32_t* __restrict__ key, const int32_t* __restr
   if (threadIdx.x < kMaxClasses) part[threadIdx.x] = 0ull;
   __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int c = -1;
+  unsigned long long v = 0;
   if (i < n) {
     const int32_t o = order[i], t = ent_t[o], s = ent_s[o];
     list_tgt[i] = t;
     list_src[i] = s;
-    const int c = (int)(key[i] / (uint32_t)nct);
+    c = (int)(key[i] / (uint32_t)nct);
     const int type = class_type(c);
     const int64_t np = deg.np[class_degree(c)];
     const int64_t ct = tt.end[t] - tt.begin[t], cs = st.end[s] - st.begin[s];
-    const int64_t v = type == BLDTT_PP ? ct * cs : type == BLDTT_PC ? ct * np : type == BLDTT_CP ? np * cs : np * np;
-    atomicAdd(&part[c], (unsigned long long)v);
+    v = (unsigned long long)(type == BLDTT_PP ? ct * cs : type == BLDTT_PC ? ct * np : type == BLDTT_CP ? np * cs : np * np);
+  }
+  // the keys are sorted: most warps have one class, and one atomic
+  if (__all_sync(0xffffffffu, c == __shfl_sync(0xffffffffu, c, 0))) {
+    for (int w = 16; w; w >>= 1) v += __shfl_xor_sync(0xffffffffu, v, w);
+    if ((threadIdx.x & 31) == 0 && c >= 0) atomicAdd(&part[c], v);
+  } else if (c >= 0) {
+    atomicAdd(&part[c], v);
   }
   if (i <= (int64_t)nclass * nct) {
     int64_t lo = 0, hi = n;

@@ -227,37 +227,67 @@ int scan_exclusive_dev(const int32_t* in, int32_t* out, int64_t n, int32_t* tota
 // inputs, LSD radix passes of 8-bit digits (three or more launches each) above
 // ---------------------------------------------------------------------------
 // Short inputs are bound by launches, not by work: 9 launches of about 2.5 us
-// for 24-bit keys against one of 4 us (4096 pairs).  The network's elements
-// are key << 32 | position: unique, so its order is the stable one.  Strides of
-// up to 32 stay within the 64 elements of a warp's 32 pairs and need no block
-// barrier (21 of the 78 steps do at 4096).
+// for 24-bit keys against one of 19 us (4096 pairs, ncu; 4 us at 1000).  The network's elements
+// are key << 32 | position: unique, so its order is the stable one.  A thread
+// holds 4 neighbouring elements in registers; strides of up to 2 stay in the
+// thread, up to 64 in the warp (shuffles), and the 15 longer ones of 78 steps at
+// 4096 go through shared memory (with all of them there: 33 us).
 constexpr int kSmallSort = 4096;
-constexpr int kSmallSortThreads = 1024;
+constexpr int kSmallSortThreads = kSmallSort / 4;
+
+__device__ __forceinline__ void order_pair(unsigned long long& a, unsigned long long& b, bool up) {
+  const bool swap = (a > b) == up;
+  const unsigned long long lo = swap ? b : a, hi = swap ? a : b;
+  a = lo;
+  b = hi;
+}
 
 __global__ void __launch_bounds__(kSmallSortThreads) k_sort_small(uint32_t* __restrict__ keys,
                                                                   int32_t* __restrict__ order, int n, int size) {
   __shared__ unsigned long long sk[kSmallSort];
-  for (int i = threadIdx.x; i < size; i += kSmallSortThreads)
-    sk[i] = i < n ? (unsigned long long)keys[i] << 32 | (unsigned)i : ~0ull;
-  __syncthreads();
+  const int i0 = 4 * threadIdx.x;
+  unsigned long long v[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    v[r] = i0 + r < n ? (unsigned long long)keys[i0 + r] << 32 | (unsigned)(i0 + r) : ~0ull;
   for (int k = 2; k <= size; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int t = threadIdx.x; t < size / 2; t += kSmallSortThreads) {
-        const int i = 2 * t - (t & (j - 1));
-        const unsigned long long a = sk[i], b = sk[i + j];
-        if ((a > b) == ((i & k) == 0)) {
-          sk[i] = b;
-          sk[i + j] = a;
-        }
+    for (int j = k >> 1; j > 64; j >>= 1) {
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < 4; ++r) sk[r * kSmallSortThreads + threadIdx.x] = v[r];
+      __syncthreads();
+      const bool low = (i0 & j) == 0, up = (i0 & k) == 0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const unsigned long long w = sk[r * kSmallSortThreads + (threadIdx.x ^ (j / 4))];
+        v[r] = ((v[r] < w) == (low == up)) ? v[r] : w;
       }
-      if (j > 32 || (j == 1 && k >= 64)) __syncthreads(); else __syncwarp();   // the next step's stride is j/2, or k
+    }
+    for (int j = min(k >> 1, 64); j > 2; j >>= 1) {
+      const bool low = (i0 & j) == 0, up = (i0 & k) == 0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const unsigned long long w = __shfl_xor_sync(0xffffffffu, v[r], j / 4);
+        v[r] = ((v[r] < w) == (low == up)) ? v[r] : w;
+      }
+    }
+    if (k > 2) {
+      const bool up = (i0 & k) == 0;
+      order_pair(v[0], v[2], up);
+      order_pair(v[1], v[3], up);
+      order_pair(v[0], v[1], up);
+      order_pair(v[2], v[3], up);
+    } else {
+      order_pair(v[0], v[1], true);
+      order_pair(v[2], v[3], false);
     }
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += kSmallSortThreads) {
-    keys[i] = (uint32_t)(sk[i] >> 32);
-    order[i] = (int32_t)(sk[i] & 0xffffffffu);
-  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    if (i0 + r < n) {
+      keys[i0 + r] = (uint32_t)(v[r] >> 32);
+      order[i0 + r] = (int32_t)(v[r] & 0xffffffffu);
+    }
 }
 
 constexpr int kRadixBits = 8;
@@ -321,9 +351,10 @@ __global__ void k_radix_scatter(const uint32_t* __restrict__ kin, const int32_t*
 int sort_order(uint32_t* keys, int32_t* order, int64_t n, int bits, cudaStream_t s, Counters& c) {
   if (n <= 0) return BLDTT_OK;
   if (n <= kSmallSort) {
-    int size = 2;
+    int size = 4;
     while (size < n) size *= 2;
-    k_sort_small<<<1, kSmallSortThreads, 0, s>>>(keys, order, (int)n, size);
+    const int threads = std::max(32, size / 4);
+    k_sort_small<<<1, threads, 0, s>>>(keys, order, (int)n, size);
     BL_LAUNCHED(c.launches);
     return BLDTT_OK;
   }
