@@ -123,6 +123,7 @@ void release(bldtt_plan* p) {
   dfree_ptr(p->prob_kappa, s);
   dfree_ptr(p->prob_prm, s);
   for (int i = 0; i + 1 < p->deg.n; ++i) {   // the highest degree aliases the tree/plan arrays
+    if (p->nodes_s[i] == p->nodes_t[i]) p->nodes_s[i] = nullptr;   // one tree for both
     dfree_ptr(p->nodes_t[i], s);
     dfree_ptr(p->nodes_s[i], s);
     dfree_ptr(p->qhat_d[i], s);
@@ -333,7 +334,8 @@ const char* bldtt_status_string(int status) {
 const char* bldtt_last_error(void) { return bldtt::last_error(); }
 
 // Selector weights: float master weights (W1 b1 W2 b2 W3 b3 W4 b4, rows =
-// outputs) -> bf16 weights (round to nearest even) and float biases.
+// outputs) -> bf16 weights (round to nearest even), each layer transposed to
+// [in][out] as the inference reads them, and float biases.
 static uint16_t host_bf16(float x) {
   uint32_t u;
   std::memcpy(&u, &x, 4);
@@ -348,12 +350,14 @@ static int upload_selector(bldtt_plan* p, const float* weights) {
   std::vector<float> b;
   size_t o = 0;
   for (int l = 0; l < 4; ++l) {
+    const size_t base = w.size();
+    w.resize(base + (size_t)in[l] * out[l]);
     for (int i = 0; i < in[l] * out[l]; ++i) {
       if (!std::isfinite(weights[o + i])) {
         set_error("selector weight %zu is not finite", o + i);
         return BLDTT_EINVAL;
       }
-      w.push_back(host_bf16(weights[o + i]));
+      w[base + (size_t)(i % in[l]) * out[l] + i / in[l]] = host_bf16(weights[o + i]);
     }
     o += (size_t)in[l] * out[l];
     for (int i = 0; i < out[l]; ++i) b.push_back(weights[o + i]);

@@ -303,6 +303,7 @@ struct bldtt_plan {
   std::vector<int> prob_kernel_h;     // host copies
   std::vector<double> prob_kappa_h;
   std::vector<float> prob_prm_h;      // host copy of prob_prm
+  std::vector<double> xfer_h[bldtt::kMaxDegrees];   // degree-change matrices as copied to xfer
   int* prob_kernel = nullptr;         // device [nprob]
   double* prob_kappa = nullptr;       // device [nprob]
   float* prob_prm = nullptr;          // device [nprob] FP32 form of the parameter
@@ -330,7 +331,7 @@ struct bldtt_plan {
   // biases, the training box of the features and the per-pair budget.
   bool learned = false;
   bool selector_net = false;          // false: the MAC fallback decides every pair
-  void* sel_w = nullptr;              // __nv_bfloat16 [64*6 + 64*64*2 + nout*64]
+  void* sel_w = nullptr;              // __nv_bfloat16 [64*6 + 64*64*2 + nout*64], [in][out] per layer
   float* sel_b = nullptr;             // [64*3 + nout]
   int sel_nout = 0;
   float sel_lo[bldtt::kFeatures] = {}, sel_hi[bldtt::kFeatures] = {};

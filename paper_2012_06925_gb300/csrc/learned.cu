@@ -132,22 +132,64 @@ __device__ float mlp_forward_warp(const NetSmem& net, const float* x, float* act
   return lane < net.nout ? neuron(W, b, lane, kHidden, net.nout, in) : 0.f;
 }
 
-// Load bf16 weights (row-major [out][in] in global memory, transposed to
-// [in][out] in shared memory) and float biases.
-__device__ void load_net(const __nv_bfloat16* gw, const float* gb, int nout, __nv_bfloat16* sw, float* sb) {
-  const int K[4] = {kFeatures, kHidden, kHidden, kHidden};
-  const int J[4] = {kHidden, kHidden, kHidden, nout};
-  int64_t o = 0;
-  for (int l = 0; l < 4; ++l) {
-    const int64_t n = (int64_t)K[l] * J[l];
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-      const int64_t j = i / K[l], k = i % K[l];
-      sw[o + k * J[l] + j] = gw[o + i];
+// The same network for kSelTogether inputs x[m] at once (the sums in the same
+// order): a neuron's sum is a chain of dependent multiply-adds, so one input at
+// a time left the warp waiting, 3.8 us each.  act: 2 x 64 x kSelTogether floats.
+constexpr int kSelTogether = 4;
+__device__ __forceinline__ void mlp_forward_together(const NetSmem& net, const float* const (&x)[kSelTogether],
+                                                     float* act, float (&y)[kSelTogether]) {
+  constexpr int M = kSelTogether;
+  const int lane = threadIdx.x & 31;
+  const __nv_bfloat16* W = net.w;
+  const float* b = net.b;
+  float4* bufs[2] = {reinterpret_cast<float4*>(act), reinterpret_cast<float4*>(act + kHidden * M)};
+  if (lane < kFeatures) bufs[1][lane] = make_float4(x[0][lane], x[1][lane], x[2][lane], x[3][lane]);
+  __syncwarp();
+  for (int l = 0; l < 3; ++l) {
+    const int K = l == 0 ? kFeatures : kHidden;
+    const float4* in = bufs[(l + 1) & 1];
+    float z[2][M];
+    for (int h = 0; h < 2; ++h)
+      for (int m = 0; m < M; ++m) z[h][m] = b[lane + 32 * h];
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+      const float4 a = in[k];
+      const float am[M] = {a.x, a.y, a.z, a.w};
+      for (int h = 0; h < 2; ++h) {
+        const float w = __bfloat162float(W[(int64_t)k * kHidden + lane + 32 * h]);
+        for (int m = 0; m < M; ++m) z[h][m] = fmaf(w, am[m], z[h][m]);
+      }
     }
-    o += n;
+    for (int h = 0; h < 2; ++h) {
+      for (int m = 0; m < M; ++m) z[h][m] = bf16r(z[h][m] > 0.f ? z[h][m] : 0.f);
+      bufs[l & 1][lane + 32 * h] = make_float4(z[h][0], z[h][1], z[h][2], z[h][3]);
+    }
+    __syncwarp();
+    W += (int64_t)kHidden * K;
+    b += kHidden;
   }
-  const int64_t nb = sel_bias_count(nout);
-  for (int64_t i = threadIdx.x; i < nb; i += blockDim.x) sb[i] = gb[i];
+  for (int m = 0; m < M; ++m) y[m] = 0.f;
+  if (lane < net.nout) {
+    const float4* in = bufs[0];
+    for (int m = 0; m < M; ++m) y[m] = b[lane];
+#pragma unroll 4
+    for (int k = 0; k < kHidden; ++k) {
+      const float4 a = in[k];
+      const float am[M] = {a.x, a.y, a.z, a.w};
+      const float w = __bfloat162float(W[(int64_t)k * net.nout + lane]);
+      for (int m = 0; m < M; ++m) y[m] = fmaf(w, am[m], y[m]);
+    }
+  }
+  __syncwarp();
+}
+
+// Load bf16 weights ([in][out] per layer) and float biases.
+__device__ void load_net(const __nv_bfloat16* gw, const float* gb, int nout, __nv_bfloat16* sw, float* sb) {
+  static_assert(kHidden % 8 == 0, "the weights of every layer are whole 16-byte words");
+  const int nw = (int)(sel_weight_count(nout) / 8), nb = (int)sel_bias_count(nout);
+  for (int i = threadIdx.x; i < nw; i += blockDim.x)
+    reinterpret_cast<uint4*>(sw)[i] = reinterpret_cast<const uint4*>(gw)[i];
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) sb[i] = gb[i];
   __syncthreads();
 }
 
@@ -161,39 +203,42 @@ struct SelParams {
   int net;   // 0: no network (MAC fallback everywhere)
 };
 
-// Per-warp scratch of k_select: the MLP's activations, then the inputs and
+// Per-warp scratch of k_select: the networks' activations, then the inputs and
 // outputs of the warp's 32 pairs.
 constexpr int kSelOutMax = 3 * kMaxDegrees;
-constexpr int kSelWarpFloats = 2 * kHidden + 32 * 8 + 32 * kSelOutMax;
+constexpr int kSelActFloats = 2 * kHidden * kSelTogether;
+constexpr int kSelWarpFloats = kSelActFloats + 32 * 8 + 32 * kSelOutMax;
 
 __host__ __device__ inline size_t select_smem_bytes(int nout) {
   size_t w = (size_t)sel_weight_count(nout) * sizeof(__nv_bfloat16);
   w = (w + 15) / 16 * 16;
-  return w + (size_t)sel_bias_count(nout) * sizeof(float) +
+  return w + (size_t)(sel_bias_count(nout) + 3) / 4 * 4 * sizeof(float) +
          (size_t)kSelWarps * kSelWarpFloats * sizeof(float);
 }
 
-// A warp takes 32 pairs at a time: each lane computes its pair's features (the
-// FP64 divisions and square root run on all lanes at once), the warp runs the
-// network for every pair inside the box in turn, and each lane decides its own
-// pair.  Same arithmetic as one pair per warp.
+// A warp takes `per_warp` pairs at a time (32 at most): each lane computes its
+// pair's features (the FP64 divisions and square root run on all lanes at once),
+// the warp runs the network for the pairs inside the box, kSelTogether at a
+// time, and each lane decides its own pair.  Same arithmetic as one pair per
+// warp.  Bound by latency: a front of a few thousand pairs, 32 to a warp on a
+// few SMs, took 0.14 ms; spread over all SMs, 4 networks at a time, 0.017 (50000 pairs 0.21 -> 0.06).
 __global__ void k_select(const int2* __restrict__ pairs, int32_t F, PairTrees T, SelParams sp,
-                         const __nv_bfloat16* __restrict__ gw, const float* __restrict__ gb,
+                         const __nv_bfloat16* __restrict__ gw, const float* __restrict__ gb, int per_warp,
                          int16_t* __restrict__ choice) {
   extern __shared__ __align__(16) unsigned char sraw[];
   __nv_bfloat16* sw = reinterpret_cast<__nv_bfloat16*>(sraw);
   size_t wbytes = ((size_t)sel_weight_count(sp.nout) * sizeof(__nv_bfloat16) + 15) / 16 * 16;
   float* sb = reinterpret_cast<float*>(sraw + wbytes);
-  float* swarp = sb + sel_bias_count(sp.nout);
+  float* swarp = sb + (sel_bias_count(sp.nout) + 3) / 4 * 4;   // 16-byte aligned
   if (sp.net) load_net(gw, gb, sp.nout, sw, sb);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* act = swarp + warp * kSelWarpFloats;
-  float* xs = act + 2 * kHidden;      // [32][8]
+  float* xs = act + kSelActFloats;    // [32][8]
   float* ys = xs + 32 * 8;            // [32][kSelOutMax]
   const NetSmem net{sw, sb, sp.nout};
-  const int64_t stride = (int64_t)gridDim.x * kSelWarps * 32;
-  for (int64_t base = ((int64_t)blockIdx.x * kSelWarps + warp) * 32; base < F; base += stride) {
-    const int64_t i = base + lane;
+  const int64_t stride = (int64_t)gridDim.x * kSelWarps * per_warp;
+  for (int64_t base = ((int64_t)blockIdx.x * kSelWarps + warp) * per_warp; base < F; base += stride) {
+    const int64_t i = lane < per_warp ? base + lane : F;
     int state = 0;   // 0 no approximation, 1 fallback, 2 network
     int t = 0, s = 0;
     if (i < F) {
@@ -212,10 +257,17 @@ __global__ void k_select(const int2* __restrict__ pairs, int32_t F, PairTrees T,
     __syncwarp();
     unsigned todo = __ballot_sync(0xffffffffu, state == 2);
     while (todo) {
-      const int j = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const float y = mlp_forward_warp(net, xs + j * 8, act, nullptr);
-      if (lane < sp.nout) ys[j * kSelOutMax + lane] = y;
+      int j[kSelTogether];
+      const float* x[kSelTogether];
+      float y[kSelTogether];
+      for (int m = 0; m < kSelTogether; ++m) {       // the last round repeats its last pair
+        j[m] = todo ? __ffs(todo) - 1 : j[m > 0 ? m - 1 : 0];
+        todo &= todo - 1;
+        x[m] = xs + j[m] * 8;
+      }
+      mlp_forward_together(net, x, act, y);
+      if (lane < sp.nout)
+        for (int m = 0; m < kSelTogether; ++m) ys[j[m] * kSelOutMax + lane] = y[m];
       __syncwarp();
     }
     if (i < F) {
@@ -263,11 +315,15 @@ int select_pairs(bldtt_plan* p, const int2* pairs, int32_t F, int16_t* choice, c
   sp.net = p->selector_net ? 1 : 0;
   const size_t sm = select_smem_bytes(p->sel_nout);
   BL_CUDA(cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  unsigned g = nblk(F, kSelWarps * 32);
+  int sms = 0;
+  BL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
+  const int64_t spread = (F + (int64_t)sms * 2 * kSelWarps - 1) / ((int64_t)sms * 2 * kSelWarps);
+  const int per_warp = (int)std::min<int64_t>(32, (spread + kSelTogether - 1) / kSelTogether * kSelTogether);
+  unsigned g = nblk(F, kSelWarps * per_warp);
   if (g > 4096) g = 4096;
   k_select<<<g, 32 * kSelWarps, sm, s>>>(pairs, F, pair_trees(p), sp,
                                           reinterpret_cast<const __nv_bfloat16*>(p->sel_w), p->sel_b,
-                                          choice);
+                                          per_warp, choice);
   BL_LAUNCHED(p->setup_counter.launches);
   return BLDTT_OK;
 }

@@ -496,10 +496,9 @@ constexpr int kGeometryThreads = 128;
 __global__ void __launch_bounds__(kGeometryThreads) k_tree_geometry(
     int32_t C, int degree, const double* __restrict__ box, double* __restrict__ center,
     double* __restrict__ radius, double* __restrict__ nodes) {
-  constexpr int kPoints = 64;
-  __shared__ double s_k[kPoints];
+  __shared__ double s_k[kMaxP];
   const int P = degree + 1;
-  for (int k = threadIdx.x; k < min(P, kPoints); k += kGeometryThreads) s_k[k] = cheb_point(k, degree);
+  for (int k = threadIdx.x; k < P; k += kGeometryThreads) s_k[k] = cheb_point(k, degree);
   __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * kGeometryThreads + threadIdx.x;
   const int64_t c = i / 3;
@@ -511,7 +510,7 @@ __global__ void __launch_bounds__(kGeometryThreads) k_tree_geometry(
   const double h = __dmul_rn(__dsub_rn(hi, lo), 0.5);
   center[c * 3 + d] = cc;
   for (int k = 0; k < P; ++k)
-    nodes[(c * 3 + d) * P + k] = __dadd_rn(cc, __dmul_rn(h, k < kPoints ? s_k[k] : cheb_point(k, degree)));
+    nodes[(c * 3 + d) * P + k] = __dadd_rn(cc, __dmul_rn(h, s_k[k]));
   if (d == 0) {
     double e[3];
     for (int k = 0; k < 3; ++k) e[k] = __dsub_rn(b[3 + k], b[k]);
