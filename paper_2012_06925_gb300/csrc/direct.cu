@@ -4,9 +4,11 @@
 // and the splits are summed in order.  Pairs at distance 0 contribute nothing.
 // Each tile of 256 sources has its own sum, so the sum's rounding grows with
 // the tile's length and the number of tiles, not with the number of sources.
-// Bound by the FP64 pipe (1.7 lanes per clock and SM): 12 instructions an
-// evaluation in FP64, 4 with G in integer arithmetic; Coulomb, 2000 targets x
-// 1E6 sources: 48.3 -> 15.3 ms.
+// In FP64 the pipe (1.7 lanes per clock and SM) bounds the sum at 12
+// instructions an evaluation; with G in integer arithmetic (fixed64.cuh) at 4,
+// the differences among them; with the coordinates in fixed point at 1, where
+// the integer pipe bounds it.  Coulomb, 2000 targets x 1E6 sources: 48.3, 15.3
+// and 9.9 ms.
 #include <float.h>
 
 #include "fixed64.cuh"
@@ -16,13 +18,48 @@ namespace bldtt {
 
 constexpr int kDirectThreads = 256;
 
-// FIXED: G in integer arithmetic (fixed64.cuh).  It wants a finite kappa >= 0,
-// as plans do; the direct sum takes any, and evaluates the others in FP64.
-template <int KERN, bool FIXED>
+// Extent of the coordinates of both sets, by dimension: key[d] and key[3 + d]
+// are the largest order-preserving keys of v and -v (0 before the first).
+__device__ __forceinline__ unsigned long long order_key(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  return b >> 63 ? ~b : b | 0x8000000000000000ull;
+}
+__device__ __forceinline__ double order_value(unsigned long long k) {
+  return __longlong_as_double((long long)(k >> 63 ? k & 0x7fffffffffffffffull : ~k));
+}
+__global__ void __launch_bounds__(kDirectThreads) k_extent(const double* __restrict__ t, int64_t M,
+                                                           const double* __restrict__ src, int64_t N,
+                                                           unsigned long long* __restrict__ key) {
+  const int d = blockIdx.y;
+  unsigned long long hi = 0, lo = 0;
+  for (int64_t i = (int64_t)blockIdx.x * kDirectThreads + threadIdx.x; i < M + N;
+       i += (int64_t)gridDim.x * kDirectThreads) {
+    const double v = i < M ? t[d * M + i] : src[d * N + i - M];
+    hi = max(hi, order_key(v));
+    lo = max(lo, order_key(-v));
+  }
+  for (int o = 16; o; o >>= 1) {
+    hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    lo = max(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(key + d, hi);
+    atomicMax(key + 3 + d, lo);
+  }
+}
+
+// Form of G: FP64 expressions; integer arithmetic on FP64 differences, for a
+// finite kappa >= 0 (the direct sum takes any); the same on coordinates in fixed
+// point, in units of the two sets' common extent (key), with FP64 differences
+// for pairs closer than 1/64 of it, and for all if the extent is 0 or not finite.
+enum DirectForm { kFormFp64, kFormFixed, kFormFixedCoords };
+
+template <int KERN, int FORM>
 __global__ void __launch_bounds__(kDirectThreads) k_direct(const double* __restrict__ t, int64_t M,
                                                            const double* __restrict__ src, int64_t N,
                                                            const double* __restrict__ q, double kappa,
-                                                           int64_t span, double* __restrict__ part) {
+                                                           int64_t span, const unsigned long long* __restrict__ key,
+                                                           double* __restrict__ part) {
   // blockIdx.y takes sources [y * span, min(N, (y + 1) * span)); part[y][i]
   __shared__ double4 tile[kDirectThreads];
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -33,20 +70,56 @@ __global__ void __launch_bounds__(kDirectThreads) k_direct(const double* __restr
     z = t[2 * M + i];
   }
   const int64_t s0 = (int64_t)blockIdx.y * span, s1 = min(N, s0 + span);
-  const fixed64::Screen screen = FIXED && KERN == BLDTT_YUKAWA ? fixed64::make_screen(kappa) : fixed64::Screen{0, 0};
+  __shared__ long long fx[FORM == kFormFixedCoords ? kDirectThreads : 1], fy[FORM == kFormFixedCoords ? kDirectThreads : 1],
+      fz[FORM == kFormFixedCoords ? kDirectThreads : 1];
+  int k2 = 0;                                       // unit 2^-k2
+  uint32_t top_min = ~0u;
+  long long X = 0, Y = 0, Z = 0;
+  if (FORM == kFormFixedCoords) {
+    double w = 0.0;
+    for (int d = 0; d < 3; ++d) w = fmax(w, order_value(key[d]) + order_value(key[3 + d]));
+    bool ok = true;
+    for (int d = 0; d < 3; ++d) ok = ok && order_value(key[d]) <= DBL_MAX && order_value(key[3 + d]) <= DBL_MAX;
+    if (ok && w >= 0x1p-900 && w <= 0x1p900) {
+      k2 = 61 - ilogb(w);                           // w < 2^(62 - k2)
+      top_min = fixed64::kFixedTop;
+    }
+    X = fixed64::to_fixed(x, k2);
+    Y = fixed64::to_fixed(y, k2);
+    Z = fixed64::to_fixed(z, k2);
+  }
+  const fixed64::Screen screen = FORM != kFormFp64 && KERN == BLDTT_YUKAWA ? fixed64::make_screen(kappa) : fixed64::Screen{0, 0};
   double acc = 0.0;
   for (int64_t base = s0; base < s1; base += kDirectThreads) {
     int64_t j = base + threadIdx.x;
     tile[threadIdx.x] = j < s1 ? make_double4(src[j], src[N + j], src[2 * N + j], q[j])
                                : make_double4(0, 0, 0, 0);
+    if (FORM == kFormFixedCoords) {
+      const double4 p = tile[threadIdx.x];
+      fx[threadIdx.x] = fixed64::to_fixed(p.x, k2);
+      fy[threadIdx.x] = fixed64::to_fixed(p.y, k2);
+      fz[threadIdx.x] = fixed64::to_fixed(p.z, k2);
+    }
     __syncthreads();
     int cnt = (int)min((int64_t)kDirectThreads, s1 - base);
     double a = 0.0;
+#pragma unroll 2
     for (int k = 0; k < cnt; ++k) {
-      double4 p = tile[k];
-      double dx = x - p.x, dy = y - p.y, dz = z - p.z;
       double g = 0.0;
-      if (FIXED) {
+      if (FORM == kFormFixedCoords) {
+        const long long ux = X - fx[k], uy = Y - fy[k], uz = Z - fz[k];
+        const uint32_t top = fixed64::fixed_top(ux, uy, uz);
+        if (top >= top_min) {
+          int E;
+          const fixed64::u64 S = fixed64::sum_squares_fixed(ux, uy, uz, top, k2, &E);
+          g = KERN == BLDTT_COULOMB ? fixed64::inv_r_of(S, E) : fixed64::screened_inv_r_of(S, E, screen);
+          a = fma(g, tile[k].w, a);
+          continue;
+        }
+      }
+      const double4 p = tile[k];
+      const double dx = x - p.x, dy = y - p.y, dz = z - p.z;
+      if (FORM != kFormFp64) {
         g = KERN == BLDTT_COULOMB  ? fixed64::inv_r(dx, dy, dz)
             : KERN == BLDTT_YUKAWA ? fixed64::screened_inv_r(dx, dy, dz, screen)
                                    : fixed64::inv_sqrt_r2_kappa2(dx, dy, dz, kappa);
@@ -72,30 +145,39 @@ __global__ void __launch_bounds__(kDirectThreads) k_direct(const double* __restr
   if (i < M) part[(int64_t)blockIdx.y * M + i] = acc;
 }
 
-// phi[i] = sum over the source splits, in split order, with each addition's
-// rounding error (Knuth's two-sum) added at the end: hundreds of splits one
-// after the other were most of the sum's error.
-__global__ void k_direct_reduce(const double* __restrict__ part, int64_t M, int splits,
-                                double* __restrict__ phi) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= M) return;
+// phi[i] = sum over the source splits, with each addition's rounding error
+// (Knuth's two-sum) added at the end: hundreds of splits one after the other were
+// most of the sum's error.  One warp per target, in an order fixed by the number
+// of splits (a thread per target: 0.16 ms for 500 targets).
+__device__ __forceinline__ void add_split(double& a, double& err, double b) {
+  const double t = a + b, w = t - a;
+  err += (a - (t - w)) + (b - w);
+  a = t;
+}
+__global__ void __launch_bounds__(kDirectThreads) k_direct_reduce(const double* __restrict__ part, int64_t M,
+                                                                  int splits, double* __restrict__ phi) {
+  const int64_t i = ((int64_t)blockIdx.x * kDirectThreads + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (i >= M) return;                               // whole warps
   double a = 0.0, err = 0.0;
-  for (int k = 0; k < splits; ++k) {
-    const double b = part[(int64_t)k * M + i], t = a + b, w = t - a;
-    err += (a - (t - w)) + (b - w);
-    a = t;
+  for (int k = lane; k < splits; k += 32) add_split(a, err, part[(int64_t)k * M + i]);
+  for (int o = 16; o; o >>= 1) {
+    const double b = __shfl_down_sync(0xffffffffu, a, o), e = __shfl_down_sync(0xffffffffu, err, o);
+    add_split(a, err, b);
+    err += e;
   }
-  phi[i] = err - err == 0.0 ? a + err : a;      // infinite sums have no error term
+  if (lane == 0) phi[i] = err - err == 0.0 ? a + err : a;   // infinite sums have no error term
 }
 
 int direct_sum(const double* targets, int64_t M, const double* sources, int64_t N,
                const double* charges, int kernel, double kappa, double* phi, cudaStream_t s) {
   const unsigned blocks = (unsigned)((M + kDirectThreads - 1) / kDirectThreads);
-  // Split the sources so that the grid fills the device (few targets, many sources).
+  // Split the sources so that the grid fills the device (few targets, many
+  // sources): eight CTAs to an SM (with four 2E4 x 2E5 takes 24.6 ms, with eight 21.5).
   int dev = 0, sms = 0;
   BL_CUDA(cudaGetDevice(&dev));
   BL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  int64_t splits = ((int64_t)4 * sms + blocks - 1) / blocks;
+  int64_t splits = ((int64_t)8 * sms + blocks - 1) / blocks;
   const int64_t max_splits = (N + kDirectThreads - 1) / kDirectThreads;
   if (splits > max_splits) splits = max_splits;
   if (splits > 1024) splits = 1024;
@@ -105,21 +187,36 @@ int direct_sum(const double* targets, int64_t M, const double* sources, int64_t 
   if (splits > 1) BL_TRY(dalloc_n(&part, (size_t)(splits * M), s));
   const dim3 grid(blocks, (unsigned)splits);
   const bool fixed = kappa >= 0.0 && kappa <= DBL_MAX;
-  void (*k)(const double*, int64_t, const double*, int64_t, const double*, double, int64_t, double*) =
-      k_direct<BLDTT_TEST_POLY, false>;
-  if (kernel == BLDTT_COULOMB)
-    k = k_direct<BLDTT_COULOMB, true>;
-  else if (kernel == BLDTT_YUKAWA)
-    k = fixed ? k_direct<BLDTT_YUKAWA, true> : k_direct<BLDTT_YUKAWA, false>;
-  else if (kernel == BLDTT_OSCILLATORY)
-    k = k_direct<BLDTT_OSCILLATORY, false>;
-  else if (kernel == BLDTT_REG_COULOMB)
-    k = fixed ? k_direct<BLDTT_REG_COULOMB, true> : k_direct<BLDTT_REG_COULOMB, false>;
-  k<<<grid, kDirectThreads, 0, s>>>(targets, M, sources, N, charges, kappa, span, part);
+  // The extent takes two launches, about 6 us: worth it from some millions of evaluations.
+  unsigned long long* key = nullptr;
   int64_t dummy = 0;
+  const bool coords = (double)M * (double)N >= 0x1p23 &&
+                      (kernel == BLDTT_COULOMB || (kernel == BLDTT_YUKAWA && fixed));
+  if (coords) {
+    BL_TRY(dalloc_n(&key, 6, s));
+    BL_CUDA(cudaMemsetAsync(key, 0, 6 * sizeof(*key), s));
+    const int64_t need = (M + N + kDirectThreads - 1) / kDirectThreads;
+    k_extent<<<dim3((unsigned)(need < 2 * sms ? need : 2 * sms), 3), kDirectThreads, 0, s>>>(targets, M, sources, N,
+                                                                                            key);
+    BL_LAUNCHED(dummy);
+  }
+  void (*k)(const double*, int64_t, const double*, int64_t, const double*, double, int64_t, const unsigned long long*,
+            double*) = k_direct<BLDTT_TEST_POLY, kFormFp64>;
+  if (kernel == BLDTT_COULOMB)
+    k = coords ? k_direct<BLDTT_COULOMB, kFormFixedCoords> : k_direct<BLDTT_COULOMB, kFormFixed>;
+  else if (kernel == BLDTT_YUKAWA)
+    k = coords  ? k_direct<BLDTT_YUKAWA, kFormFixedCoords>
+        : fixed ? k_direct<BLDTT_YUKAWA, kFormFixed>
+                : k_direct<BLDTT_YUKAWA, kFormFp64>;
+  else if (kernel == BLDTT_OSCILLATORY)
+    k = k_direct<BLDTT_OSCILLATORY, kFormFp64>;
+  else if (kernel == BLDTT_REG_COULOMB)
+    k = fixed ? k_direct<BLDTT_REG_COULOMB, kFormFixed> : k_direct<BLDTT_REG_COULOMB, kFormFp64>;
+  k<<<grid, kDirectThreads, 0, s>>>(targets, M, sources, N, charges, kappa, span, key, part);
   BL_LAUNCHED(dummy);
+  dfree(key, s);
   if (splits > 1) {
-    k_direct_reduce<<<blocks, kDirectThreads, 0, s>>>(part, M, (int)splits, phi);
+    k_direct_reduce<<<(unsigned)((M * 32 + kDirectThreads - 1) / kDirectThreads), kDirectThreads, 0, s>>>(part, M, (int)splits, phi);
     BL_LAUNCHED(dummy);
     dfree(part, s);
   }

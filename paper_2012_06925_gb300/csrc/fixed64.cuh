@@ -71,6 +71,21 @@ __host__ __device__ __forceinline__ int leading_zeros(u64 v) {
   return __builtin_clzll(v);
 #endif
 }
+__host__ __device__ __forceinline__ int leading_zeros32(uint32_t v) {
+#ifdef __CUDA_ARCH__
+  return __clz((int)v);
+#else
+  return __builtin_clz(v);
+#endif
+}
+// High word of the pair (hi, lo) shifted left by s, 0 <= s < 32.
+__host__ __device__ __forceinline__ uint32_t shl_pair(uint32_t hi, uint32_t lo, int s) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_l(lo, hi, (uint32_t)s);
+#else
+  return (uint32_t)((((u64)hi << 32 | lo) << s) >> 32);
+#endif
+}
 // Right shifts of 32 bits and of the word pair (hi, lo) by s >= 0, the latter's
 // low word; 0 (or, for the pair, of no use: its high word is 0) from s = 32 on.
 __host__ __device__ __forceinline__ uint32_t shr(uint32_t v, int s) {
@@ -153,15 +168,49 @@ __host__ __device__ __forceinline__ u64 sum_squares(double dx, double dy, double
   return S + (C >> 30);
 }
 
+// Differences in 64-bit fixed point, units of 2^-k, |d| < 2^62: nothing is left
+// to the FP64 pipe but the accumulation.  Each coordinate's rounding to whole
+// units moves d by one unit at most, so pairs below 2^56 units (kFixedTop: the
+// size of the largest high word) are left to FP64 differences: there the unit
+// is 2^-56 of r, beyond it less, against 2^-54 of an FP64 result.
+constexpr uint32_t kFixedTop = 1u << 24;
+__host__ __device__ __forceinline__ int32_t high_ones(i64 d) {
+  const int32_t h = (int32_t)(d >> 32);
+  return h ^ (h >> 31);
+}
+__host__ __device__ __forceinline__ uint32_t fixed_top(i64 dx, i64 dy, i64 dz) {     // < 2^30
+  return (uint32_t)(high_ones(dx) | high_ones(dy) | high_ones(dz));
+}
+// Sum of squares as sum_squares gives it, top >= kFixedTop.
+__host__ __device__ __forceinline__ u64 sum_squares_fixed(i64 dx, i64 dy, i64 dz, uint32_t top, int k, int* E) {
+  const int s = leading_zeros32(top) - 1;
+  *E = 1085 - k - s;
+  u64 S = 0;
+  i64 C = 0;
+  const i64 d[3] = {dx, dy, dz};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const u64 a = (u64)d[i];
+    const int32_t h = (int32_t)shl_pair((uint32_t)(a >> 32), (uint32_t)a, s);
+    const int32_t l = (int32_t)(((uint32_t)a << s) >> 2);
+    S += (u64)((i64)h * h);
+    C += (i64)h * l;
+  }
+  return S + (u64)(C >> 29);
+}
+
 // 1/r; 0 where FP64's r^2 is 0 (or overflows).
-__host__ __device__ __forceinline__ double inv_r(double dx, double dy, double dz) {
-  int E;
-  const u64 S = sum_squares(dx, dy, dz, &E);
+__host__ __device__ __forceinline__ double inv_r_of(u64 S, int E) {
   const u64 Y = inv_sqrt(S);
   // Y in (2^61.2, 2^63]: two cases instead of a count of leading zeros
   const bool big = (Y >> 62) != 0;
   const u64 b = ((u64)(uint32_t)((big ? 2044 : 2043) - E) << 52) + (big ? (Y + 512) >> 10 : (Y + 256) >> 9);
   return of_bits((unsigned)(E - kMinE) <= (unsigned)(kMaxE - kMinE) ? b : 0ull);
+}
+__host__ __device__ __forceinline__ double inv_r(double dx, double dy, double dz) {
+  int E;
+  const u64 S = sum_squares(dx, dy, dz, &E);
+  return inv_r_of(S, E);
 }
 
 // 1/sqrt(r^2 + kappa^2), kappa >= 0; 0 where FP64's r^2 is 0 (or overflows).
@@ -279,9 +328,7 @@ u64 kExp2[256] = {
 
 // exp(-kappa r)/r; 0 where FP64's r^2 is 0 (or overflows) or the result is
 // below the normal range.
-__host__ __device__ __forceinline__ double screened_inv_r(double dx, double dy, double dz, const Screen& k) {
-  int E;
-  const u64 S = sum_squares(dx, dy, dz, &E);
+__host__ __device__ __forceinline__ double screened_inv_r_of(u64 S, int E, const Screen& k) {
   const u64 Y = inv_sqrt(S);
   const u64 R = mul_hi(S, Y) << 3;              // r = R 2^-63 2^(E - 1022)
   const u64 Z = mul_hi(R, k.m);                 // t = kappa log2(e) r = Z 2^-w
@@ -305,6 +352,26 @@ __host__ __device__ __forceinline__ double screened_inv_r(double dx, double dy, 
   const u64 X = T - mul_hi(T, D);               // 2^-t 2^n in units of 2^-63, in (2^62, 2^63]
   const u64 M = mul_hi(Y, X) << 1;              // units of 2^-62
   return ok ? to_double(M, 1022 - E - n) : 0.0;
+}
+__host__ __device__ __forceinline__ double screened_inv_r(double dx, double dy, double dz, const Screen& k) {
+  int E;
+  const u64 S = sum_squares(dx, dy, dz, &E);
+  return screened_inv_r_of(S, E, k);
+}
+
+// v in units of 2^-k, rounded to nearest, modulo 2^64 (differences of values
+// less than 2^62 units apart are right); k so that |v| 2^k < 2^1000.
+__host__ __device__ __forceinline__ i64 to_fixed(double v, int k) {
+  const u64 b = bits_of(v);
+  const int e = exponent_of(b);
+  const u64 m = e ? (b & 0xfffffffffffffull) | 0x10000000000000ull : b & 0xfffffffffffffull;
+  const int sh = (e ? e : 1) - 1075 + k;          // v = m 2^(sh - k)
+  u64 f;
+  if (sh >= 0)
+    f = sh > 63 ? 0ull : m << sh;
+  else
+    f = sh < -54 ? 0ull : ((m >> (-sh - 1)) + 1) >> 1;
+  return (i64)((b >> 63) ? 0ull - f : f);
 }
 
 }  // namespace fixed64

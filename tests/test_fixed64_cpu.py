@@ -26,6 +26,20 @@ extern "C" void scr(const double* d, long n, double kappa, double* o) {
 extern "C" void reg(const double* d, long n, double kappa, double* o) {
   for (long i = 0; i < n; ++i) o[i] = inv_sqrt_r2_kappa2(d[3 * i], d[3 * i + 1], d[3 * i + 2], kappa);
 }
+extern "C" void fix(const double* xy, long n, double kd, double kappa, double* o) {
+  const int k = (int)kd;
+  const Screen sc = make_screen(kappa);
+  for (long i = 0; i < n; ++i) {
+    const double *x = xy + 6 * i, *y = x + 3;
+    const i64 a = to_fixed(x[0], k) - to_fixed(y[0], k), b = to_fixed(x[1], k) - to_fixed(y[1], k),
+              c = to_fixed(x[2], k) - to_fixed(y[2], k);
+    const uint32_t top = fixed_top(a, b, c);
+    int E;
+    if (top < kFixedTop) { o[i] = -1; continue; }
+    const u64 S = sum_squares_fixed(a, b, c, top, k, &E);
+    o[i] = kappa < 0 ? inv_r_of(S, E) : screened_inv_r_of(S, E, sc);
+  }
+}
 """
 
 
@@ -108,3 +122,34 @@ def test_ends_of_the_range(lib):
     one = np.array([[1.0, 0, 0], [0, -0.5, 0], [3.0, 0, 4.0], [2.0 ** -500, 0, 0]])
     assert np.array_equal(call(lib, "inv", one), [1.0, 2.0, 0.2, 2.0 ** 500])
     assert call(lib, "scr", [[1e4, 0, 0]], 1.0)[0] == 0.0       # exp(-1e4) is 0 in FP64 too
+
+
+@pytest.mark.parametrize("shift,scale", [(0.0, 1.0), (1e6, 1.0), (-3e9, 2.0 ** -20), (0.0, 2.0 ** 400),
+                                         (5e-150, 2.0 ** -480)])
+@pytest.mark.parametrize("kappa", [-1.0, 0.0, 0.7])
+def test_fixed_coordinates(lib, shift, scale, kappa):
+    """Coordinates in units of 2^-62 of the extent (offsets wrap around): 1.2e-16 for the evaluation
+    and 2^-56 sqrt(3) for the units of the closest pairs taken (1/64 of the extent)."""
+    rng = np.random.default_rng(1)
+    xy = rng.uniform(-1, 1, (20000, 6))
+    xy[::3, 3:] = xy[::3, :3] + rng.uniform(-1, 1, (len(xy[::3]), 3)) * 2.0 ** -rng.integers(0, 9, (len(xy[::3]), 1))
+    xy[::5, 2] = xy[::5, 5]
+    xy[:2] = [[-1, -1, -1, 1, 1, 1], [1, -1, 1, -1, 1, -1]]
+    xy = np.clip(xy, -1, 1) * scale + shift
+    w = np.ptp(xy.reshape(-1, 3), axis=0).max()
+    k = 61 - int(np.floor(np.log2(w)))
+    a = np.ascontiguousarray(xy)
+    out = np.empty(len(a))
+    p = ctypes.POINTER(ctypes.c_double)
+    lib.fix(a.ctypes.data_as(p), ctypes.c_long(len(a)), ctypes.c_double(k), ctypes.c_double(kappa / scale),
+            out.ctypes.data_as(p))
+    x = a.astype(np.longdouble)
+    r = np.sqrt(((x[:, :3] - x[:, 3:]) ** 2).sum(axis=1))
+    want = np.exp(-np.longdouble(max(kappa, 0) / scale) * r) / r
+    taken = out >= 0
+    far = np.abs(x[:, :3] - x[:, 3:]).max(axis=1)
+    assert np.all(taken[far >= 2.0 ** (56 - k) * (1 + 2.0 ** -20)]) and not np.any(taken[far < 2.0 ** (56 - k) * (1 - 2.0 ** -20)])
+    err = np.abs(out[taken].astype(np.longdouble) / want[taken] - 1)
+    t = max(kappa, 0) / scale * r[taken]
+    assert np.all(err <= 1.2e-16 + np.sqrt(3.0) * 2.0 ** -56 * (1 + t) + t * 1.45 * 2.0 ** -58)
+    assert taken[:2].all()

@@ -91,3 +91,28 @@ def test_partial_target_tiles(m, kernel, kappa):
     ref = B.direct_sum(tgt, src, q, kernel, kappa)
     scale = B.direct_sum(tgt, src, q, B.COULOMB, 0.0)       # bounds the sum of |terms|
     assert torch.max(torch.abs(phi - ref) / scale).item() <= 310 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("case", ["uniform", "shifted", "clustered", "one_point", "infinite"])
+@pytest.mark.parametrize("kernel,kappa", [(B.COULOMB, 0.0), (B.YUKAWA, 0.6), (B.REG_COULOMB, 0.01)])
+def test_direct_sum_in_fixed_coordinates(case, kernel, kappa):
+    """A sum large enough for fixed-point coordinates against the same targets in calls that are
+    not: terms to 2e-16 in each, tiles of 256 and their sums one after the other."""
+    rng = np.random.default_rng(6)
+    m, n = 300, 40000
+    src, tgt = rng.uniform(-1, 1, (3, n)), rng.uniform(-1, 1, (3, m))
+    if case == "shifted":
+        src, tgt = src + 1e5, tgt + 1e5
+    elif case == "clustered":                       # most pairs far closer than 1/64 of the extent
+        src[:, 1:], tgt[:, 3:] = src[:, 1:] * 1e-4, tgt[:, 3:] * 1e-4
+    elif case == "one_point":
+        src[:], tgt[:] = 0.3, 0.3
+    elif case == "infinite":
+        tgt[1, 5], src[2, 7] = np.inf, -np.inf
+    tgt[:, :100] = src[:, :100]                     # coincident pairs
+    q = torch.from_numpy(rng.uniform(0.5, 1.5, n)).cuda()
+    src, tgt = torch.from_numpy(src).cuda(), torch.from_numpy(np.ascontiguousarray(tgt)).cuda()
+    whole = B.direct_sum(tgt, src, q, kernel, kappa)
+    parts = torch.cat([B.direct_sum(tgt[:, i:i + 100].contiguous(), src, q, kernel, kappa)
+                       for i in range(0, m, 100)])
+    torch.testing.assert_close(whole, parts, rtol=4e-16 + 2 * (256 + n / 256) * 2.0 ** -53, atol=0)
