@@ -828,12 +828,12 @@ __global__ void k_item_boxes(int32_t nitems, const int4* __restrict__ items, con
 
 // Chunks of a task: a tile's sources are split so that the plan's tile-chunks
 // (counted from its kernel evaluations) make about kTasksPerCta tasks per CTA
-// of six on an SM, but not below a few chunks, where a task's start costs more
-// than the even load gives.  Measured (interaction kernel, GB300): 1E6 points
-// (1.9E6 tile-chunks) 31.9 ms at 4 tasks per CTA, 31.4 at 16-24, 31.3 at 50
-// with 0.2 ms more to list them; 2E4 points on a sphere (4800) 0.25 ms at 1-3
-// chunks, 0.18 at 4-6, 0.21 at 8, 0.45 whole; 2E4 points in FP64 2.2 ms at 1-2,
-// 2.3 at 3, 2.4 at 4.  A plan of many short tiles (512 problems) is not split.
+// of six on an SM; FP64 tasks have two chunks at least.  Measured (interaction
+// kernel, GB300): 1E6 points (1.9E6 tile-chunks) 31.9 ms at 4 tasks per CTA, 31.4
+// at 16-24, 31.3 at 50 with 0.2 ms more to list them; 2E4 points on a sphere
+// (4800) 0.14 ms at 1-3 chunks, 0.16 at 4 and 8, 0.45 whole; 1000 points (20)
+// 0.024 ms at 1, 0.032 at 2-3, 0.046 at 4 and more; 2E4 points in FP64 2.2 ms at
+// 1-2, 2.3 at 3, 2.4 at 4.  A plan of many short tiles (512 problems) is not split.
 constexpr int kTasksPerCta = 16;
 static int64_t task_chunks(const bldtt_plan* p) {
   if (const char* e = std::getenv("BLDTT_TASK_CHUNKS"))   // testing: results do not depend on the split
@@ -843,7 +843,7 @@ static int64_t task_chunks(const bldtt_plan* p) {
   double evals = 0.0;
   for (int k = 0; k < 4; ++k) evals += p->interactions[k];
   const double tiles = evals / ((double)kTile * kChunk);
-  return std::max<int64_t>(p->precision == BLDTT_FP32_BULK ? 4 : 2,
+  return std::max<int64_t>(p->precision == BLDTT_FP32_BULK ? 1 : 2,
                            (int64_t)(tiles / ((double)sms * 6 * kTasksPerCta)));
 }
 
