@@ -423,72 +423,86 @@ __device__ __forceinline__ void put(float4* pool, const float4* frame, int64_t i
   r[4] = frame_coord(z, f.z);
   r[6] = (float)q;
 }
+__device__ __forceinline__ void clear_entry(float4* pool, int64_t i) {
+  const int64_t j = i % kChunk;
+  float* r = reinterpret_cast<float*>(pool) + ((i / kChunk) * (kChunk / 2) + j / 2) * 8 + (j & 1);
+  for (int d = 0; d < 4; ++d) r[2 * d] = 0.f;
+}
+__device__ __forceinline__ void clear_entry(double4*, int64_t) {}   // FP64 chunks are single entries
 __device__ __forceinline__ void put(double4* pool, const float4*, int64_t i, double x, double y,
                                     double z, double q) {
   pool[i] = make_double4(x, y, z, q);
 }
 
-template <typename Vec>
-__global__ void k_pool_particles(const int32_t* __restrict__ leaf_ids, const int32_t* __restrict__ begin,
-                                 const int32_t* __restrict__ end, const int32_t* __restrict__ pad_prefix,
-                                 const float4* __restrict__ frame, const double* __restrict__ x,
-                                 const double* __restrict__ y, const double* __restrict__ z,
-                                 const double* __restrict__ q, Vec* __restrict__ pool) {
-  const int lf = blockIdx.x;
-  const int c = leaf_ids[lf];
-  const int64_t o = pad_prefix[lf];
-  for (int32_t i = begin[c] + threadIdx.x; i < end[c]; i += blockDim.x)
-    put(pool, frame, o + (i - begin[c]), x[i], y[i], z[i], q[i]);
+// Proxy blocks of the degrees whose proxies some entry reads.
+struct ProxyBlocks {
+  int count = 0;
+  int n[kMaxDegrees], np_pad[kMaxDegrees];
+  int64_t base[kMaxDegrees];
+  const double* nodes[kMaxDegrees];
+  const double* qhat[kMaxDegrees];
+  int64_t first_block[kMaxDegrees + 1];   // chunk descriptions: first block of each
+};
+static ProxyBlocks proxy_blocks(const bldtt_plan* p) {
+  ProxyBlocks b;
+  for (int i = 0; i < p->deg.n; ++i) {
+    if (!p->deg_used[i]) continue;
+    b.n[b.count] = p->deg.d[i];
+    b.np_pad[b.count] = p->deg.np_pad[i];
+    b.base[b.count] = p->deg.proxy_base[i];
+    b.nodes[b.count] = p->nodes_s[i];
+    b.qhat[b.count] = p->qhat_d[i];
+    ++b.count;
+  }
+  return b;
 }
 
+// The whole pool in one launch: a block per source leaf, then one per source
+// cluster and degree.  Of the padding only the entry that fills an odd chunk's
+// last pair record is read; it is written here (zeros), so the pool needs no
+// clearing (with a memset and a launch per degree: 2E4 points 227 instead of 223 us
+// a product; 512 problems, upward pass and pool, 2.49 instead of 2.40 ms).
 template <typename Vec>
-__global__ void k_pool_proxies(int n, int np_pad, int64_t base, const double* __restrict__ nodes,
-                               const float4* __restrict__ frame, const double* __restrict__ qhat,
-                               Vec* __restrict__ pool) {
-  const int c = blockIdx.x;
-  const int P = n + 1, np = P * P * P;
-  const double* nd = nodes + (int64_t)c * 3 * P;
-  for (int k = threadIdx.x; k < np; k += blockDim.x) {
-    int k1 = k / (P * P), k2 = (k / P) % P, k3 = k % P;
-    put(pool, frame, base + (int64_t)c * np_pad + k, nd[k1], nd[P + k2], nd[2 * P + k3],
-        qhat[(int64_t)c * np + k]);
+__global__ void __launch_bounds__(256) k_pool(int nleaves, const int32_t* __restrict__ leaf_ids,
+                                              const int32_t* __restrict__ begin, const int32_t* __restrict__ end,
+                                              const int32_t* __restrict__ pad_prefix,
+                                              const float4* __restrict__ frame, const double* __restrict__ x,
+                                              const double* __restrict__ y, const double* __restrict__ z,
+                                              const double* __restrict__ q, int nclusters, ProxyBlocks b,
+                                              Vec* __restrict__ pool) {
+  int64_t o;
+  int m;                                            // entries
+  if ((int)blockIdx.x < nleaves) {
+    const int lf = blockIdx.x, c = leaf_ids[lf], i0 = begin[c];
+    o = pad_prefix[lf];
+    m = end[c] - i0;
+    for (int i = threadIdx.x; i < m; i += blockDim.x)
+      put(pool, frame, o + i, x[i0 + i], y[i0 + i], z[i0 + i], q[i0 + i]);
+  } else {
+    const int t = blockIdx.x - nleaves, di = t / nclusters, c = t % nclusters;
+    const int P = b.n[di] + 1;
+    const double* nd = b.nodes[di] + (int64_t)c * 3 * P;
+    m = P * P * P;
+    o = b.base[di] + (int64_t)c * b.np_pad[di];
+    for (int k = threadIdx.x; k < m; k += blockDim.x) {
+      const int k1 = k / (P * P), k2 = (k / P) % P, k3 = k % P;
+      put(pool, frame, o + k, nd[k1], nd[P + k2], nd[2 * P + k3], b.qhat[di][(int64_t)c * m + k]);
+    }
   }
+  if (threadIdx.x == 0 && (m & 1)) clear_entry(pool, o + m);
 }
 
 int build_pool(bldtt_plan* p, cudaStream_t s) {
-  Counters& cnt = p->compute_counter;
   const Tree& T = p->st;
-  const bool f32 = p->precision == BLDTT_FP32_BULK;
-  size_t esz = f32 ? sizeof(float4) : sizeof(double4);
-  BL_CUDA(cudaMemsetAsync(p->pool, 0, (size_t)p->pool_len * esz, s));
-  if (f32) {
-    k_pool_particles<float4><<<T.nleaves, 256, 0, s>>>(T.leaf_ids, T.begin, T.end, p->pad_prefix,
-                                                       p->chunk_frame, T.x, T.y, T.z, p->q_tree,
-                                                       (float4*)p->pool);
-    BL_LAUNCHED(cnt.launches);
-    for (int i = 0; i < p->deg.n; ++i) {
-      if (!p->deg_used[i]) continue;
-      k_pool_proxies<float4><<<T.nclusters, 256, 0, s>>>(p->deg.d[i], p->deg.np_pad[i],
-                                                         p->deg.proxy_base[i], p->nodes_s[i],
-                                                         p->chunk_frame, p->qhat_d[i],
-                                                         (float4*)p->pool);
-      if (i + 1 < p->deg.n) BL_LAUNCHED(cnt.launches);
-    }
-  } else {
-    k_pool_particles<double4><<<T.nleaves, 256, 0, s>>>(T.leaf_ids, T.begin, T.end, p->pad_prefix,
-                                                        p->chunk_frame, T.x, T.y, T.z, p->q_tree,
-                                                        (double4*)p->pool);
-    BL_LAUNCHED(cnt.launches);
-    for (int i = 0; i < p->deg.n; ++i) {
-      if (!p->deg_used[i]) continue;
-      k_pool_proxies<double4><<<T.nclusters, 256, 0, s>>>(p->deg.d[i], p->deg.np_pad[i],
-                                                          p->deg.proxy_base[i], p->nodes_s[i],
-                                                          p->chunk_frame, p->qhat_d[i],
-                                                          (double4*)p->pool);
-      if (i + 1 < p->deg.n) BL_LAUNCHED(cnt.launches);
-    }
-  }
-  BL_LAUNCHED(cnt.launches);
+  const ProxyBlocks b = proxy_blocks(p);
+  const unsigned grid = (unsigned)(T.nleaves + (int64_t)b.count * T.nclusters);
+  if (p->precision == BLDTT_FP32_BULK)
+    k_pool<float4><<<grid, 256, 0, s>>>(T.nleaves, T.leaf_ids, T.begin, T.end, p->pad_prefix, p->chunk_frame, T.x,
+                                        T.y, T.z, p->q_tree, T.nclusters, b, (float4*)p->pool);
+  else
+    k_pool<double4><<<grid, 256, 0, s>>>(T.nleaves, T.leaf_ids, T.begin, T.end, p->pad_prefix, p->chunk_frame, T.x,
+                                         T.y, T.z, p->q_tree, T.nclusters, b, (double4*)p->pool);
+  BL_LAUNCHED(p->compute_counter.launches);
   return BLDTT_OK;
 }
 
@@ -521,11 +535,31 @@ __device__ __forceinline__ void store_chunk(float4* info, int64_t q, const doubl
   info[kChunkInfo * q + 1] = make_float4(ef[0], ef[1], ef[2], tau);
 }
 
-// One CTA per source leaf, one warp per chunk of the leaf's pool segment.
-__global__ void k_frames_particles(const int32_t* __restrict__ leaf_ids, const int32_t* __restrict__ begin,
-                                   const int32_t* __restrict__ end, const int32_t* __restrict__ pad_prefix,
-                                   const double* __restrict__ x, const double* __restrict__ y,
-                                   const double* __restrict__ z, float4* __restrict__ frame) {
+// The descriptions of all chunks and the particles' frame residuals (in the
+// pool's pair-record layout, x0,x1, y0,y1, z0,z1, unused: read only by the
+// careful path) in one launch: a CTA per source leaf, one warp per chunk of its
+// pool segment, then the residuals in the frames just found; then the proxies'
+// chunks, a thread each.
+constexpr int kFrameThreads = 256;
+__global__ void __launch_bounds__(kFrameThreads) k_chunk_frames(
+    int nleaves, const int32_t* __restrict__ leaf_ids, const int32_t* __restrict__ begin,
+    const int32_t* __restrict__ end, const int32_t* __restrict__ pad_prefix, const double* __restrict__ x,
+    const double* __restrict__ y, const double* __restrict__ z, int nclusters, ProxyBlocks pb,
+    const double* __restrict__ center, const double* __restrict__ box, float4* frame, float* __restrict__ res) {
+  if ((int)blockIdx.x >= nleaves) {
+    const int64_t blk = blockIdx.x - nleaves;
+    int di = 0;
+    while (di + 1 < pb.count && blk >= pb.first_block[di + 1]) ++di;
+    const int64_t t = (blk - pb.first_block[di]) * kFrameThreads + threadIdx.x;
+    const int per = pb.np_pad[di] / kChunk, np = (pb.n[di] + 1) * (pb.n[di] + 1) * (pb.n[di] + 1);
+    if (t >= (int64_t)nclusters * per) return;
+    const int64_t c = t / per;
+    const int k = (int)(t % per);
+    double e3[3];
+    for (int d = 0; d < 3; ++d) e3[d] = 0.5 * (box[c * 6 + 3 + d] - box[c * 6 + d]);
+    store_chunk(frame, pb.base[di] / kChunk + t, center + c * 3, e3, min(kChunk, np - k * kChunk), false);
+    return;
+  }
   const int lf = blockIdx.x;
   const int c = leaf_ids[lf];
   const int64_t q0 = pad_prefix[lf] / kChunk, q1 = pad_prefix[lf + 1] / kChunk;
@@ -560,36 +594,19 @@ __global__ void k_frames_particles(const int32_t* __restrict__ leaf_ids, const i
       store_chunk(frame, q, c3, e3, (int)(e > b ? e - b : 0), true);
     }
   }
-}
-
-__global__ void k_frames_proxies(int32_t nclusters, int64_t first_chunk, int32_t chunks_per_cluster,
-                                 int32_t np, const double* __restrict__ center,
-                                 const double* __restrict__ box, float4* __restrict__ frame) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)nclusters * chunks_per_cluster) return;
-  const int64_t c = t / chunks_per_cluster;
-  const int k = (int)(t % chunks_per_cluster);
-  double e3[3];
-  for (int d = 0; d < 3; ++d) e3[d] = 0.5 * (box[c * 6 + 3 + d] - box[c * 6 + d]);
-  store_chunk(frame, first_chunk + t, center + c * 3, e3, min(kChunk, np - k * kChunk), false);
-}
-
-// Frame residuals of the pool's particles, in the pool's pair-record layout
-// (x0,x1, y0,y1, z0,z1, unused): read only by the careful path.
-__global__ void k_pool_residuals(const int32_t* __restrict__ leaf_ids, const int32_t* __restrict__ begin,
-                                 const int32_t* __restrict__ end, const int32_t* __restrict__ pad_prefix,
-                                 const float4* __restrict__ frame, const double* __restrict__ x,
-                                 const double* __restrict__ y, const double* __restrict__ z,
-                                 float* __restrict__ res) {
-  const int lf = blockIdx.x;
-  const int c = leaf_ids[lf];
+  if (!res) return;                                 // FP64 pool
+  __syncthreads();
   const int64_t o = pad_prefix[lf];
-  for (int32_t i = begin[c] + threadIdx.x; i < end[c]; i += blockDim.x) {
-    const int64_t k = o + (i - begin[c]);
-    const float4 f = frame[kChunkInfo * (k / kChunk)];
-    const int64_t j = k % kChunk;
+  const int32_t i0 = begin[c], m = end[c] - i0;
+  for (int32_t i = threadIdx.x; i < m + (m & 1); i += kFrameThreads) {   // an odd chunk's last pair is filled up
+    const int64_t k = o + i, j = k % kChunk;
     float* r = res + ((k / kChunk) * (kChunk / 2) + j / 2) * 8 + (j & 1);
-    const double v[3] = {x[i], y[i], z[i]};
+    if (i == m) {
+      for (int d = 0; d < 3; ++d) r[2 * d] = 0.f;
+      break;
+    }
+    const float4 f = __ldcg(frame + kChunkInfo * (k / kChunk));
+    const double v[3] = {x[i0 + i], y[i0 + i], z[i0 + i]};
     const float cf[3] = {f.x, f.y, f.z};
     for (int d = 0; d < 3; ++d) {
       float hi, lo;
@@ -600,31 +617,19 @@ __global__ void k_pool_residuals(const int32_t* __restrict__ leaf_ids, const int
 }
 
 int build_chunk_frames(bldtt_plan* p, cudaStream_t s) {
-  Counters& cnt = p->setup_counter;
   const Tree& T = p->st;
-  const int64_t nchunks = p->pool_len / kChunk;
-  BL_TRY(dalloc_n(&p->chunk_frame, (size_t)nchunks * kChunkInfo, s));
-  const int64_t pchunks = p->pool_particles / kChunk;
-  if (pchunks > 0) {
-    k_frames_particles<<<T.nleaves, 128, 0, s>>>(T.leaf_ids, T.begin, T.end, p->pad_prefix, T.x, T.y,
-                                                 T.z, p->chunk_frame);
-    BL_LAUNCHED(cnt.launches);
-  }
-  for (int i = 0; i < p->deg.n; ++i) {
-    if (!p->deg_used[i]) continue;
-    const int32_t cpc = p->deg.np_pad[i] / kChunk;
-    k_frames_proxies<<<nblk((int64_t)T.nclusters * cpc, 256), 256, 0, s>>>(
-        T.nclusters, p->deg.proxy_base[i] / kChunk, cpc, p->deg.np[i], T.center, T.box,
-        p->chunk_frame);
-    BL_LAUNCHED(cnt.launches);
-  }
-  if (p->precision == BLDTT_FP32_BULK && pchunks > 0) {
+  BL_TRY(dalloc_n(&p->chunk_frame, (size_t)(p->pool_len / kChunk) * kChunkInfo, s));
+  if (p->precision == BLDTT_FP32_BULK && p->pool_particles > 0)
     BL_TRY(dalloc_n(&p->pool_res, (size_t)p->pool_particles * 4, s));
-    BL_CUDA(cudaMemsetAsync(p->pool_res, 0, (size_t)p->pool_particles * 4 * sizeof(float), s));
-    k_pool_residuals<<<T.nleaves, 256, 0, s>>>(T.leaf_ids, T.begin, T.end, p->pad_prefix,
-                                               p->chunk_frame, T.x, T.y, T.z, p->pool_res);
-    BL_LAUNCHED(cnt.launches);
-  }
+  ProxyBlocks b = proxy_blocks(p);
+  b.first_block[0] = 0;
+  for (int i = 0; i < b.count; ++i)
+    b.first_block[i + 1] =
+        b.first_block[i] + nblk((int64_t)T.nclusters * (b.np_pad[i] / kChunk), kFrameThreads);
+  k_chunk_frames<<<(unsigned)(T.nleaves + b.first_block[b.count]), kFrameThreads, 0, s>>>(
+      T.nleaves, T.leaf_ids, T.begin, T.end, p->pad_prefix, T.x, T.y, T.z, T.nclusters, b, T.center, T.box,
+      p->chunk_frame, p->pool_res);
+  BL_LAUNCHED(p->setup_counter.launches);
   return BLDTT_OK;
 }
 
