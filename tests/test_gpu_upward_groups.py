@@ -1,4 +1,4 @@
-"""Proxy charges of every inner cluster, with the children side by side in eight
+"""Proxy charges of every cluster: leaves of one to a few chunks of 64 particles, and inner clusters with the children side by side in eight
 groups (levels of few clusters) and in two (levels of more than 2048 / P): the
 interpolation reproduces polynomials of degree n, so the moments
 sum_k qhat_k s_k^m of a cluster are those of its particles, m <= n."""
@@ -12,7 +12,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,count,leaf", [(1, 40, 3), (3, 3000, 2), (6, 3000, 4), (8, 1200, 5), (11, 700, 40),
-                                          (16, 400, 60)])
+                                          (16, 400, 60), (1, 700, 200), (2, 129, 150), (4, 900, 190), (5, 64, 80),
+                                          (7, 1500, 260), (8, 700, 128)])
 def test_moments_of_every_cluster(n, count, leaf):
     rng = np.random.default_rng(n)
     pts = rng.uniform(-1, 1, (3, count))
