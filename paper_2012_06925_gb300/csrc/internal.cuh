@@ -478,7 +478,7 @@ int build_lists(bldtt_plan* p, cudaStream_t s);
 int build_work_items(bldtt_plan* p, cudaStream_t s);
 
 // ---- passes (passes.cu) ----
-int permute_charges(bldtt_plan* p, const double* charges_user, cudaStream_t s);
+int permute_charges(bldtt_plan* p, const double* charges_user, int* bad, cudaStream_t s);
 int upward_pass(bldtt_plan* p, cudaStream_t s);
 int build_pool(bldtt_plan* p, cudaStream_t s);
 // Proxy nodes and degree-transfer matrices of the degrees below the highest.

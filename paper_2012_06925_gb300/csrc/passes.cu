@@ -18,16 +18,20 @@ namespace bldtt {
 // ---------------------------------------------------------------------------
 // Charges into source tree order
 // ---------------------------------------------------------------------------
+// bad (may be null) is set if some charge is not finite.
 __global__ void k_permute(const double* __restrict__ src, const int32_t* __restrict__ perm, int64_t n,
-                          double* __restrict__ dst) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = src[perm[i]];
+                          double* __restrict__ dst, int* __restrict__ bad) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double v = src[perm[i]];
+  dst[i] = v;
+  if (bad && !isfinite(v)) *bad = 1;
 }
 
 static inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
-int permute_charges(bldtt_plan* p, const double* charges, cudaStream_t s) {
-  k_permute<<<nblk(p->N, 256), 256, 0, s>>>(charges, p->st.perm, p->N, p->q_tree);
+int permute_charges(bldtt_plan* p, const double* charges, int* bad, cudaStream_t s) {
+  k_permute<<<nblk(p->N, 256), 256, 0, s>>>(charges, p->st.perm, p->N, p->q_tree, bad);
   BL_LAUNCHED(p->setup_counter.launches);
   return BLDTT_OK;
 }
