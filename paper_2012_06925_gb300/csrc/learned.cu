@@ -473,8 +473,8 @@ __global__ void __launch_bounds__(32 * kSelWarps) k_train_samples(
 }
 
 // Weight and bias gradients of all layers in one launch: dW[j][k] = sum_b
-// g[b][j] a[b][k] / cnt, db[j] = sum_b g[b][j] / cnt, each sum sequential over
-// the batch in float.  A block takes kGradJ neurons of one layer, a thread one
+// g[b][j] a[b][k] / cnt, db[j] = sum_b g[b][j] / cnt, each sum in float over
+// kGradB samples, then over those sums, in order.  A block takes kGradJ neurons of one layer, a thread one
 // input k of them (thread 64: the biases), so a sample's activation is read
 // once for kGradJ products; kGradB samples at a time come through shared memory
 // (one thread per weight reading both factors from memory took 4 x ~100 us at
@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(kGradThreads) k_weight_grads(const float* __re
     }
     asm volatile("cp.async.commit_group;");
   };
-  float acc[kGradJ] = {0.f, 0.f, 0.f, 0.f};
+  float total[kGradJ] = {0.f, 0.f, 0.f, 0.f};
   const bool mine = tid < K || tid == kHidden;
   stage(0, 0);
   for (int64_t base = 0, it = 0; base < B; base += kGradB, ++it) {
@@ -546,6 +546,7 @@ __global__ void __launch_bounds__(kGradThreads) k_weight_grads(const float* __re
     __syncthreads();
     const int n = (int)min((int64_t)kGradB, B - base);
     if (mine) {
+      float acc[kGradJ] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 8
       for (int b = 0; b < n; ++b) {
         const float a = tid < kHidden ? sa[buf][b][tid] : 1.f;
@@ -555,6 +556,7 @@ __global__ void __launch_bounds__(kGradThreads) k_weight_grads(const float* __re
         acc[2] = fmaf(g.z, a, acc[2]);
         acc[3] = fmaf(g.w, a, acc[3]);
       }
+      for (int r = 0; r < kGradJ; ++r) total[r] += acc[r];
     }
     __syncthreads();
   }
@@ -563,9 +565,9 @@ __global__ void __launch_bounds__(kGradThreads) k_weight_grads(const float* __re
     const int j = j0 + r;
     if (j >= J) break;
     if (tid < kHidden)
-      out[L.w[l] + (int64_t)j * K + tid] = acc[r] / scnt;
+      out[L.w[l] + (int64_t)j * K + tid] = total[r] / scnt;
     else
-      out[L.b[l] + j] = acc[r] / scnt;
+      out[L.b[l] + j] = total[r] / scnt;
   }
 }
 
