@@ -1,7 +1,8 @@
 // FP64 direct summation, Eq. (1), for error measurements on sampled targets.
 // One thread per target and source split (the sources are split so that few
 // targets still fill the device); sources are staged through shared memory
-// and the splits are summed in order.  Pairs at distance 0 contribute nothing.
+// and the splits are summed in order.  Pairs at distance 0 contribute nothing,
+// whatever their charge (this entry point takes infinities and NaN).
 // Each tile of 256 sources has its own sum, so the sum's rounding grows with
 // the tile's length and the number of tiles, not with the number of sources.
 // In FP64 the pipe (1.7 lanes per clock and SM) bounds the sum at 12
@@ -54,8 +55,52 @@ __global__ void __launch_bounds__(kDirectThreads) k_extent(const double* __restr
 // for pairs closer than 1/64 of it, and for all if the extent is 0 or not finite.
 enum DirectForm { kFormFp64, kFormFixed, kFormFixedCoords };
 
+// q G in FP64 expressions added to a; nothing for a pair at distance 0.
+template <int KERN>
+__device__ __forceinline__ double add_fp64(double dx, double dy, double dz, double q, double kappa, double a) {
+  const double r2 = dx * dx + dy * dy + dz * dz;
+  if (!(r2 > 0.0)) return a;
+  const double r = sqrt(r2);
+  double g;
+  if (KERN == BLDTT_COULOMB)
+    g = 1.0 / r;
+  else if (KERN == BLDTT_YUKAWA)
+    g = exp(-kappa * r) / r;
+  else if (KERN == BLDTT_OSCILLATORY)
+    g = sin(kappa * r) / r;
+  else if (KERN == BLDTT_REG_COULOMB)
+    g = 1.0 / sqrt(r2 + kappa * kappa);
+  else
+    g = 1.0 + dx - 2.0 * dy + 3.0 * dz + dx * dy - dy * dz + dx * dx * dz * dz - 0.5 * dy * dy;
+  return fma(g, q, a);
+}
+// The fixed-point forms give a pair at distance 0 the factor 0, which does not
+// leave out a charge that is not finite: a split's sum that is not finite is
+// taken again here, from the sources in memory and out of line, so that the
+// forms' loops keep their registers.
+template <int KERN>
+__device__ __noinline__ double split_again(const double* t, int64_t M, int64_t i, const double* src, int64_t N,
+                                           const double* q, double kappa, int64_t s0, int64_t s1) {
+  const double x = t[i], y = t[M + i], z = t[2 * M + i];
+  double acc = 0.0, a = 0.0;
+#pragma unroll 1
+  for (int64_t j = s0; j < s1; ++j) {
+    if ((j - s0) % kDirectThreads == 0) {
+      acc += a;
+      a = 0.0;
+    }
+    a = add_fp64<KERN>(x - src[j], y - src[N + j], z - src[2 * N + j], q[j], kappa, a);
+  }
+  return acc + a;
+}
+
+// CTAs of a form that an SM holds (their registers; split_again's must not take more).
 template <int KERN, int FORM>
-__global__ void __launch_bounds__(kDirectThreads) k_direct(const double* __restrict__ t, int64_t M,
+constexpr int direct_ctas() {
+  return FORM == kFormFp64 ? 0 : KERN == BLDTT_YUKAWA ? 5 : FORM == kFormFixedCoords ? 6 : 8;
+}
+template <int KERN, int FORM>
+__global__ void __launch_bounds__(kDirectThreads, direct_ctas<KERN, FORM>()) k_direct(const double* __restrict__ t, int64_t M,
                                                            const double* __restrict__ src, int64_t N,
                                                            const double* __restrict__ q, double kappa,
                                                            int64_t span, const unsigned long long* __restrict__ key,
@@ -105,14 +150,13 @@ __global__ void __launch_bounds__(kDirectThreads) k_direct(const double* __restr
     double a = 0.0;
 #pragma unroll 2
     for (int k = 0; k < cnt; ++k) {
-      double g = 0.0;
       if (FORM == kFormFixedCoords) {
         const long long ux = X - fx[k], uy = Y - fy[k], uz = Z - fz[k];
         const uint32_t top = fixed64::fixed_top(ux, uy, uz);
         if (top >= top_min) {
           int E;
           const fixed64::u64 S = fixed64::sum_squares_fixed(ux, uy, uz, top, k2, &E);
-          g = KERN == BLDTT_COULOMB ? fixed64::inv_r_of(S, E) : fixed64::screened_inv_r_of(S, E, screen);
+          const double g = KERN == BLDTT_COULOMB ? fixed64::inv_r_of(S, E) : fixed64::screened_inv_r_of(S, E, screen);
           a = fma(g, tile[k].w, a);
           continue;
         }
@@ -120,29 +164,21 @@ __global__ void __launch_bounds__(kDirectThreads) k_direct(const double* __restr
       const double4 p = tile[k];
       const double dx = x - p.x, dy = y - p.y, dz = z - p.z;
       if (FORM != kFormFp64) {
-        g = KERN == BLDTT_COULOMB  ? fixed64::inv_r(dx, dy, dz)
-            : KERN == BLDTT_YUKAWA ? fixed64::screened_inv_r(dx, dy, dz, screen)
-                                   : fixed64::inv_sqrt_r2_kappa2(dx, dy, dz, kappa);
+        const double g = KERN == BLDTT_COULOMB  ? fixed64::inv_r(dx, dy, dz)
+                         : KERN == BLDTT_YUKAWA ? fixed64::screened_inv_r(dx, dy, dz, screen)
+                                                : fixed64::inv_sqrt_r2_kappa2(dx, dy, dz, kappa);
+        a = fma(g, p.w, a);
       } else {
-        const double r2 = dx * dx + dy * dy + dz * dz;
-        if (r2 > 0.0) {
-          const double r = sqrt(r2);
-          if (KERN == BLDTT_YUKAWA)
-            g = exp(-kappa * r) / r;
-          else if (KERN == BLDTT_OSCILLATORY)
-            g = sin(kappa * r) / r;
-          else if (KERN == BLDTT_REG_COULOMB)
-            g = 1.0 / sqrt(r2 + kappa * kappa);
-          else
-            g = 1.0 + dx - 2.0 * dy + 3.0 * dz + dx * dy - dy * dz + dx * dx * dz * dz - 0.5 * dy * dy;
-        }
+        a = add_fp64<KERN>(dx, dy, dz, p.w, kappa, a);
       }
-      a = fma(g, p.w, a);
     }
     acc += a;
     __syncthreads();
   }
-  if (i < M) part[(int64_t)blockIdx.y * M + i] = acc;
+  if (i >= M) return;
+  if (FORM != kFormFp64 && fixed64::exponent_of(fixed64::bits_of(acc)) == 0x7ff)
+    acc = split_again<KERN>(t, M, i, src, N, q, kappa, s0, s1);
+  part[(int64_t)blockIdx.y * M + i] = acc;
 }
 
 // phi[i] = sum over the source splits, with each addition's rounding error
