@@ -12,6 +12,8 @@
 // and 9.9 ms.
 #include <float.h>
 
+#include <algorithm>
+
 #include "fixed64.cuh"
 #include "internal.cuh"
 
@@ -209,15 +211,22 @@ int direct_sum(const double* targets, int64_t M, const double* sources, int64_t 
                const double* charges, int kernel, double kappa, double* phi, cudaStream_t s) {
   const unsigned blocks = (unsigned)((M + kDirectThreads - 1) / kDirectThreads);
   // Split the sources so that the grid fills the device (few targets, many
-  // sources): eight CTAs to an SM (with four 2E4 x 2E5 takes 24.6 ms, with eight 21.5).
+  // sources): up to eight CTAs to an SM (with four 2E4 x 2E5 takes 24.6 ms, with
+  // eight 21.5), and of those numbers of splits down to half of it the one whose
+  // fullest SM has the least to do.
   int dev = 0, sms = 0;
   BL_CUDA(cudaGetDevice(&dev));
   BL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  int64_t splits = ((int64_t)8 * sms + blocks - 1) / blocks;
-  const int64_t max_splits = (N + kDirectThreads - 1) / kDirectThreads;
-  if (splits > max_splits) splits = max_splits;
-  if (splits > 1024) splits = 1024;
-  if (splits < 1) splits = 1;
+  const int64_t most = std::max<int64_t>(
+      1, std::min({((int64_t)8 * sms + blocks - 1) / blocks, (N + kDirectThreads - 1) / kDirectThreads, (int64_t)1024}));
+  int64_t splits = most, least = INT64_MAX;
+  for (int64_t k = most; 2 * k > most; --k) {
+    const int64_t load = (blocks * k + sms - 1) / sms * ((N + k - 1) / k);
+    if (load < least) {
+      least = load;
+      splits = k;
+    }
+  }
   const int64_t span = (N + splits - 1) / splits;
   double* part = phi;
   if (splits > 1) BL_TRY(dalloc_n(&part, (size_t)(splits * M), s));
