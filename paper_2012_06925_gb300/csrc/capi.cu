@@ -146,7 +146,6 @@ void release(bldtt_plan* p) {
 float fp32_parameter(int kernel, double kappa) {
   if (kernel == BLDTT_YUKAWA) return (float)(-kappa * 1.4426950408889634);   // -kappa log2(e)
   if (kernel == BLDTT_REG_COULOMB) return (float)(kappa * kappa);
-  if (kernel == BLDTT_OSCILLATORY) return (float)(kappa * 0.31830988618379067154);          // kappa / pi
   return (float)kappa;
 }
 

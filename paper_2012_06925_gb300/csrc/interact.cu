@@ -444,36 +444,57 @@ struct Producer {
 };
 
 // ---- consumers --------------------------------------------------------------
-// sin(pi k r) of two values: k r = n + f with n the nearest integer, sin =
-// (-1)^n f P(f^2) with P the degree-4 minimax polynomial of sin(pi f)/f on
-// |f| <= 1/2 (absolute error 7.6e-9 with these float coefficients, found one
-// after the other so that each absorbs the rounding of those before it).  n comes from
-// adding 1.5 * 2^23 (its parity is the sum's last bit; rint and the conversion
-// to int run on the MUFU's pipe, which the rsqrts fill), and the fraction from
-// one fused multiply-add, so it carries the rounding of r and of k only, as an
-// argument k r rounded to float would.  For arguments beyond 2^22 the phase is
-// noise in float; the clamp keeps |sin| <= 1.
-__device__ __forceinline__ f2_t sinpi2(f2_t r, f2_t k) {
+// Kernel parameter of a work item in FP32: fp32_parameter's value k, and for the
+// oscillatory kernel kappa / pi and pi k / (kappa kPiHigh) - 1 (see sin2).
+struct Param32 {
+  float k, turns, rest;
+};
+struct Param32x2 {               // each duplicated
+  f2_t k, turns, rest;
+};
+__device__ __forceinline__ Param32x2 duplicate(const Param32& p) {
+  return Param32x2{f2_pack(p.k, p.k), f2_pack(p.turns, p.turns), f2_pack(p.rest, p.rest)};
+}
+constexpr float kPiHigh = 3.140625f;
+__device__ __forceinline__ Param32 oscillatory_param(float k, double kappa) {
+  const double pi = 3.14159265358979323846;
+  const double scale = kappa > 0.0 ? (double)k / kappa : 1.0;
+  return Param32{k, (float)(kappa / pi), (float)(pi / (double)kPiHigh * scale - 1.0)};
+}
+
+// sin(kappa r) of two values: kappa r = n pi + f with n the nearest integer, sin =
+// (-1)^n sin f.  n comes from adding 1.5 * 2^23 (its parity is the sum's last
+// bit; rint and the conversion to int run on the MUFU's pipe, which the rsqrts
+// fill).  With k the float nearest to kappa, f k / kappa = k r - n (pi k / kappa), and
+// pi k / kappa is kPiHigh (1 + rest): n kPiHigh comes from one multiply-add, exact
+// to n = 2^15.  So neither the product k r nor kappa's rounding counts n times;
+// what is left of the latter scales f by less than 2^-24, as a product rounded to
+// float would.
+// Where n = 0 and kappa is a float nothing is rounded at all.
+// sin f = f + f^3 Q(f^2), Q the degree-3 minimax polynomial of the relative error on
+// |f| <= pi/2 (6.3e-9 with these float coefficients, found one after the other so
+// that each absorbs the rounding of those before it).  For arguments
+// beyond 2^22 pi the phase is noise in float; the clamp keeps |sin| <= 1.
+__device__ __forceinline__ f2_t sin2(f2_t r, const Param32x2& p) {
   const f2_t big = f2_pack(12582912.f, 12582912.f);
-  const f2_t t = f2_fma(r, k, big);
+  const f2_t t = f2_fma(r, p.turns, big);
+  const f2_t m = f2_fma(t, f2_pack(-kPiHigh, -kPiHigh), f2_pack(12582912.f * kPiHigh, 12582912.f * kPiHigh));   // -n kPiHigh
   float f0, f1, t0, t1, p0, p1;
-  f2_unpack(f2_fma(r, k, f2_sub(big, t)), f0, f1);
+  f2_unpack(f2_fma(m, p.rest, f2_fma(r, p.k, m)), f0, f1);
   f2_unpack(t, t0, t1);
-  const f2_t f = f2_pack(fminf(fmaxf(f0, -0.5f), 0.5f), fminf(fmaxf(f1, -0.5f), 0.5f));
+  const f2_t f = f2_pack(fminf(fmaxf(f0, -1.5707964f), 1.5707964f), fminf(fmaxf(f1, -1.5707964f), 1.5707964f));
   const f2_t s = f2_mul(f, f);
-  f2_t p = f2_fma(s, f2_pack(0.07643287628889084f, 0.07643287628889084f),
-                  f2_pack(-0.597625195980072f, -0.597625195980072f));
-  p = f2_fma(p, s, f2_pack(2.549957752227783f, 2.549957752227783f));
-  p = f2_fma(p, s, f2_pack(-5.1677021980285645f, -5.1677021980285645f));
-  p = f2_fma(p, s, f2_pack(3.141592502593994f, 3.141592502593994f));
-  f2_unpack(f2_mul(p, f), p0, p1);
+  f2_t q = f2_fma(s, f2_pack(2.6060538402816746e-6f, 2.6060538402816746e-6f),
+                  f2_pack(-1.9809768127743155e-4f, -1.9809768127743155e-4f));
+  q = f2_fma(q, s, f2_pack(0.008333069272339344f, 0.008333069272339344f));
+  q = f2_fma(q, s, f2_pack(-0.16666659712791443f, -0.16666659712791443f));
+  f2_unpack(f2_fma(f2_mul(f, s), q, f), p0, p1);
   return f2_pack(__uint_as_float(__float_as_uint(p0) ^ (__float_as_uint(t0) << 31)),
                  __uint_as_float(__float_as_uint(p1) ^ (__float_as_uint(t1) << 31)));
 }
 
 // Packed evaluation of target k against the source pair (s0, s1) at
-// differences d: acc += (q0 G(x - s0), q1 G(x - s1)).  prm2 is the kernel
-// parameter as fp32_parameter gives it, duplicated.  GUARD: a pair at r = 0 is
+// differences d: acc += (q0 G(x - s0), q1 G(x - s1)).  GUARD: a pair at r = 0 is
 // left out (two compares and two selects a pair of evaluations).  The scalar
 // guarded loop that the oscillatory and regularized kernels used to take for
 // every pair (four shared-memory loads and a branch per evaluation, sinf) ran
@@ -481,26 +502,26 @@ __device__ __forceinline__ f2_t sinpi2(f2_t r, f2_t k) {
 // Coulomb loop; packed with the guard on every pair 3.8 and 9.4, with the guard
 // in near chunks only 4.5 and 11.1.
 template <int KERN, bool GUARD = false>
-__device__ __forceinline__ f2_t pair2_eval(f2_t dx, f2_t dy, f2_t dz, f2_t q2, f2_t acc, f2_t prm2) {
+__device__ __forceinline__ f2_t pair2_eval(f2_t dx, f2_t dy, f2_t dz, f2_t q2, f2_t acc, const Param32x2& prm) {
   f2_t r2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
   float r0, r1;
   f2_unpack(r2, r0, r1);
   const bool k0 = !GUARD || r0 > 0.f, k1 = !GUARD || r1 > 0.f;   // a coincident pair contributes nothing
-  if (KERN == BLDTT_REG_COULOMB) f2_unpack(f2_add(r2, prm2), r0, r1);
+  if (KERN == BLDTT_REG_COULOMB) f2_unpack(f2_add(r2, prm.k), r0, r1);
   const float i0 = rsqrt_approx(r0), i1 = rsqrt_approx(r1);
   const f2_t ri = f2_pack(k0 ? i0 : 0.f, k1 ? i1 : 0.f);
   if (KERN == BLDTT_COULOMB || KERN == BLDTT_REG_COULOMB) return f2_fma(q2, ri, acc);
   const f2_t r = f2_mul(r2, ri);
-  if (KERN == BLDTT_OSCILLATORY) return f2_fma(f2_mul(q2, ri), sinpi2(r, prm2), acc);
+  if (KERN == BLDTT_OSCILLATORY) return f2_fma(f2_mul(q2, ri), sin2(r, prm), acc);
   // Yukawa: q ri exp2(-kappa log2(e) r)
   float e0, e1;
-  f2_unpack(f2_mul(r, prm2), e0, e1);
+  f2_unpack(f2_mul(r, prm.k), e0, e1);
   return f2_fma(f2_mul(q2, ri), f2_pack(exp2_approx(e0), exp2_approx(e1)), acc);
 }
 template <int KERN>
 __device__ __forceinline__ f2_t pair2_f32(f2_t tx, f2_t ty, f2_t tz, const ulonglong2& a,
-                                          const ulonglong2& b, f2_t acc, f2_t nk2) {
-  return pair2_eval<KERN>(f2_sub(tx, a.x), f2_sub(ty, a.y), f2_sub(tz, b.x), b.y, acc, nk2);
+                                          const ulonglong2& b, f2_t acc, const Param32x2& prm) {
+  return pair2_eval<KERN>(f2_sub(tx, a.x), f2_sub(ty, a.y), f2_sub(tz, b.x), b.y, acc, prm);
 }
 // Careful variant: d = fma(m, x_r - y_r, x'' - y'') with m = 1 for a target
 // near the chunk (frame residuals added) and m = 0 otherwise (exactly the
@@ -509,10 +530,10 @@ template <int KERN, bool GUARD>
 __device__ __forceinline__ f2_t pair2_careful(f2_t tx, f2_t ty, f2_t tz, f2_t rx, f2_t ry, f2_t rz,
                                               f2_t m2, const ulonglong2& a, const ulonglong2& b,
                                               const ulonglong2& ra, const ulonglong2& rb, f2_t acc,
-                                              f2_t nk2) {
+                                              const Param32x2& prm) {
   return pair2_eval<KERN, GUARD>(f2_fma(m2, f2_sub(rx, ra.x), f2_sub(tx, a.x)),
                           f2_fma(m2, f2_sub(ry, ra.y), f2_sub(ty, a.y)),
-                          f2_fma(m2, f2_sub(rz, rb.x), f2_sub(tz, b.x)), b.y, acc, nk2);
+                          f2_fma(m2, f2_sub(rz, rb.x), f2_sub(tz, b.x)), b.y, acc, prm);
 }
 
 // Sum over the staged chunk of q G for K targets; two partial sums per target.
@@ -522,9 +543,9 @@ __device__ __forceinline__ f2_t pair2_careful(f2_t tx, f2_t ty, f2_t tz, f2_t rx
 // and the oscillatory kernel 3.88, 3.83 and 3.77.
 template <int KERN, int K>
 __device__ __forceinline__ void chunk_f32(const ulonglong2* __restrict__ sb, int npairs,
-                                          const f2_t (&x2)[K][3], float (&a)[K], float nk) {
+                                          const f2_t (&x2)[K][3], float (&a)[K], const Param32& prm) {
   f2_t acc[K];
-  const f2_t nk2 = f2_pack(nk, nk);
+  const Param32x2 prm2 = duplicate(prm);
 #pragma unroll
   for (int k = 0; k < K; ++k) acc[k] = 0ull;
   if (KERN != BLDTT_OSCILLATORY && npairs == kChunk / 2) {
@@ -532,14 +553,14 @@ __device__ __forceinline__ void chunk_f32(const ulonglong2* __restrict__ sb, int
     for (int jp = 0; jp < kChunk / 2; ++jp) {
       const ulonglong2 A = sb[2 * jp], Bq = sb[2 * jp + 1];
 #pragma unroll
-      for (int k = 0; k < K; ++k) acc[k] = pair2_f32<KERN>(x2[k][0], x2[k][1], x2[k][2], A, Bq, acc[k], nk2);
+      for (int k = 0; k < K; ++k) acc[k] = pair2_f32<KERN>(x2[k][0], x2[k][1], x2[k][2], A, Bq, acc[k], prm2);
     }
   } else {
 #pragma unroll 8
     for (int jp = 0; jp < npairs; ++jp) {
       const ulonglong2 A = sb[2 * jp], Bq = sb[2 * jp + 1];
 #pragma unroll
-      for (int k = 0; k < K; ++k) acc[k] = pair2_f32<KERN>(x2[k][0], x2[k][1], x2[k][2], A, Bq, acc[k], nk2);
+      for (int k = 0; k < K; ++k) acc[k] = pair2_f32<KERN>(x2[k][0], x2[k][1], x2[k][2], A, Bq, acc[k], prm2);
     }
   }
 #pragma unroll
@@ -579,8 +600,8 @@ __device__ __forceinline__ void chunk_f32_careful(const ulonglong2* __restrict__
                                                   const ulonglong2* __restrict__ sr, int npairs,
                                                   const f2_t (&x2)[K][3], const TargetSplit& ts,
                                                   const float* c, unsigned near, float (&a)[K],
-                                                  float nk) {
-  const f2_t nk2 = f2_pack(nk, nk);
+                                                  const Param32& prm) {
+  const Param32x2 prm2 = duplicate(prm);
   f2_t acc[K], m2[K], r2x[K][3];
 #pragma unroll
   for (int k = 0; k < K; ++k) {
@@ -598,7 +619,7 @@ __device__ __forceinline__ void chunk_f32_careful(const ulonglong2* __restrict__
 #pragma unroll
     for (int k = 0; k < K; ++k)
       acc[k] = pair2_careful<KERN, GUARD>(x2[k][0], x2[k][1], x2[k][2], r2x[k][0], r2x[k][1], r2x[k][2],
-                                   m2[k], A, Bq, RA, RB, acc[k], nk2);
+                                   m2[k], A, Bq, RA, RB, acc[k], prm2);
   }
 #pragma unroll
   for (int k = 0; k < K; ++k) {
@@ -790,7 +811,7 @@ __device__ __forceinline__ void frame_targets(const TargetSplit& ts, const float
 template <int KERN, int K>
 __device__ __noinline__ PartialSums<K> careful_sums(const float* sf, const float* res, int count,
                                                     const TargetSplit ts, const float* c, unsigned near,
-                                                    float prm) {
+                                                    const Param32 prm) {
   f2_t x2[K][3];
   frame_targets<K>(ts, c, x2);
   PartialSums<K> out;
@@ -816,7 +837,7 @@ template <int KERN, int K>
 __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rbuf, int count,
                                                const f2_t (&x2)[K][3], const TargetSplit& ts,
                                                const float* c, const float4* ext_p, unsigned slot, bool warp_full,
-                                               float prm, float (&a)[K]) {
+                                               const Param32& prm, float (&a)[K]) {
   const float* sf = reinterpret_cast<const float*>(buf);
   const float* res = reinterpret_cast<const float*>(rbuf);
   float xs[K][3];
@@ -922,7 +943,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
   __shared__ double s_tot[K * kConsumers];   // the item's finished segments (in shared memory: no register)
   bool warp_full = true;
   bool warp_active = true;
-  float prm = 0.f;              // its FP32 parameter
+  Param32 prm{};                // its FP32 parameter
   Param64 prm64{};              // its FP64 parameter
   bool yukawa = KERN == BLDTT_YUKAWA;   // the fused Coulomb/Yukawa launch: this item's kernel
   for (uint32_t it = 0;; ++it) {
@@ -932,7 +953,8 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
     if (smeta[s].flags & kTaskStart) {
       item = v.items[smeta[s].item];
       const int pid = v.t_problem[item.x];
-      prm = v.prob_prm[pid];
+      prm.k = v.prob_prm[pid];
+      if (F32 && KERN == BLDTT_OSCILLATORY) prm = oscillatory_param(prm.k, v.prob_kappa[pid]);
       if (!F32) {
         prm64.kappa = v.prob_kappa[pid];
         if (KERN == BLDTT_YUKAWA || KERN == kKernCoulombYukawa) prm64.screen = fixed64::make_screen(prm64.kappa);
@@ -1036,7 +1058,13 @@ static const void* kernel_for_skip(int base) {
     if (base == 1) return reinterpret_cast<const void*>(&k_interact<F32, KERN, 2, 4, 6, 3, SKIP>);
     if (base == 2) return reinterpret_cast<const void*>(&k_interact<F32, KERN, 4, 2, 5, 4, SKIP>);
   }
-  return reinterpret_cast<const void*>(&k_interact<F32, KERN, 4, 2, 6, 3, SKIP>);
+  // The oscillatory kernel's packed loop takes 90 registers; at six CTAs its
+  // spills cost more than the two CTAs give (1E5 points of a Plummer sphere, n 6, leaves of
+  // 1000, whole compute phase: 4.39 ms at six, 4.27 at five, 4.20 at four).
+  if constexpr (F32 && KERN == BLDTT_OSCILLATORY)
+    return reinterpret_cast<const void*>(&k_interact<F32, KERN, 4, 2, 4, 3, SKIP>);
+  else
+    return reinterpret_cast<const void*>(&k_interact<F32, KERN, 4, 2, 6, 3, SKIP>);
 }
 
 template <bool F32, int KERN>
