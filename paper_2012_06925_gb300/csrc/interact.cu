@@ -494,19 +494,26 @@ __device__ __forceinline__ f2_t sin2(f2_t r, const Param32x2& p) {
 }
 
 // Packed evaluation of target k against the source pair (s0, s1) at
-// differences d: acc += (q0 G(x - s0), q1 G(x - s1)).  GUARD: a pair at r = 0 is
-// left out (two compares and two selects a pair of evaluations).  The scalar
+// differences d: acc += (q0 G(x - s0), q1 G(x - s1)).  A guard gives a pair at r =
+// 0 the factor 0 (two compares and two selects a pair of evaluations); kGuardPair
+// leaves its charge out as well, which may be infinite in float.  The scalar
 // guarded loop that the oscillatory and regularized kernels used to take for
 // every pair (four shared-memory loads and a branch per evaluation, sinf) ran
 // at 0.67 and 2.6 evaluations per clock and SM against 12.4 of the packed
 // Coulomb loop; packed with the guard on every pair 3.8 and 9.4, with the guard
 // in near chunks only 4.5 and 11.1.
-template <int KERN, bool GUARD = false>
+enum Guard { kNoGuard, kGuardFactor, kGuardPair };
+template <int KERN, Guard GUARD = kNoGuard>
 __device__ __forceinline__ f2_t pair2_eval(f2_t dx, f2_t dy, f2_t dz, f2_t q2, f2_t acc, const Param32x2& prm) {
   f2_t r2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
   float r0, r1;
   f2_unpack(r2, r0, r1);
-  const bool k0 = !GUARD || r0 > 0.f, k1 = !GUARD || r1 > 0.f;   // a coincident pair contributes nothing
+  const bool k0 = GUARD == kNoGuard || r0 > 0.f, k1 = GUARD == kNoGuard || r1 > 0.f;
+  if (GUARD == kGuardPair) {
+    float q0, q1;
+    f2_unpack(q2, q0, q1);
+    q2 = f2_pack(k0 ? q0 : 0.f, k1 ? q1 : 0.f);
+  }
   if (KERN == BLDTT_REG_COULOMB) f2_unpack(f2_add(r2, prm.k), r0, r1);
   const float i0 = rsqrt_approx(r0), i1 = rsqrt_approx(r1);
   const f2_t ri = f2_pack(k0 ? i0 : 0.f, k1 ? i1 : 0.f);
@@ -526,7 +533,7 @@ __device__ __forceinline__ f2_t pair2_f32(f2_t tx, f2_t ty, f2_t tz, const ulong
 // Careful variant: d = fma(m, x_r - y_r, x'' - y'') with m = 1 for a target
 // near the chunk (frame residuals added) and m = 0 otherwise (exactly the
 // packed difference x'' - y'').
-template <int KERN, bool GUARD>
+template <int KERN, Guard GUARD>
 __device__ __forceinline__ f2_t pair2_careful(f2_t tx, f2_t ty, f2_t tz, f2_t rx, f2_t ry, f2_t rz,
                                               f2_t m2, const ulonglong2& a, const ulonglong2& b,
                                               const ulonglong2& ra, const ulonglong2& rb, f2_t acc,
@@ -595,7 +602,7 @@ __device__ __forceinline__ void target_residual(const TargetSplit& ts, const flo
 }
 
 // Careful packed sum over the staged chunk (sr: its frame residual records).
-template <int KERN, int K, bool GUARD>
+template <int KERN, int K, Guard GUARD>
 __device__ __forceinline__ void chunk_f32_careful(const ulonglong2* __restrict__ sb,
                                                   const ulonglong2* __restrict__ sr, int npairs,
                                                   const f2_t (&x2)[K][3], const TargetSplit& ts,
@@ -806,17 +813,17 @@ __device__ __forceinline__ void frame_targets(const TargetSplit& ts, const float
     }
   }
 }
-// The careful path's sums with the r = 0 guard.  A call of its own: its
+// The careful path's sums with an r = 0 guard.  A call of its own: its
 // registers must not crowd the plain loop's.
-template <int KERN, int K>
+template <int KERN, int K, Guard GUARD>
 __device__ __noinline__ PartialSums<K> careful_sums(const float* sf, const float* res, int count,
                                                     const TargetSplit ts, const float* c, unsigned near,
                                                     const Param32 prm) {
   f2_t x2[K][3];
   frame_targets<K>(ts, c, x2);
   PartialSums<K> out;
-  chunk_f32_careful<KERN, K, true>(reinterpret_cast<const ulonglong2*>(sf), reinterpret_cast<const ulonglong2*>(res),
-                             (count + 1) / 2, x2, ts, c, near, out.v, prm);
+  chunk_f32_careful<KERN, K, GUARD>(reinterpret_cast<const ulonglong2*>(sf), reinterpret_cast<const ulonglong2*>(res),
+                              (count + 1) / 2, x2, ts, c, near, out.v, prm);
   return out;
 }
 // One staged chunk in FP32 for K targets (partial sums in a[]).  ts holds
@@ -827,7 +834,7 @@ __device__ __noinline__ PartialSums<K> careful_sums(const float* sf, const float
 // packed path, which adds the frame residuals for near targets only, and with
 // the r = 0 guard if a target lies inside the chunk's box (or within a
 // thousandth of tau of it).  Otherwise the plain packed path runs.  A sum that
-// is not finite is redone with the guard.
+// is not finite is redone with coincident pairs left out, charge and all.
 // The chunk that a tile shares with its own targets used to run twice, the
 // second time in a scalar loop at an eighth of the rate: 1000 particles 0.099
 // -> 0.046 ms in this kernel, 2E4 on a sphere 0.184 -> 0.139, 512 problems of
@@ -869,10 +876,10 @@ __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rb
   }
   const ulonglong2* sb = reinterpret_cast<const ulonglong2*>(buf);
   if (any_near && !inside) {
-    chunk_f32_careful<KERN, K, false>(sb, reinterpret_cast<const ulonglong2*>(rbuf), (count + 1) / 2, x2,
+    chunk_f32_careful<KERN, K, kNoGuard>(sb, reinterpret_cast<const ulonglong2*>(rbuf), (count + 1) / 2, x2,
                                       ts, c, near, a, prm);
   } else if (any_near) {
-    const PartialSums<K> r = careful_sums<KERN, K>(sf, res, count, ts, c, near, prm);
+    const PartialSums<K> r = careful_sums<KERN, K, kGuardFactor>(sf, res, count, ts, c, near, prm);
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = r.v[k];
   } else if (K > 1 && !warp_full) {
@@ -891,7 +898,7 @@ __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rb
   for (int k = 0; k < K; ++k) bad = bad || not_finite(a[k]);
   if (__any_sync(0xffffffffu, bad)) {
     // residuals that were not staged are not read: any finite numbers do (their factor is 0)
-    const PartialSums<K> r = careful_sums<KERN, K>(sf, slot ? res : sf, count, ts, c, near, prm);
+    const PartialSums<K> r = careful_sums<KERN, K, kGuardPair>(sf, slot ? res : sf, count, ts, c, near, prm);
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = r.v[k];
   }
