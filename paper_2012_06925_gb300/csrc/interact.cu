@@ -96,6 +96,7 @@ struct InteractView {
   const float* prob_prm;       // FP32 kernel parameter (fp32_parameter)
   const double* prob_kappa;
   const int* prob_kernel;      // kernel of each problem (read per item by the fused launch)
+  bool overlap;                // a target may lie at a source proxy (clusters_may_overlap)
 };
 
 // Flags of a staged chunk: first of its task, last of its segment, last of its task.
@@ -834,7 +835,9 @@ __device__ __noinline__ PartialSums<K> careful_sums(const float* sf, const float
 // packed path, which adds the frame residuals for near targets only, and with
 // the r = 0 guard if a target lies inside the chunk's box (or within a
 // thousandth of tau of it).  Otherwise the plain packed path runs.  A sum that
-// is not finite is redone with coincident pairs left out, charge and all.
+// is not finite is redone with coincident pairs left out, charge and all.  The
+// regularized kernel is finite at r = 0: where a target may lie at a source proxy
+// (overlap), its proxy chunks take the guarded call too.
 // The chunk that a tile shares with its own targets used to run twice, the
 // second time in a scalar loop at an eighth of the rate: 1000 particles 0.099
 // -> 0.046 ms in this kernel, 2E4 on a sphere 0.184 -> 0.139, 512 problems of
@@ -844,7 +847,7 @@ template <int KERN, int K>
 __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rbuf, int count,
                                                const f2_t (&x2)[K][3], const TargetSplit& ts,
                                                const float* c, const float4* ext_p, unsigned slot, bool warp_full,
-                                               const Param32& prm, float (&a)[K]) {
+                                               bool overlap, const Param32& prm, float (&a)[K]) {
   const float* sf = reinterpret_cast<const float*>(buf);
   const float* res = reinterpret_cast<const float*>(rbuf);
   float xs[K][3];
@@ -880,6 +883,10 @@ __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rb
                                       ts, c, near, a, prm);
   } else if (any_near) {
     const PartialSums<K> r = careful_sums<KERN, K, kGuardFactor>(sf, res, count, ts, c, near, prm);
+#pragma unroll
+    for (int k = 0; k < K; ++k) a[k] = r.v[k];
+  } else if (KERN == BLDTT_REG_COULOMB && overlap && !(ext_p->w >= 0.f)) {
+    const PartialSums<K> r = careful_sums<KERN, K, kGuardFactor>(sf, sf, count, ts, c, 0u, prm);
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = r.v[k];
   } else if (K > 1 && !warp_full) {
@@ -1004,11 +1011,11 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
       }
       float a[K];
       if (KERN != kKernCoulombYukawa)
-        eval_chunk_f32<KERN, K>(sbuf[s], sres[s], count, x2, ts, c, ext, slot, warp_full, prm, a);
+        eval_chunk_f32<KERN, K>(sbuf[s], sres[s], count, x2, ts, c, ext, slot, warp_full, v.overlap, prm, a);
       else if (yukawa)
-        eval_chunk_f32<BLDTT_YUKAWA, K>(sbuf[s], sres[s], count, x2, ts, c, ext, slot, warp_full, prm, a);
+        eval_chunk_f32<BLDTT_YUKAWA, K>(sbuf[s], sres[s], count, x2, ts, c, ext, slot, warp_full, v.overlap, prm, a);
       else
-        eval_chunk_f32<BLDTT_COULOMB, K>(sbuf[s], sres[s], count, x2, ts, c, ext, slot, warp_full, prm, a);
+        eval_chunk_f32<BLDTT_COULOMB, K>(sbuf[s], sres[s], count, x2, ts, c, ext, slot, warp_full, v.overlap, prm, a);
 #pragma unroll
       for (int k = 0; k < K; ++k) acc[k] += (double)a[k];
     } else {
@@ -1131,6 +1138,15 @@ int interaction_grids(bldtt_plan* p) {
   return BLDTT_OK;
 }
 
+// Whether a pair of overlapping or touching clusters may be approximated.  With
+// (r_t + r_s) < theta R all points of the two are (1 - theta) R or more apart: far
+// more than their rounding in FP32 (6e-8 R) up to theta = 0.999.  The learned
+// selector may take any pair below 1 that lies in its box of features (the
+// fifth is (r_t + r_s)/R).
+static bool clusters_may_overlap(const bldtt_plan* p) {
+  return p->theta > 0.999 || (p->learned && p->selector_net && p->sel_hi[4] > 0.999f);
+}
+
 static InteractView make_view(const bldtt_plan* p) {
   const Tree& tt = p->tt;
   const Tree& st = p->st;
@@ -1166,6 +1182,7 @@ static InteractView make_view(const bldtt_plan* p) {
   v.prob_prm = p->prob_prm;
   v.prob_kappa = p->prob_kappa;
   v.prob_kernel = p->prob_kernel;
+  v.overlap = clusters_may_overlap(p);
   return v;
 }
 
