@@ -143,14 +143,18 @@ __host__ __device__ __forceinline__ u64 inv_sqrt(u64 S) {
   return ((u64)Y0 << 38) + (u64)((ch * (i64)Y0) << 8) + (wide((uint32_t)c, Y0) >> 24);
 }
 
-// M 2^-62 2^X as a double (M > 0), rounded to nearest; 0 below the normal range.
-__host__ __device__ __forceinline__ double to_double(u64 M, int X) {
+// M 2^-62 2^X as a double (M > 0), rounded to nearest; 0 if !ok.
+__host__ __device__ __forceinline__ double to_double(u64 M, int X, bool ok) {
   const int lz = leading_zeros(M);
   const int e = 1023 + X + 1 - lz;              // biased exponent, before a carry of the rounding
   const u64 n = M << lz;
   // the implicit bit of n >> 11 adds one to the exponent field
-  const u64 b = ((u64)(uint32_t)(e - 1) << 52) + (n >> 11) + ((n >> 10) & 1);
-  return of_bits(e >= 1 ? b : 0ull);
+  u64 b = ((u64)(uint32_t)(e - 1) << 52) + (n >> 11) + ((n >> 10) & 1);
+  if (!(ok && e >= 1)) {                        // one branch for both: rarely taken
+    const int sh = 12 - e;                      // subnormal: units of 2^-1074
+    b = !ok || sh > 64 ? 0ull : sh == 64 ? n >> 63 : (n >> sh) + ((n >> (sh - 1)) & 1);
+  }
+  return of_bits(b);
 }
 
 // Sum of squares of the three differences (and, for the regularized kernel, of
@@ -231,7 +235,7 @@ __host__ __device__ __forceinline__ double inv_sqrt_r2_kappa2(double dx, double 
   // four squares: S in [2^60, 2^64]; S just below 4 2^62 at most, as h < 2^31
   const u64 Y = inv_sqrt(S);
   const bool ok = (unsigned)(E3 - kMinE) <= (unsigned)(kMaxE - kMinE) && e <= kMaxE;
-  return ok ? to_double(Y, 1022 - e) : 0.0;
+  return to_double(Y, 1022 - e, ok);
 }
 
 // kappa log2(e) = m 2^-64 2^x, m of 64 significant bits (m = 0: kappa = 0).
@@ -326,8 +330,8 @@ u64 kExp2[256] = {
     0x40b268f9de0183baull, 0x4085a050ec0a036aull, 0x4058f6a7ecccd5b6ull, 0x402c6be96af2fb58ull,
 };
 
-// exp(-kappa r)/r; 0 where FP64's r^2 is 0 (or overflows) or the result is
-// below the normal range.
+// exp(-kappa r)/r; 0 where FP64's r^2 is 0 (or overflows), and where t = kappa
+// log2(e) r is 2^11 or more (1/r is below 2^538).
 __host__ __device__ __forceinline__ double screened_inv_r_of(u64 S, int E, const Screen& k) {
   const u64 Y = inv_sqrt(S);
   const u64 R = mul_hi(S, Y) << 3;              // r = R 2^-63 2^(E - 1022)
@@ -335,8 +339,8 @@ __host__ __device__ __forceinline__ double screened_inv_r_of(u64 S, int E, const
   const int w = 1085 - k.x - E;
   const int sh = w > 56 ? w - 56 : 0, F = w > 56 ? 56 : w;
   const u64 U = sh > 63 ? 0ull : Z >> sh;       // t in units of 2^-F
-  const bool ok = (unsigned)(E - kMinE) <= (unsigned)(kMaxE - kMinE) && (w >= 52 || k.m == 0);
-  const int Fs = F < 52 ? 52 : F;
+  const bool ok = (unsigned)(E - kMinE) <= (unsigned)(kMaxE - kMinE) && (w >= 51 || k.m == 0);   // below: t >= 2^11
+  const int Fs = F < 51 ? 51 : F;
   const u64 V = k.m == 0 ? 0ull : U;
   const int n = (int)(V >> Fs);
   const u64 G = V << (64 - Fs);                 // fraction, units of 2^-64
@@ -351,7 +355,7 @@ __host__ __device__ __forceinline__ double screened_inv_r_of(u64 S, int E, const
   const u64 T = kExp2[G >> 56];
   const u64 X = T - mul_hi(T, D);               // 2^-t 2^n in units of 2^-63, in (2^62, 2^63]
   const u64 M = mul_hi(Y, X) << 1;              // units of 2^-62
-  return ok ? to_double(M, 1022 - E - n) : 0.0;
+  return to_double(M, 1022 - E - n, ok);
 }
 __host__ __device__ __forceinline__ double screened_inv_r(double dx, double dy, double dz, const Screen& k) {
   int E;
