@@ -66,7 +66,8 @@ constexpr uint64_t kWaitNs = 20ull * 1000ull * 1000ull * 1000ull;   // 20 s boun
 struct InteractView {
   const int4* items;
   const int4* parts;            // {first chunk, chunks, segment-sum slot or -1, segments | segment length << 8}
-  double* seg_sums;             // [slots][kMaxSegments][kTile]
+  double* seg_sums;             // [groups of 32 rows]: from slot_rows[slot] on, [segments][groups of the tile]
+  const int32_t* slot_rows;
   int32_t* arrived;             // [slots][kItemGroups]: segments finished, per consumer warp
   int32_t nitems;
   int32_t* counter;
@@ -770,9 +771,12 @@ __device__ __noinline__ void end_segment(const InteractView& v, const int4 item,
     }
     return;
   }
-  double* sums = v.seg_sums + (int64_t)slot * (kMaxSegments * kTile);
+  const int rows = (item.z + 31) / 32 * 32;
+  if (ct >= rows) return;                       // whole warps: no row of this tile
+  double* sums = v.seg_sums + (int64_t)v.slot_rows[slot] * 32;
 #pragma unroll
-  for (int k = 0; k < K; ++k) sums[seg * kTile + k * NCW * 32 + ct] = a.v[k];
+  for (int k = 0; k < K; ++k)
+    if (k * NCW * 32 + ct < rows) sums[seg * rows + k * NCW * 32 + ct] = a.v[k];
   if (!(flags & kTaskEnd)) return;
   const int4 part = v.parts[task];
   const int nseg = part.w & 0xff, len = part.w >> 8;
@@ -786,8 +790,9 @@ __device__ __noinline__ void end_segment(const InteractView& v, const int4 item,
   __threadfence();
   for (int k = 0; k < K; ++k) {
     const int r = k * NCW * 32 + ct;
+    if (r >= rows) break;
     double t = 0.0;
-    for (int g = 0; g < nseg; ++g) t += __ldcg(sums + g * kTile + r);
+    for (int g = 0; g < nseg; ++g) t += __ldcg(sums + g * rows + r);
     store_output(v, item, r, t);
   }
   if (lane == 0) *count = 0;
@@ -1154,6 +1159,7 @@ static InteractView make_view(const bldtt_plan* p) {
   v.items = p->items;
   v.parts = p->parts;
   v.seg_sums = p->seg_sums;
+  v.slot_rows = p->slot_rows;
   v.arrived = p->item_counter + kMaxSegmentsLaunch;
   v.nitems = p->nitems;
   v.counter = p->item_counter;

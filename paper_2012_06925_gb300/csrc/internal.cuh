@@ -359,7 +359,11 @@ struct bldtt_plan {
   int4* parts = nullptr;              // task i: {first chunk, chunks, split slot or -1, nseg | len << 8}
   int32_t nitems = 0;                 // tasks: the tiles, long ones split over their sources (plan_parts)
   int32_t nsplit = 0;                 // split tiles
-  double* seg_sums = nullptr;         // [nsplit][kMaxSegments][kTile] segment sums of the split tiles
+  // Segment sums of the split tiles, in groups of 32 target rows: a tile has its segments x its own
+  // groups, from group slot_rows[slot] on (as many segments and rows for every tile: 32 KB each).
+  double* seg_sums = nullptr;         // [sum_groups][32]
+  int32_t* slot_rows = nullptr;       // [nsplit]
+  int32_t sum_groups = 0;
   // [kMaxSegmentsLaunch] next task of each segment, then [nsplit][kItemGroups] finished segments
   int32_t* item_counter = nullptr;
   size_t counter_words = 0;
