@@ -106,7 +106,6 @@ void release(bldtt_plan* p) {
   dfree_ptr(p->items, s);
   dfree_ptr(p->parts, s);
   dfree_ptr(p->seg_sums, s);
-  dfree_ptr(p->slot_rows, s);
   dfree_ptr(p->item_counter, s);
   dfree_ptr(p->chunk_frame, s);
   dfree_ptr(p->pool_res, s);
@@ -264,11 +263,11 @@ int setup_impl(bldtt_plan* p, const double* targets, const double* sources, cons
   p->qhat_d[p->deg.n - 1] = p->qhat;
   p->phit_d[p->deg.n - 1] = p->phit;
   BL_TRY(dalloc_n(&p->phi_near, (size_t)p->M, s));
-  p->counter_words = kMaxSegmentsLaunch + (size_t)p->nsplit * kItemGroups;
+  p->counter_words = kMaxSegmentsLaunch + (size_t)p->sum_groups;
   BL_TRY(dalloc_n(&p->item_counter, p->counter_words, s));
   // autotuning runs a launch by itself: the finished-segment counts start (and end) at zero
   BL_CUDA(cudaMemsetAsync(p->item_counter, 0, p->counter_words * sizeof(int32_t), s));
-  if (p->nsplit > 0) BL_TRY(dalloc_n(&p->seg_sums, (size_t)p->sum_groups * 32, s));
+  if (p->sum_groups > 0) BL_TRY(dalloc_n(&p->seg_sums, (size_t)p->sum_groups * 32, s));
   BL_TRY(build_chunk_frames(p, s));
   // Default layout: warps of empty rows skip their work when that saves at
   // least 2 % of the evaluations (many items smaller than a tile).

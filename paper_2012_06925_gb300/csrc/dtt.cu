@@ -654,8 +654,7 @@ __global__ void k_item_count(int32_t nct, ListView L, const int32_t* __restrict_
                              int64_t* __restrict__ cost_part, int64_t* __restrict__ cost_prox,
                              unsigned long long* __restrict__ executed,   // [2]: skip, no skip
                              int64_t* __restrict__ eval_part, int64_t* __restrict__ eval_prox,
-                             int64_t part_len, int32_t* __restrict__ nsplit, int32_t* __restrict__ longest,
-                             int32_t* __restrict__ sum_rows) {
+                             int64_t part_len, int32_t* __restrict__ sum_groups, int32_t* __restrict__ longest) {
   const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (c >= nct) return;                 // whole warps
   int64_t cp = 0, sp = 0;
@@ -671,8 +670,7 @@ __global__ void k_item_count(int32_t nct, ListView L, const int32_t* __restrict_
   const PartPlan pp = plan_parts(cp, part_len);
   int64_t len = (int64_t)pp.per * pp.len;     // chunks of its longest task, or more
   int32_t items = tp * pp.parts;
-  int32_t split = pp.parts > 1 ? tp : 0;
-  int32_t rows = pp.parts > 1 ? pp.nseg * ((end[c] - begin[c] + 31) / 32) : 0;   // segment sums, in 32-row groups
+  int32_t groups = pp.parts > 1 ? pp.nseg * ((end[c] - begin[c] + 31) / 32) : 0;   // segment sums of split tiles
   unsigned long long ex = cp > 0 ? (unsigned long long)executed_rows_skip(end[c] - begin[c]) * sp : 0ull;
   unsigned long long ex_ns = cp > 0 ? (unsigned long long)executed_rows_noskip(end[c] - begin[c]) * sp : 0ull;
   int64_t evq = 0;
@@ -686,10 +684,7 @@ __global__ void k_item_count(int32_t nct, ListView L, const int32_t* __restrict_
     const PartPlan pq = plan_parts(cq, part_len);
     len = max(len, (int64_t)pq.per * pq.len);
     items += tq * pq.parts;
-    if (pq.parts > 1) {
-      split += tq;
-      rows += pq.nseg * ((L.deg.np[i] + 31) / 32);
-    }
+    if (pq.parts > 1) groups += pq.nseg * ((L.deg.np[i] + 31) / 32);
     if (lane == 0) cost_prox[(int64_t)c * kMaxDegrees + i] = cq;
     if (cq > 0) {
       ex += (unsigned long long)executed_rows_skip(L.deg.np[i]) * sq;
@@ -702,10 +697,7 @@ __global__ void k_item_count(int32_t nct, ListView L, const int32_t* __restrict_
   eval_prox[c] = evq;
   nitems[c] = items;
   cost_part[c] = cp;
-  if (split) {
-    atomicAdd(nsplit, split);
-    atomicAdd(sum_rows, rows);
-  }
+  if (groups) atomicAdd(sum_groups, groups);
   atomicMax(longest, (int32_t)min(len, (int64_t)INT32_MAX));
   // evaluations the kernel performs: every target slot of every tile meets every real source
   if (ex) atomicAdd(executed, ex);
@@ -723,20 +715,15 @@ struct SegmentMap {
 
 // The tasks of one tile {c, r, rows, kind} of `chunks` source chunks.
 __device__ __forceinline__ void fill_tasks(int4 tile, int64_t chunks, int64_t part_len, uint32_t key_base,
-                                           uint32_t key_max, int32_t& o, int32_t* next_slot,
-                                           int32_t* next_rows, int32_t* slot_rows, int4* items, int4* parts,
-                                           uint32_t* keys) {
+                                           uint32_t key_max, int32_t& o, int32_t* next_group, int4* items,
+                                           int4* parts, uint32_t* keys) {
   const PartPlan q = plan_parts(chunks, part_len);
-  // the slot numbers depend on the order of the atomics, the results do not
-  int32_t slot = -1;
-  if (q.parts > 1) {
-    slot = atomicAdd(next_slot, 1);
-    slot_rows[slot] = atomicAdd(next_rows, q.nseg * ((tile.z + 31) / 32));
-  }
+  // where its sums lie depends on the order of the atomics, the results do not
+  const int32_t group = q.parts > 1 ? atomicAdd(next_group, q.nseg * ((tile.z + 31) / 32)) : -1;
   for (int32_t i = 0; i < q.parts; ++i) {
     const int64_t b = (int64_t)i * q.per * q.len, e = min(chunks, b + (int64_t)q.per * q.len);
     items[o] = tile;
-    parts[o] = make_int4((int)b, (int)(e - b), slot, q.nseg | (q.len << 8));
+    parts[o] = make_int4((int)b, (int)(e - b), group, q.nseg | (q.len << 8));
     keys[o] = key_base | (key_max - (uint32_t)min((int64_t)key_max, e - b));
     ++o;
   }
@@ -747,8 +734,8 @@ __global__ void k_item_fill(int32_t nct, const int32_t* __restrict__ off,
                             const int32_t* __restrict__ begin, const int32_t* __restrict__ end,
                             const int32_t* __restrict__ problem, const int* __restrict__ prob_kernel,
                             SegmentMap segmap, DegreeSet deg, int64_t part_len, int len_bits,
-                            int32_t* __restrict__ next_slot, int32_t* __restrict__ next_rows,
-                            int32_t* __restrict__ slot_rows, int4* __restrict__ items, int4* __restrict__ parts, uint32_t* __restrict__ keys) {
+                            int32_t* __restrict__ next_group,
+                            int4* __restrict__ items, int4* __restrict__ parts, uint32_t* __restrict__ keys) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= nct) return;
   int32_t o = off[c];
@@ -765,14 +752,14 @@ __global__ void k_item_fill(int32_t nct, const int32_t* __restrict__ off,
   if (cost_part[c] > 0)
     for (int32_t r = begin[c]; r < end[c]; r += kTile)
       fill_tasks(make_int4(c, r, min(kTile, end[c] - r), kItemParticles), cost_part[c], part_len, key_base,
-                 key_max, o, next_slot, next_rows, slot_rows, items, parts, keys);
+                 key_max, o, next_group, items, parts, keys);
   for (int i = 0; i < deg.n; ++i) {
     const int64_t cq = cost_prox[(int64_t)c * kMaxDegrees + i];
     if (cq <= 0) continue;
     const int32_t np = deg.np[i];
     for (int32_t r = 0; r < np; r += kTile)
       fill_tasks(make_int4(c, r, min(kTile, np - r), kItemProxies + i), cq, part_len, key_base, key_max, o,
-                 next_slot, next_rows, slot_rows, items, parts, keys);
+                 next_group, items, parts, keys);
   }
 }
 
@@ -886,16 +873,15 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
   int32_t *nitems = nullptr, *off = nullptr;
   int64_t *cost_part = nullptr, *cost_prox = nullptr;
   unsigned long long* summary = nullptr;   // [0, 2): executed counters; [2, 6): segment starts; then:
-  // [0] items, [1] padded pool particles, [2] split tiles, [3] longest task's chunks, [4] 32-row groups of
-  // segment sums, [5] next split slot, [6] next group
+  // [0] items, [1] padded pool particles, [2] 32-row groups of segment sums, [3] longest task's chunks, [4] next group
   Arena scratch;
   scratch.add(&nitems, nct);
   scratch.add(&off, nct);
   scratch.add(&cost_part, nct);
   scratch.add(&cost_prox, (size_t)nct * kMaxDegrees);
-  scratch.add(&summary, 10);
+  scratch.add(&summary, 9);
   BL_TRY(scratch.alloc(s));
-  BL_CUDA(cudaMemsetAsync(summary, 0, 10 * sizeof(unsigned long long), s));
+  BL_CUDA(cudaMemsetAsync(summary, 0, 9 * sizeof(unsigned long long), s));
   int32_t* totals = reinterpret_cast<int32_t*>(summary + 6);
   unsigned long long* executed = summary;
   dfree_ptr(p->eval_part, s);
@@ -905,16 +891,15 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
   const int64_t part_len = task_chunks(p);
   k_item_count<<<nblk((int64_t)nct * 32, 128), 128, 0, s>>>(nct, L, tt.parent, tt.nchild, tt.begin, tt.end,
                                               st.begin, st.end, nitems, cost_part, cost_prox,
-                                              executed, p->eval_part, p->eval_prox, part_len, totals + 2, totals + 3, totals + 4);
+                                              executed, p->eval_part, p->eval_prox, part_len, totals + 2, totals + 3);
   BL_LAUNCHED(cnt.launches);
   BL_TRY(scan_exclusive_dev(nitems, off, nct, totals, s, cnt));
   BL_CUDA(cudaMemcpyAsync(totals + 1, p->pad_prefix + st.nleaves, sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-  int32_t h_tot[5];
+  int32_t h_tot[4];
   BL_TRY(read_device(totals, h_tot, sizeof(h_tot), s));
   const int32_t ni = h_tot[0];
   p->nitems = ni;
-  p->nsplit = h_tot[2];
-  p->sum_groups = h_tot[4];
+  p->sum_groups = h_tot[2];
   p->pool_particles = h_tot[1];
   p->pool_len = h_tot[1];
   for (int i = 0; i < p->deg.n; ++i) {   // proxy blocks of every source cluster, per degree
@@ -933,7 +918,6 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
   BL_TRY(unsorted.alloc(s));
   BL_TRY(dalloc_n(&p->parts, ni, s));
   BL_TRY(dalloc_n(&p->items, ni, s));
-  if (p->nsplit > 0) BL_TRY(dalloc_n(&p->slot_rows, p->nsplit, s));
   // Bits of the sort key: the longest task's, the kernel of a shared
   // Coulomb/Yukawa segment, the segment.  As few as hold them: each 8 cost the
   // sort a pass.
@@ -943,8 +927,8 @@ int build_work_items(bldtt_plan* p, cudaStream_t s) {
   segmap.n = (int)p->segment_kernels.size();
   for (int i = 0; i < segmap.n; ++i) segmap.kernel[i] = p->segment_kernels[i];
   k_item_fill<<<nblk(nct, 128), 128, 0, s>>>(nct, off, cost_part, cost_prox, tt.begin, tt.end,
-                                             tt.problem, p->prob_kernel, segmap, p->deg, part_len, len_bits, totals + 5, totals + 6,
-                                             p->slot_rows,                                             items, parts, keys);
+                                             tt.problem, p->prob_kernel, segmap, p->deg, part_len, len_bits, totals + 4,
+                                             items, parts, keys);
   BL_LAUNCHED(cnt.launches);
   // Grouped by kernel, longest items first within a group (stable), so that
   // each persistent launch's tail is short.

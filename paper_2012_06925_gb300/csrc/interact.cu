@@ -65,10 +65,9 @@ constexpr uint64_t kWaitNs = 20ull * 1000ull * 1000ull * 1000ull;   // 20 s boun
 
 struct InteractView {
   const int4* items;
-  const int4* parts;            // {first chunk, chunks, segment-sum slot or -1, segments | segment length << 8}
-  double* seg_sums;             // [groups of 32 rows]: from slot_rows[slot] on, [segments][groups of the tile]
-  const int32_t* slot_rows;
-  int32_t* arrived;             // [slots][kItemGroups]: segments finished, per consumer warp
+  const int4* parts;            // {first chunk, chunks, first group of segment sums or -1, segments | segment length << 8}
+  double* seg_sums;             // [groups][32]: from a split tile's first group on, [segments][groups of the tile]
+  int32_t* arrived;             // [groups]: at a split tile's first groups, segments finished per consumer warp
   int32_t nitems;
   int32_t* counter;
   // lists and source layout (producer)
@@ -106,7 +105,7 @@ constexpr unsigned kTaskStart = 1, kSegEnd = 2, kTaskEnd = 4;
 struct StageMeta {
   int item;                     // task index (-1: no more work)
   int count;                    // real sources in the staged chunk
-  int slot;                     // split item: its segment-sum slot (-1: the task is a whole item)
+  int slot;                     // split item: first group of its segment sums (-1: the task is a whole item)
   int seg;                      // the chunk's segment
   unsigned flags;               // kTaskStart | kSegEnd | kTaskEnd
   unsigned near;                // bit g: target group g may be near the chunk (residuals staged)
@@ -447,21 +446,28 @@ struct Producer {
 
 // ---- consumers --------------------------------------------------------------
 // Kernel parameter of a work item in FP32: fp32_parameter's value k, and for the
-// oscillatory kernel kappa / pi and pi k / (kappa kPiHigh) - 1 (see sin2).
-struct Param32 {
-  float k, turns, rest;
+// oscillatory kernel kappa / pi and pi k / (kappa kPiHigh) - 1 (see sin2); the
+// second form has each value duplicated.
+template <typename T>
+struct PlainParam {
+  T k;
 };
-struct Param32x2 {               // each duplicated
-  f2_t k, turns, rest;
+template <typename T>
+struct PhaseParam {
+  T k, turns, rest;
 };
-__device__ __forceinline__ Param32x2 duplicate(const Param32& p) {
-  return Param32x2{f2_pack(p.k, p.k), f2_pack(p.turns, p.turns), f2_pack(p.rest, p.rest)};
+template <int KERN, typename T>
+using Param = std::conditional_t<KERN == BLDTT_OSCILLATORY, PhaseParam<T>, PlainParam<T>>;
+__device__ __forceinline__ PlainParam<f2_t> duplicate(const PlainParam<float>& p) { return {f2_pack(p.k, p.k)}; }
+__device__ __forceinline__ PhaseParam<f2_t> duplicate(const PhaseParam<float>& p) {
+  return {f2_pack(p.k, p.k), f2_pack(p.turns, p.turns), f2_pack(p.rest, p.rest)};
 }
 constexpr float kPiHigh = 3.140625f;
-__device__ __forceinline__ Param32 oscillatory_param(float k, double kappa) {
+__device__ __forceinline__ void set_param(PlainParam<float>& p, float k, const double*) { p.k = k; }
+__device__ __forceinline__ void set_param(PhaseParam<float>& p, float k, const double* kappa) {
   const double pi = 3.14159265358979323846;
-  const double scale = kappa > 0.0 ? (double)k / kappa : 1.0;
-  return Param32{k, (float)(kappa / pi), (float)(pi / (double)kPiHigh * scale - 1.0)};
+  const double scale = *kappa > 0.0 ? (double)k / *kappa : 1.0;
+  p = {k, (float)(*kappa / pi), (float)(pi / (double)kPiHigh * scale - 1.0)};
 }
 
 // sin(kappa r) of two values: kappa r = n pi + f with n the nearest integer, sin =
@@ -477,7 +483,7 @@ __device__ __forceinline__ Param32 oscillatory_param(float k, double kappa) {
 // |f| <= pi/2 (6.3e-9 with these float coefficients, found one after the other so
 // that each absorbs the rounding of those before it).  For arguments
 // beyond 2^22 pi the phase is noise in float; the clamp keeps |sin| <= 1.
-__device__ __forceinline__ f2_t sin2(f2_t r, const Param32x2& p) {
+__device__ __forceinline__ f2_t sin2(f2_t r, const PhaseParam<f2_t>& p) {
   const f2_t big = f2_pack(12582912.f, 12582912.f);
   const f2_t t = f2_fma(r, p.turns, big);
   const f2_t m = f2_fma(t, f2_pack(-kPiHigh, -kPiHigh), f2_pack(12582912.f * kPiHigh, 12582912.f * kPiHigh));   // -n kPiHigh
@@ -506,7 +512,7 @@ __device__ __forceinline__ f2_t sin2(f2_t r, const Param32x2& p) {
 // in near chunks only 4.5 and 11.1.
 enum Guard { kNoGuard, kGuardFactor, kGuardPair };
 template <int KERN, Guard GUARD = kNoGuard>
-__device__ __forceinline__ f2_t pair2_eval(f2_t dx, f2_t dy, f2_t dz, f2_t q2, f2_t acc, const Param32x2& prm) {
+__device__ __forceinline__ f2_t pair2_eval(f2_t dx, f2_t dy, f2_t dz, f2_t q2, f2_t acc, const Param<KERN, f2_t>& prm) {
   f2_t r2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
   float r0, r1;
   f2_unpack(r2, r0, r1);
@@ -521,7 +527,7 @@ __device__ __forceinline__ f2_t pair2_eval(f2_t dx, f2_t dy, f2_t dz, f2_t q2, f
   const f2_t ri = f2_pack(k0 ? i0 : 0.f, k1 ? i1 : 0.f);
   if (KERN == BLDTT_COULOMB || KERN == BLDTT_REG_COULOMB) return f2_fma(q2, ri, acc);
   const f2_t r = f2_mul(r2, ri);
-  if (KERN == BLDTT_OSCILLATORY) return f2_fma(f2_mul(q2, ri), sin2(r, prm), acc);
+  if constexpr (KERN == BLDTT_OSCILLATORY) return f2_fma(f2_mul(q2, ri), sin2(r, prm), acc);
   // Yukawa: q ri exp2(-kappa log2(e) r)
   float e0, e1;
   f2_unpack(f2_mul(r, prm.k), e0, e1);
@@ -529,7 +535,7 @@ __device__ __forceinline__ f2_t pair2_eval(f2_t dx, f2_t dy, f2_t dz, f2_t q2, f
 }
 template <int KERN>
 __device__ __forceinline__ f2_t pair2_f32(f2_t tx, f2_t ty, f2_t tz, const ulonglong2& a,
-                                          const ulonglong2& b, f2_t acc, const Param32x2& prm) {
+                                          const ulonglong2& b, f2_t acc, const Param<KERN, f2_t>& prm) {
   return pair2_eval<KERN>(f2_sub(tx, a.x), f2_sub(ty, a.y), f2_sub(tz, b.x), b.y, acc, prm);
 }
 // Careful variant: d = fma(m, x_r - y_r, x'' - y'') with m = 1 for a target
@@ -539,7 +545,7 @@ template <int KERN, Guard GUARD>
 __device__ __forceinline__ f2_t pair2_careful(f2_t tx, f2_t ty, f2_t tz, f2_t rx, f2_t ry, f2_t rz,
                                               f2_t m2, const ulonglong2& a, const ulonglong2& b,
                                               const ulonglong2& ra, const ulonglong2& rb, f2_t acc,
-                                              const Param32x2& prm) {
+                                              const Param<KERN, f2_t>& prm) {
   return pair2_eval<KERN, GUARD>(f2_fma(m2, f2_sub(rx, ra.x), f2_sub(tx, a.x)),
                           f2_fma(m2, f2_sub(ry, ra.y), f2_sub(ty, a.y)),
                           f2_fma(m2, f2_sub(rz, rb.x), f2_sub(tz, b.x)), b.y, acc, prm);
@@ -552,9 +558,9 @@ __device__ __forceinline__ f2_t pair2_careful(f2_t tx, f2_t ty, f2_t tz, f2_t rx
 // and the oscillatory kernel 3.88, 3.83 and 3.77.
 template <int KERN, int K>
 __device__ __forceinline__ void chunk_f32(const ulonglong2* __restrict__ sb, int npairs,
-                                          const f2_t (&x2)[K][3], float (&a)[K], const Param32& prm) {
+                                          const f2_t (&x2)[K][3], float (&a)[K], const Param<KERN, float>& prm) {
   f2_t acc[K];
-  const Param32x2 prm2 = duplicate(prm);
+  const Param<KERN, f2_t> prm2 = duplicate(prm);
 #pragma unroll
   for (int k = 0; k < K; ++k) acc[k] = 0ull;
   if (KERN != BLDTT_OSCILLATORY && npairs == kChunk / 2) {
@@ -609,8 +615,8 @@ __device__ __forceinline__ void chunk_f32_careful(const ulonglong2* __restrict__
                                                   const ulonglong2* __restrict__ sr, int npairs,
                                                   const f2_t (&x2)[K][3], const TargetSplit& ts,
                                                   const float* c, unsigned near, float (&a)[K],
-                                                  const Param32& prm) {
-  const Param32x2 prm2 = duplicate(prm);
+                                                  const Param<KERN, float>& prm) {
+  const Param<KERN, f2_t> prm2 = duplicate(prm);
   f2_t acc[K], m2[K], r2x[K][3];
 #pragma unroll
   for (int k = 0; k < K; ++k) {
@@ -773,7 +779,7 @@ __device__ __noinline__ void end_segment(const InteractView& v, const int4 item,
   }
   const int rows = (item.z + 31) / 32 * 32;
   if (ct >= rows) return;                       // whole warps: no row of this tile
-  double* sums = v.seg_sums + (int64_t)v.slot_rows[slot] * 32;
+  double* sums = v.seg_sums + (int64_t)slot * 32;
 #pragma unroll
   for (int k = 0; k < K; ++k)
     if (k * NCW * 32 + ct < rows) sums[seg * rows + k * NCW * 32 + ct] = a.v[k];
@@ -781,7 +787,7 @@ __device__ __noinline__ void end_segment(const InteractView& v, const int4 item,
   const int4 part = v.parts[task];
   const int nseg = part.w & 0xff, len = part.w >> 8;
   const int mine = (part.x + part.y + len - 1) / len - part.x / len;
-  int32_t* count = v.arrived + (int64_t)slot * kItemGroups + (ct >> 5);
+  int32_t* count = v.arrived + slot + (ct >> 5);
   __threadfence();
   __syncwarp();
   int done = 0;
@@ -819,17 +825,21 @@ __device__ __forceinline__ void frame_targets(const TargetSplit& ts, const float
     }
   }
 }
-// The careful path's sums with an r = 0 guard.  A call of its own: its
-// registers must not crowd the plain loop's.
-template <int KERN, int K, Guard GUARD>
+// The careful path's sums with the r = 0 guard, of the charges too if near has
+// kWholePair set.  A call of its own: its registers must not crowd the plain loop's.
+constexpr unsigned kWholePair = 0x80000000u;
+template <int KERN, int K>
 __device__ __noinline__ PartialSums<K> careful_sums(const float* sf, const float* res, int count,
                                                     const TargetSplit ts, const float* c, unsigned near,
-                                                    const Param32 prm) {
+                                                    const Param<KERN, float> prm) {
   f2_t x2[K][3];
   frame_targets<K>(ts, c, x2);
+  const ulonglong2 *sb = reinterpret_cast<const ulonglong2*>(sf), *rb = reinterpret_cast<const ulonglong2*>(res);
   PartialSums<K> out;
-  chunk_f32_careful<KERN, K, GUARD>(reinterpret_cast<const ulonglong2*>(sf), reinterpret_cast<const ulonglong2*>(res),
-                              (count + 1) / 2, x2, ts, c, near, out.v, prm);
+  if (near & kWholePair)
+    chunk_f32_careful<KERN, K, kGuardPair>(sb, rb, (count + 1) / 2, x2, ts, c, near, out.v, prm);
+  else
+    chunk_f32_careful<KERN, K, kGuardFactor>(sb, rb, (count + 1) / 2, x2, ts, c, near, out.v, prm);
   return out;
 }
 // One staged chunk in FP32 for K targets (partial sums in a[]).  ts holds
@@ -852,7 +862,7 @@ template <int KERN, int K>
 __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rbuf, int count,
                                                const f2_t (&x2)[K][3], const TargetSplit& ts,
                                                const float* c, const float4* ext_p, unsigned slot, bool warp_full,
-                                               bool overlap, const Param32& prm, float (&a)[K]) {
+                                               bool overlap, const Param<KERN, float>& prm, float (&a)[K]) {
   const float* sf = reinterpret_cast<const float*>(buf);
   const float* res = reinterpret_cast<const float*>(rbuf);
   float xs[K][3];
@@ -887,11 +897,11 @@ __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rb
     chunk_f32_careful<KERN, K, kNoGuard>(sb, reinterpret_cast<const ulonglong2*>(rbuf), (count + 1) / 2, x2,
                                       ts, c, near, a, prm);
   } else if (any_near) {
-    const PartialSums<K> r = careful_sums<KERN, K, kGuardFactor>(sf, res, count, ts, c, near, prm);
+    const PartialSums<K> r = careful_sums<KERN, K>(sf, res, count, ts, c, near, prm);
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = r.v[k];
   } else if (KERN == BLDTT_REG_COULOMB && overlap && !(ext_p->w >= 0.f)) {
-    const PartialSums<K> r = careful_sums<KERN, K, kGuardFactor>(sf, sf, count, ts, c, 0u, prm);
+    const PartialSums<K> r = careful_sums<KERN, K>(sf, sf, count, ts, c, 0u, prm);
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = r.v[k];
   } else if (K > 1 && !warp_full) {
@@ -910,7 +920,7 @@ __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rb
   for (int k = 0; k < K; ++k) bad = bad || not_finite(a[k]);
   if (__any_sync(0xffffffffu, bad)) {
     // residuals that were not staged are not read: any finite numbers do (their factor is 0)
-    const PartialSums<K> r = careful_sums<KERN, K, kGuardPair>(sf, slot ? res : sf, count, ts, c, near, prm);
+    const PartialSums<K> r = careful_sums<KERN, K>(sf, slot ? res : sf, count, ts, c, near | kWholePair, prm);
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = r.v[k];
   }
@@ -962,7 +972,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
   __shared__ double s_tot[K * kConsumers];   // the item's finished segments (in shared memory: no register)
   bool warp_full = true;
   bool warp_active = true;
-  Param32 prm{};                // its FP32 parameter
+  Param<KERN, float> prm{};     // its FP32 parameter
   Param64 prm64{};              // its FP64 parameter
   bool yukawa = KERN == BLDTT_YUKAWA;   // the fused Coulomb/Yukawa launch: this item's kernel
   for (uint32_t it = 0;; ++it) {
@@ -972,8 +982,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
     if (smeta[s].flags & kTaskStart) {
       item = v.items[smeta[s].item];
       const int pid = v.t_problem[item.x];
-      prm.k = v.prob_prm[pid];
-      if (F32 && KERN == BLDTT_OSCILLATORY) prm = oscillatory_param(prm.k, v.prob_kappa[pid]);
+      if (F32) set_param(prm, v.prob_prm[pid], v.prob_kappa + pid);
       if (!F32) {
         prm64.kappa = v.prob_kappa[pid];
         if (KERN == BLDTT_YUKAWA || KERN == kKernCoulombYukawa) prm64.screen = fixed64::make_screen(prm64.kappa);
@@ -1015,7 +1024,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) k_interact(InteractView 
         for (int k = 0; k < K; ++k) slot |= ((gm >> (k * NCW + warp)) & 1u) << k;
       }
       float a[K];
-      if (KERN != kKernCoulombYukawa)
+      if constexpr (KERN != kKernCoulombYukawa)
         eval_chunk_f32<KERN, K>(sbuf[s], sres[s], count, x2, ts, c, ext, slot, warp_full, v.overlap, prm, a);
       else if (yukawa)
         eval_chunk_f32<BLDTT_YUKAWA, K>(sbuf[s], sres[s], count, x2, ts, c, ext, slot, warp_full, v.overlap, prm, a);
@@ -1159,7 +1168,6 @@ static InteractView make_view(const bldtt_plan* p) {
   v.items = p->items;
   v.parts = p->parts;
   v.seg_sums = p->seg_sums;
-  v.slot_rows = p->slot_rows;
   v.arrived = p->item_counter + kMaxSegmentsLaunch;
   v.nitems = p->nitems;
   v.counter = p->item_counter;

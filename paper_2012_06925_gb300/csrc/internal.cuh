@@ -356,15 +356,15 @@ struct bldtt_plan {
 
   // Work items of the interaction kernel, sorted by decreasing cost.
   int4* items = nullptr;              // {cluster, row_begin, row_count, kind}
-  int4* parts = nullptr;              // task i: {first chunk, chunks, split slot or -1, nseg | len << 8}
+  int4* parts = nullptr;              // task i: {first chunk, chunks, its tile's first group of sums or -1, nseg | len << 8}
   int32_t nitems = 0;                 // tasks: the tiles, long ones split over their sources (plan_parts)
-  int32_t nsplit = 0;                 // split tiles
-  // Segment sums of the split tiles, in groups of 32 target rows: a tile has its segments x its own
-  // groups, from group slot_rows[slot] on (as many segments and rows for every tile: 32 KB each).
+  // Segment sums of the split tiles, in groups of 32 target rows: each tile has its segments x its own
+  // groups from its task's first group on (with 16 segments of 256 rows for every tile, 32 KB, a plan of 4E5
+  // targets in leaves of 30 took 1275 MB instead of 235).
   double* seg_sums = nullptr;         // [sum_groups][32]
-  int32_t* slot_rows = nullptr;       // [nsplit]
   int32_t sum_groups = 0;
-  // [kMaxSegmentsLaunch] next task of each segment, then [nsplit][kItemGroups] finished segments
+  // [kMaxSegmentsLaunch] next task of each segment; then, at each split tile's first groups, its finished
+  // segments per consumer warp (a warp with rows of the tile has a group there)
   int32_t* item_counter = nullptr;
   size_t counter_words = 0;
   double executed_evaluations = 0.0;
