@@ -228,17 +228,19 @@ int direct_sum(const double* targets, int64_t M, const double* sources, int64_t 
     }
   }
   const int64_t span = (N + splits - 1) / splits;
-  double* part = phi;
-  if (splits > 1) BL_TRY(dalloc_n(&part, (size_t)(splits * M), s));
   const dim3 grid(blocks, (unsigned)splits);
   const bool fixed = kappa >= 0.0 && kappa <= DBL_MAX;
   // The extent takes two launches, about 6 us: worth it from some millions of evaluations.
-  unsigned long long* key = nullptr;
   int64_t dummy = 0;
   const bool coords = (double)M * (double)N >= 0x1p23 &&
                       (kernel == BLDTT_COULOMB || (kernel == BLDTT_YUKAWA && fixed));
+  double* part = phi;
+  unsigned long long* key = nullptr;
+  Arena scratch;                       // freed, in stream order, when it goes out of scope
+  if (splits > 1) scratch.add(&part, (size_t)(splits * M));
+  if (coords) scratch.add(&key, 6);
+  if (splits > 1 || coords) BL_TRY(scratch.alloc(s));
   if (coords) {
-    BL_TRY(dalloc_n(&key, 6, s));
     BL_CUDA(cudaMemsetAsync(key, 0, 6 * sizeof(*key), s));
     const int64_t need = (M + N + kDirectThreads - 1) / kDirectThreads;
     k_extent<<<dim3((unsigned)(need < 2 * sms ? need : 2 * sms), 3), kDirectThreads, 0, s>>>(targets, M, sources, N,
@@ -259,11 +261,9 @@ int direct_sum(const double* targets, int64_t M, const double* sources, int64_t 
     k = fixed ? k_direct<BLDTT_REG_COULOMB, kFormFixed> : k_direct<BLDTT_REG_COULOMB, kFormFp64>;
   k<<<grid, kDirectThreads, 0, s>>>(targets, M, sources, N, charges, kappa, span, key, part);
   BL_LAUNCHED(dummy);
-  dfree(key, s);
   if (splits > 1) {
     k_direct_reduce<<<(unsigned)((M * 32 + kDirectThreads - 1) / kDirectThreads), kDirectThreads, 0, s>>>(part, M, (int)splits, phi);
     BL_LAUNCHED(dummy);
-    dfree(part, s);
   }
   return BLDTT_OK;
 }
