@@ -272,7 +272,8 @@ int setup_impl(bldtt_plan* p, const double* targets, const double* sources, cons
   // Default layout: warps of empty rows skip their work when that saves at
   // least 2 % of the evaluations (many items smaller than a tile).
   const bool skip = p->skip_saved_evaluations > 0.02 * p->executed_noskip;
-  p->executed_evaluations = skip ? p->executed_skip : p->executed_noskip;
+  // The FP64 kernels leave idle row groups out in every layout.
+  p->executed_evaluations = skip || p->precision == BLDTT_FP64 ? p->executed_skip : p->executed_noskip;
   p->interact_layout = skip ? kLayoutSkip : 0;
   if (const char* lay = std::getenv("BLDTT_INTERACT_LAYOUT")) {
     int l = std::atoi(lay);
