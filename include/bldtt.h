@@ -65,7 +65,8 @@ enum bldtt_kernel {
 enum bldtt_precision {
     BLDTT_FP64 = 0,       /* FP64 results everywhere; the Coulomb, Yukawa and
                              regularized kernels are evaluated in 64-bit fixed point,
-                             to within FP64's last rounding */
+                             Coulomb and regularized to within FP64's last rounding,
+                             Yukawa with kappa r 1.45 2^-58 of the value beside it */
     BLDTT_FP32_BULK = 1   /* kernel evaluations and Lagrange contractions in FP32, in
                              coordinate frames local to each source cluster, summed in
                              FP64 every 256 sources; barycentric weights, the
@@ -516,7 +517,8 @@ int bldtt_export_proxy_potentials(bldtt_plan* plan, double* phit);
 /*
  * bldtt_direct_sum - FP64 direct summation, Eq. (1), on the device: for
  * every target i, phi[i] = sum_j G(x_i, y_j) q_j with pairs at distance 0
- * skipped.  Pointers are device memory in the layouts above.  Used to measure
+ * skipped, whatever their charge (charges are not checked here; an infinite
+ * or NaN one reaches every other target).  Pointers are device memory in the layouts above.  Used to measure
  * the error of the fast method on sampled targets.  Asynchronous on
  * cuda_stream.  Errors: EINVAL, ECUDA.
  */

@@ -5,9 +5,10 @@
 // for r^2, 5 around the reciprocal square root, 1 to accumulate), one of
 // exp(-kappa r)/r about 40.  Here only the differences and the accumulation
 // stay FP64 (4 instructions).  From the differences' bits on the value is
-// carried in 64-bit fixed point with 58 or more significant bits, so its error
-// is below the final rounding to 53 bits; the FP64 expressions it replaces
-// round r^2, the square root and the quotient or product one by one.
+// carried in 64-bit fixed point with 58 or more significant bits, so the error of
+// 1/r and 1/sqrt(r^2 + kappa^2) is below the final rounding to 53 bits; the FP64
+// expressions they replace round r^2, the square root and the quotient or product
+// one by one.
 //
 //   d      53-bit mantissas aligned to the largest exponent E of the three
 //   S      sum of squares over 2^64 (the squares of the low words, below
@@ -17,6 +18,11 @@
 //   exp2   2^-t, t = kappa log2(e) r: integer part, 8 table bits and a degree-5
 //          Taylor polynomial of the rest (Tang's table-driven scheme, ACM TOMS
 //          15, 1989, in fixed point)
+//
+// exp(-kappa r) turns r's relative error of about 2^-59 into kappa r times as
+// much, so the screened value is off by up to kappa r 1.45 2^-58 beside the last
+// rounding (9 units of 2^-53 at kappa r = 300; FP64 expressions, which round r and
+// kappa r to 2^-53, up to some hundreds).
 //
 // Functions are plain C++ so that they can be checked on a host against
 // extended precision.

@@ -16,9 +16,9 @@
 // An item with many source chunks is split into tasks over its chunks
 // (plan_parts), so that a plan with few items still fills the device and the
 // last tasks are short: 2E4 points make ~200 items for 152 SMs x 6 CTAs, and
-// the launch lasted as long as the longest of them (interaction kernel, GB300:
-// FP64 at 2E4 points, n = 4, 28.3 -> 9.6 ms; FP64 Yukawa at 6E4 321 -> 51 ms;
-// FP32 on a sphere of 2E4 0.45 -> 0.18 ms; 1E6 points 32.4 -> 31.4 ms).
+// the launch would last as long as the longest of them (this kernel on a GB300,
+// whole items and tasks: FP64 at 2E4 points, n = 4, 9.5 and 2.3 ms; FP32 on a sphere
+// of 2E4 0.31 and 0.14 ms; 1E6 points 31.7 and 31.2 ms).
 //
 // Per CTA, one producer warp takes tasks from a global counter, walks their
 // lists and streams the sources, kChunk at a time, from the source pool into
@@ -50,9 +50,10 @@
 //
 // A pair at distance 0 contributes nothing.  Only a target near a chunk (or in
 // it) can meet one, so the guard stands in the careful path alone, for warps
-// with a target inside the chunk's box; the plain path evaluates unguarded, and
-// a sum that is not finite all the same (r^2 underflows) is redone with the
-// guard.  The arithmetic and the order are the same throughout, so a target's
+// with a target inside the chunk's box (and in proxy chunks of plans whose
+// clusters may overlap); the plain path evaluates unguarded, and a sum that is
+// not finite all the same (r^2 underflows, a charge beyond float) is redone with
+// such pairs left out.  The arithmetic and the order are the same throughout, so a target's
 // result never depends on which warp or consumer layout evaluated it.
 #include <type_traits>
 
@@ -237,9 +238,10 @@ struct Param64 {
   fixed64::Screen screen;
 };
 // Coulomb, Yukawa and regularized run in fixed point: the FP64 pipe (1.7 lanes
-// per clock and SM) took 12 to 45 instructions per evaluation, now 4.  2E4
-// Coulomb particles: 9.6 -> 3.2 ms in this kernel (n 4, theta 0.7, leaves of
-// 500); 6E4 Yukawa (n 7, theta 0.8, leaves of 1000): 51 -> 9.7 ms.
+// per clock and SM) would take 12 to 45 instructions per evaluation, here 4.  2E4
+// Coulomb particles (n 4, theta 0.7, leaves of 500) 2.3 ms in this kernel, a third
+// of its time with FP64 expressions; 6E4 Yukawa (n 7, theta 0.8, leaves of 1000) 9.5
+// ms, a fifth.
 template <int KERN>
 __device__ __forceinline__ double kernel_f64(double dx, double dy, double dz, const Param64& prm) {
   if (KERN == BLDTT_COULOMB) return fixed64::inv_r(dx, dy, dz);
@@ -374,10 +376,10 @@ struct Producer {
     return true;
   }
 
-  // The lists of target cluster a: class cls0 as particles (degree index -1),
-  // and for lane l in [1, nlists) the class of lane l as proxies of degree
-  // index deg_of(l); one list_ptr pair per lane.
-  __device__ bool run_particles(int32_t leaf) {   // PP and PC of every degree, leaf and ancestors
+  // The lists of a leaf's particles: on the leaf and on each of its ancestors, PP
+  // and then PC of every degree.  Lane 0 holds an ancestor's PP range of the CSR,
+  // lane i + 1 its PC range of degree index i.
+  __device__ bool run_particles(int32_t leaf) {
     for (int32_t a = leaf; a >= 0 && left > 0;) {
       const int32_t up = v.t_parent[a];
       int32_t e0 = 0, e1 = 0;
@@ -504,12 +506,10 @@ __device__ __forceinline__ f2_t sin2(f2_t r, const PhaseParam<f2_t>& p) {
 // Packed evaluation of target k against the source pair (s0, s1) at
 // differences d: acc += (q0 G(x - s0), q1 G(x - s1)).  A guard gives a pair at r =
 // 0 the factor 0 (two compares and two selects a pair of evaluations); kGuardPair
-// leaves its charge out as well, which may be infinite in float.  The scalar
-// guarded loop that the oscillatory and regularized kernels used to take for
-// every pair (four shared-memory loads and a branch per evaluation, sinf) ran
-// at 0.67 and 2.6 evaluations per clock and SM against 12.4 of the packed
-// Coulomb loop; packed with the guard on every pair 3.8 and 9.4, with the guard
-// in near chunks only 4.5 and 11.1.
+// leaves its charge out as well, which may be infinite in float.  Evaluations
+// per clock and SM: Coulomb 12.8, Yukawa 8.7, regularized 11.1 (9.4 with the guard
+// on every pair instead of near chunks only, 2.6 in a scalar guarded loop),
+// oscillatory 4.2 (0.67 in a scalar loop with sinf).
 enum Guard { kNoGuard, kGuardFactor, kGuardPair };
 template <int KERN, Guard GUARD = kNoGuard>
 __device__ __forceinline__ f2_t pair2_eval(f2_t dx, f2_t dy, f2_t dz, f2_t q2, f2_t acc, const Param<KERN, f2_t>& prm) {
@@ -554,8 +554,7 @@ __device__ __forceinline__ f2_t pair2_careful(f2_t tx, f2_t ty, f2_t tz, f2_t rx
 // Sum over the staged chunk of q G for K targets; two partial sums per target.
 // Full chunks have a loop of fixed length (the oscillatory kernel's loop body
 // is long enough to do without); the others are unrolled as far: 1E6 particles,
-// whose leaves end in a partial chunk, 31.5 ms unrolled by 2, 31.1 by 4 and 8,
-// and the oscillatory kernel 3.88, 3.83 and 3.77.
+// whose leaves end in a partial chunk, 31.5 ms unrolled by 2, 31.1 by 4 and 8.
 template <int KERN, int K>
 __device__ __forceinline__ void chunk_f32(const ulonglong2* __restrict__ sb, int npairs,
                                           const f2_t (&x2)[K][3], float (&a)[K], const Param<KERN, float>& prm) {
@@ -706,7 +705,7 @@ __device__ __forceinline__ void chunk_f64(const double4* __restrict__ sb, int co
 // The same for the warp's real rows: its last target slot is left out where
 // none of its rows holds a target.  The FP64 pipe bounds this path, so an idle
 // row costs what a real one does: 2E4 Coulomb particles in leaves of 312 (a
-// full tile and one of 56 rows) 3.2 -> 2.2 ms.
+// full tile and one of 56 rows) 2.3 ms, 3.2 with the idle rows.
 template <int KERN, int K>
 __device__ __forceinline__ void rows_f64(const double4* __restrict__ sb, int count, const double (&x)[K][3],
                                          bool warp_full, double (&a)[K], const Param64& prm) {
@@ -853,11 +852,10 @@ __device__ __noinline__ PartialSums<K> careful_sums(const float* sf, const float
 // is not finite is redone with coincident pairs left out, charge and all.  The
 // regularized kernel is finite at r = 0: where a target may lie at a source proxy
 // (overlap), its proxy chunks take the guarded call too.
-// The chunk that a tile shares with its own targets used to run twice, the
-// second time in a scalar loop at an eighth of the rate: 1000 particles 0.099
-// -> 0.046 ms in this kernel, 2E4 on a sphere 0.184 -> 0.139, 512 problems of
-// 16k (lists of about 30 chunks) 77.7 -> 74.0.  With the guard on all near
-// chunks the latter is 75.5, and the unequal sets' 82.6 become 83.2.
+// The guard costs what its selects do: on all near chunks 512 problems of 16k
+// (lists of about 30 chunks) take 75.5 ms in this kernel instead of 74.0, the
+// unequal sets 83.2 instead of 82.6; and a tile's own chunk evaluated unguarded
+// first and guarded after 77.7.
 template <int KERN, int K>
 __device__ __forceinline__ void eval_chunk_f32(const void* buf, const float4* rbuf, int count,
                                                const f2_t (&x2)[K][3], const TargetSplit& ts,

@@ -329,7 +329,7 @@ int select_pairs(bldtt_plan* p, const int2* pairs, int32_t F, int16_t* choice, c
 }
 
 // ---- training ------------------------------------------------------------------
-// The master parameters of one layer into shared memory as bf16: Wt[k][j] (the
+// The master parameters of all layers into shared memory as bf16, per layer Wt[k][j] (the
 // forward pass: a warp's lanes read neighbouring neurons) and, if Wr is given,
 // Wr[j][k] (the backward pass: neighbouring inputs).
 __device__ void load_params(const float* __restrict__ params, const ParamLayout& L, int nout, __nv_bfloat16* wt,
