@@ -398,9 +398,11 @@ int bldtt_compute_graph(bldtt_plan* plan, double* phi, void* cuda_stream);
  * warps x targets per thread: 4 x 2 or 2 x 4), the CTAs per SM the registers
  * are sized for (6 or 5), the depth of the shared-memory ring of source
  * chunks (3 or 4 stages) and whether warps whose rows hold no real target
- * skip their work: layouts 0 = 4x2, 6 CTAs, 3 stages; 1 = 2x4, 6 CTAs, 3
- * stages; 2 = 4x2, 5 CTAs, 4 stages; 3-5 = the same with skipping (Coulomb
- * and the shared Coulomb/Yukawa launch; other kernels: layouts 0 and 3).
+ * skip their work: layouts 0 = 4x2, 6 CTAs (the oscillatory kernel in FP32:
+ * 4), 3 stages; 1 = 2x4, 6 CTAs, 3 stages; 2 = 4x2, 5 CTAs, 4 stages; 3-5 =
+ * the same with skipping (Coulomb and the shared Coulomb/Yukawa launch; other
+ * kernels: layouts 0 and 3).  FP64 kernels skip in every layout: their 3-5
+ * are 0-2 again.
  * Results do not depend on the layout (bit for bit).  *chosen (may be NULL)
  * receives the layout picked for the plan's first launch; the searched table
  * is kept for bldtt_autotune_table.  Synchronous.  Errors: EINVAL, ECUDA,
